@@ -101,13 +101,16 @@ extern "C" long long sph_launch_count(const sph_ctx* ctx) { return ctx ? ctx->la
 
 extern "C" int sph_bounds_report(int* first) {
 #ifdef SPH_CHECKED
-  int h[5] = {0, 0, 0, 0, 0}, z[5] = {0, 0, 0, 0, 0}, hb[5] = {0, 0, 0, 0, 0};
+  int h[5] = {0, 0, 0, 0, 0}, z[5] = {0, 0, 0, 0, 0}, o[2][5];
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpyFromSymbol(h, g_bounds, sizeof h) != cudaSuccess ||
-      cudaMemcpyToSymbol(g_bounds, z, sizeof z) != cudaSuccess || bounds_take_batch(hb) != SPH_OK)
+      cudaMemcpyToSymbol(g_bounds, z, sizeof z) != cudaSuccess || bounds_take_batch(o[0]) != SPH_OK ||
+      bounds_take_f64(o[1]) != SPH_OK)
     return SPH_ERR_CUDA;
-  if (h[0] == 0)
-    for (int q = 1; q < 5; q++) h[q] = hb[q];
-  h[0] += hb[0];
+  for (int u = 0; u < 2; u++) {
+    if (h[0] == 0)
+      for (int q = 1; q < 5; q++) h[q] = o[u][q];
+    h[0] += o[u][0];
+  }
   if (first)
     for (int q = 0; q < 4; q++) first[q] = h[1 + q];
   return h[0];
@@ -141,7 +144,7 @@ static void free_all(sph_ctx* c) {
   if (c->efork) cudaEventDestroy(c->efork);
   bufs_free(c->d64);
   bufs_free(c->d32);
-  cudaFree(c->bg); cudaFree(c->acc); cudaFree(c->flag); cudaFree(c->rows64);
+  cudaFree(c->bg); cudaFree(c->acc); cudaFree(c->flag); cudaFree(c->rows64); cudaFree(c->tab64);
   cudaFree(c->wmean64); cudaFree(c->wmean32); cudaFree(c->wnext);
   cudaFree(c->wzero64); cudaFree(c->wzero32);
   cudaFree(c->adjS); cudaFree(c->adjW); cudaFree(c->adjC);
@@ -274,6 +277,10 @@ static int upload_background(sph_ctx* c, const double* pref, const double* Tref)
   }
   int e = upload_tables(c, c->d64, c->hmet, der, nr);
   if (e == SPH_OK && c->prec == SPH_PREC_MIXED) e = upload_tables(c, c->d32, c->hmet, der, nr);
+  if (e == SPH_OK && c->tab64) {
+    f64_tables(c);
+    if (cudaGetLastError() != cudaSuccess) e = SPH_ERR_CUDA;
+  }
   free(der);
   return e;
 }
@@ -362,20 +369,21 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
                         !cuda_ok(cudaMalloc((void**)&c->flag, sizeof(int)))))
     err = SPH_ERR_NOMEM;
   if (err == SPH_OK && !mixed) {
-    // the line rows of the FP64 mode: 12 planes over the centres per direction,
-    // 5 + 6 over the faces of each kind
-    size_t nrows = 36 * (size_t)c->N + 11 * (c->nf[1] + c->nf[2] + c->nf[3]);
-    if (!cuda_ok(cudaMalloc((void**)&c->rows64, nrows * sizeof(double)))) {
+    // the line rows of the FP64 mode and the tables of its kernels
+    const size_t rc = f64::ROWS_C * (size_t)c->N, rf = f64::ROWS_F, rs = f64::ROWS_S;
+    if (!cuda_ok(cudaMalloc((void**)&c->rows64, (3 * rc + (rf + rs) * (c->nf[1] + c->nf[2] + c->nf[3])) * sizeof(double))) ||
+        !cuda_ok(cudaMalloc((void**)&c->tab64, f64::tabs_doubles(nr, nt) * sizeof(double)))) {
       err = SPH_ERR_NOMEM;
     } else {
       double* p = c->rows64;
       c->rows.nc = c->N;
-      for (int d = 0; d < 3; d++) { c->rows.c[d] = p; p += 12 * (size_t)c->N; }
+      for (int d = 0; d < 3; d++) { c->rows.c[d] = p; p += rc; }
       for (int d = 0; d < 3; d++) {
         c->rows.nf[d] = (long)c->nf[1 + d];
-        c->rows.f[d] = p; p += 5 * c->nf[1 + d];
-        c->rows.s[d] = p; p += 6 * c->nf[1 + d];
+        c->rows.f[d] = p; p += rf * c->nf[1 + d];
+        c->rows.s[d] = p; p += rs * c->nf[1 + d];
       }
+      c->tabs = f64::tabs_of(c->tab64, nr, nt);
     }
   }
   if (err != SPH_OK) { cudaGetLastError(); free_all(c); free(c); return err; }
@@ -661,7 +669,9 @@ static int prepare(sph_ctx* c, Bufs<R>& b, int have_iter, CF<R>* ub_out, double*
   }
   k_begin(c, SPH_K_COEF);
   const Geo<double>& gg = c->d64.g;
-  if (b.g.hasw) k_coef<R, true><<<tile_grid(gg.np, gg.nt, gg.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, ub, b.c);
+  if constexpr (sizeof(R) == sizeof(double)) {
+    f64_coef(c, ub);
+  } else if (b.g.hasw) k_coef<R, true><<<tile_grid(gg.np, gg.nt, gg.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, ub, b.c);
   else k_coef<R, false><<<tile_grid(gg.np, gg.nt, gg.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, ub, b.c);
   if (launch_ok(c)) return SPH_ERR_CUDA;
   *ub_out = ub;
@@ -688,38 +698,31 @@ static int join_aux(sph_ctx* c, int n) {
 // The right-hand side stage: centre rows on the context's stream, the
 // momentum rows of the three components on side streams, concurrently (timed
 // as one stage).
+template <bool W>
+static void launch_rhs32(sph_ctx* c, Bufs<float>& b, CF<float> ub, CF<float> ul, CF<float> Dv, int hasD, float tr,
+                         CF<double> src, int has_src, MF<float> Rout) {
+  const Geo<double>& g = c->d64.g;
+  k_rhs_c<float, W><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, b.c, ub, ul, Dv, hasD, src,
+                                                                           has_src, tr, Rout);
+  k_rhs_u<float, 0, W><<<tile_grid(g.np, g.nt, g.nr + 1), TILE_BLOCK, 0, c->aux[0]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
+                                                                                      has_src, tr, Rout);
+  k_rhs_u<float, 1, W><<<tile_grid(g.np, g.nt + 1, g.nr), TILE_BLOCK, 0, c->aux[1]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
+                                                                                      has_src, tr, Rout);
+  k_rhs_u<float, 2, W><<<tile_grid(g.npf, g.nt, g.nr), TILE_BLOCK, 0, c->aux[2]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
+                                                                                   has_src, tr, Rout);
+}
+
 template <typename R>
-static int run_rhs(sph_ctx* c, Bufs<R>& b, CF<R> ub, CF<double> uk, int hasD, double tau, CF<double> src, int has_src,
-                   MF<R> Rout) {
-  CF<double> un = cf_of(c->U[c->cur]);
+static int run_rhs(sph_ctx* c, Bufs<R>& b, CF<R> ub, int hasD, double tau, CF<double> src, int has_src, MF<R> Rout) {
   CF<R> Dv = cf_of(b.Db);  // U^k - U^n from the averaging stage (zero, and not read, when hasD = 0)
-  CF<R> ul = sizeof(R) == sizeof(float) ? cf_of(b.UbLo) : ub;  // velocity remainders of Ubar (FP32 mode)
-  R tr = (R)tau;
-  // FP64 mode: the kernels also store the line rows the sweeps read
-  Rows64 rows = c->rows;
-  if (sizeof(R) != sizeof(double)) memset(&rows, 0, sizeof rows);
   k_begin(c, SPH_K_RHS);
   if (fork_aux(c, 3)) return SPH_ERR_CUDA;
-  const Geo<double>& gg = c->d64.g;
-  int nr = gg.nr, nt = gg.nt, np = gg.np, npf = gg.npf;
-  if (b.g.hasw) {
-    k_rhs_c<R, true><<<tile_grid(np, nt, nr), TILE_BLOCK, 0, c->st>>>(b.g, c->d64.g, c->P, b.c, ub, ul, un, uk, Dv,
-                                                                      hasD, src, has_src, tr, Rout, rows);
-    k_rhs_u<R, 0, true><<<tile_grid(np, nt, nr + 1), TILE_BLOCK, 0, c->aux[0]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                 has_src, tr, Rout, rows);
-    k_rhs_u<R, 1, true><<<tile_grid(np, nt + 1, nr), TILE_BLOCK, 0, c->aux[1]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                 has_src, tr, Rout, rows);
-    k_rhs_u<R, 2, true><<<tile_grid(npf, nt, nr), TILE_BLOCK, 0, c->aux[2]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                              has_src, tr, Rout, rows);
+  if constexpr (sizeof(R) == sizeof(double)) {
+    f64_rhs(c, ub, Dv, hasD, tau, src, has_src, Rout);   // also stores the line rows the sweeps read
   } else {
-    k_rhs_c<R, false><<<tile_grid(np, nt, nr), TILE_BLOCK, 0, c->st>>>(b.g, c->d64.g, c->P, b.c, ub, ul, un, uk, Dv,
-                                                                       hasD, src, has_src, tr, Rout, rows);
-    k_rhs_u<R, 0, false><<<tile_grid(np, nt, nr + 1), TILE_BLOCK, 0, c->aux[0]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                  has_src, tr, Rout, rows);
-    k_rhs_u<R, 1, false><<<tile_grid(np, nt + 1, nr), TILE_BLOCK, 0, c->aux[1]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                  has_src, tr, Rout, rows);
-    k_rhs_u<R, 2, false><<<tile_grid(npf, nt, nr), TILE_BLOCK, 0, c->aux[2]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                               has_src, tr, Rout, rows);
+    CF<float> ul = cf_of(b.UbLo);  // velocity remainders of Ubar
+    if (b.g.hasw) launch_rhs32<true>(c, b, ub, ul, Dv, hasD, (float)tau, src, has_src, Rout);
+    else launch_rhs32<false>(c, b, ub, ul, Dv, hasD, (float)tau, src, has_src, Rout);
   }
   if (join_aux(c, 3)) return SPH_ERR_CUDA;
   c->launches += 3;  // launch_ok counts the fourth
@@ -858,21 +861,28 @@ static int run_lines_d(sph_ctx* c, SweepArgs<float>& S, int n) {
 // bound: warp-sized blocks spread the block lines evenly over the SMs
 // (measured, 128 x 256 x 256 FP64 step: 64.9 ms at 128 threads a block, 62.6
 // at 64, 60.1 at 32; theta and phi sweeps 13.7 and 15.9 -> 11.7 and 13.2 ms).
-#ifndef SPH_SWEEP64_BLOCK
-#define SPH_SWEEP64_BLOCK 32
-#endif
 template <typename R>
-static constexpr int sweep_block() { return sizeof(R) == sizeof(double) ? SPH_SWEEP64_BLOCK : 128; }
+static constexpr int sweep_block() { return sizeof(R) == sizeof(double) ? 32 : 128; }
+
+// The FP64 sweep along d on the rows the right-hand side (or f64_rows) stored;
+// transposed: the adjoint's.  norms: accumulate the squares of the increments.
+static int run_lines64(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base,
+                       MF<double> uk, bool transposed, bool norms) {
+  if (!transposed) k_begin(c, SPH_K_SWEEP_R + d);
+  f64_lines(c, d, tau, rhs, x, update, base, uk, transposed, norms);
+  return launch_ok(c);
+}
 
 template <typename R>
 static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> rhs, MF<R> x, int update,
-                     CF<double> base, MF<double> uk, int rows_ready = 0) {
+                     CF<double> base, MF<double> uk, int norms = 0) {
+  if constexpr (sizeof(R) == sizeof(double))
+    if (c->line_solver != SPH_LINES_THOMAS) return run_lines64(c, d, tau, rhs, x, update, base, uk, false, norms);
   SweepArgs<R> S;
   memset(&S, 0, sizeof S);
   S.g = b.g; S.P = c->P; S.c = b.c; S.ub = ub; S.d = d; S.h = (R)(0.5 * tau);
   S.rhs = rhs; S.x = x; S.update = update; S.base = base; S.uk = uk;
   S.scr = b.scr; S.acc = c->acc; S.flag = c->flag;
-  S.rows = c->rows;
   line_layout(c->d64.g, d, S);
   if (sizeof(R) == sizeof(float) && c->line_solver != SPH_LINES_THOMAS && lines_ok(c, d)) {
     SweepArgs<float>& Sf = *reinterpret_cast<SweepArgs<float>*>(&S);
@@ -886,27 +896,6 @@ static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> 
   if (S.nl[1] > mx) mx = S.nl[1];
   if (S.nl[2] > mx) mx = S.nl[2];
   constexpr int TB = sweep_block<R>();
-  if constexpr (sizeof(R) == sizeof(double)) {
-    if (c->line_solver != SPH_LINES_THOMAS && !(d == 2 && c->d64.g.per)) {
-      // walled lines in the FP64 mode: two threads per line, eliminating from both ends
-      static_assert(TB % 32 == 0, "k_sweep2 takes whole warps");
-      constexpr int LPB = TB / 2;
-      dim3 grid2((unsigned)((mx + LPB - 1) / LPB), 3);
-      k_begin(c, SPH_K_SWEEP_R + d);
-      // rows_ready: the right-hand side of this iteration has just stored the
-      // line rows (steps); a sweep on its own (sph_sweep) forms them
-      if (rows_ready && c->rows64) {
-        if (d == 0) k_sweep2<R, 0, true><<<grid2, TB, 0, c->st>>>(S);
-        else if (d == 1) k_sweep2<R, 1, true><<<grid2, TB, 0, c->st>>>(S);
-        else k_sweep2<R, 2, true><<<grid2, TB, 0, c->st>>>(S);
-      } else {
-        if (d == 0) k_sweep2<R, 0, false><<<grid2, TB, 0, c->st>>>(S);
-        else if (d == 1) k_sweep2<R, 1, false><<<grid2, TB, 0, c->st>>>(S);
-        else k_sweep2<R, 2, false><<<grid2, TB, 0, c->st>>>(S);
-      }
-      return launch_ok(c);
-    }
-  }
   dim3 grid((unsigned)((mx + TB - 1) / TB), 3);
   k_begin(c, SPH_K_SWEEP_R + d);
   if (d == 0) k_sweep<R, 0><<<grid, TB, 0, c->st>>>(S);
@@ -959,9 +948,8 @@ static int rhs_impl(sph_ctx* c, Bufs<R>& b, double dt, CF<double> src, int has, 
   CF<R> ub;
   int e = prepare(c, b, c->iterate_set, &ub);
   if (e) return e;
-  CF<double> uk = cf_of(c->iterate_set ? c->U[1 - c->cur] : c->U[c->cur]);
-  if (sizeof(R) == sizeof(double)) return run_rhs(c, b, ub, uk, c->iterate_set, dt, src, has, mf_of((R* const*)R_out));
-  e = run_rhs(c, b, ub, uk, c->iterate_set, dt, src, has, mf_of(b.Rb));
+  if (sizeof(R) == sizeof(double)) return run_rhs(c, b, ub, c->iterate_set, dt, src, has, mf_of((R* const*)R_out));
+  e = run_rhs(c, b, ub, c->iterate_set, dt, src, has, mf_of(b.Rb));
   if (e) return e;
   return convert_out(c, b.Rb, R_out);
 }
@@ -983,7 +971,11 @@ static int sweep_impl(sph_ctx* c, Bufs<R>& b, int dir, double dt, const double* 
   if (cudaMemsetAsync(c->flag, 0, sizeof(int), c->st) != cudaSuccess) return SPH_ERR_CUDA;
   CF<double> base = cf_of(c->U[c->cur]);
   MF<double> ukm = mf_of(c->U[1 - c->cur]);
-  if (sizeof(R) == sizeof(double)) {
+  if constexpr (sizeof(R) == sizeof(double)) {
+    if (c->line_solver != SPH_LINES_THOMAS) {
+      f64_rows(c, ub, dir);
+      c->launches++;
+    }
     e = run_sweep(c, b, dir, dt, ub, cf_of((R* const*)rhs), mf_of((R* const*)x), 0, base, ukm);
   } else {
     e = convert_in(c, rhs, b.Rb);
@@ -1018,11 +1010,12 @@ static int step_impl(sph_ctx* c, Bufs<R>& b, double dt, int n_iter, CF<double> s
     e = prepare(c, b, iter, &ub);
     if (e) break;
     CF<double> ukin = cf_of(iter ? uk : un);
-    e = run_rhs(c, b, ub, ukin, iter, dt, src, has, mf_of(b.Rb));
-    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(b.X1), 0, ukin, mf_of(uk), 1);
-    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(b.X1), mf_of(b.Rb), 0, ukin, mf_of(uk), 1);
-    if (!e && it == n_iter - 1 && cudaMemsetAsync(c->acc, 0, 5 * sizeof(double), c->st) != cudaSuccess) e = SPH_ERR_CUDA;
-    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(b.Rb), mf_of(b.X1), 1, ukin, mf_of(uk), 1);
+    const int last = it == n_iter - 1;   // the residual is the last increment's
+    e = run_rhs(c, b, ub, iter, dt, src, has, mf_of(b.Rb));
+    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(b.X1), 0, ukin, mf_of(uk));
+    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(b.X1), mf_of(b.Rb), 0, ukin, mf_of(uk));
+    if (!e && last && cudaMemsetAsync(c->acc, 0, 5 * sizeof(double), c->st) != cudaSuccess) e = SPH_ERR_CUDA;
+    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(b.Rb), mf_of(b.X1), 1, ukin, mf_of(uk), last);
   }
   if (c->nvtx_open) {  // a stage that failed before its launch check
     nvtxRangePop();
@@ -1140,6 +1133,7 @@ static int adj_axpy(sph_ctx* c, double s, double* x, double* y) {
 // the transposed sweep along d: x = P A_d^{-T} P rhs (P: zero on the wall faces)
 static int run_sweep_T(sph_ctx* c, int d, double tau, CF<double> ub, CF<double> rhs, MF<double> x) {
   Bufs<double>& b = c->d64;
+  if (c->line_solver != SPH_LINES_THOMAS) return run_lines64(c, d, tau, rhs, x, 0, rhs, x, true, false);
   SweepArgs<double> S;
   memset(&S, 0, sizeof S);
   S.g = b.g; S.P = c->P; S.c = b.c; S.ub = ub; S.d = d; S.h = 0.5 * tau;
@@ -1247,10 +1241,10 @@ extern "C" int sph_step_adjoint(sph_ctx* c, double dt, int n_iter, const double*
     const int iter = k > 0 || first;
     CF<double> ub;
     e = prepare(c, b, iter, &ub, Sk);
-    if (!e) e = run_rhs(c, b, ub, cf_of(iter ? Sk : un), iter, dt, src, has, mf_of(b.Rb));
-    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(b.X1), 0, cf_of(Sk), mf_of(Sn), 1);
-    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(b.X1), mf_of(b.Rb), 0, cf_of(Sk), mf_of(Sn), 1);
-    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(b.Rb), mf_of(Sn), 1, cf_of(Sk), mf_of(Sn), 1);
+    if (!e) e = run_rhs(c, b, ub, iter, dt, src, has, mf_of(b.Rb));
+    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(b.X1), 0, cf_of(Sk), mf_of(Sn));
+    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(b.X1), mf_of(b.Rb), 0, cf_of(Sk), mf_of(Sn));
+    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(b.Rb), mf_of(Sn), 1, cf_of(Sk), mf_of(Sn));
   }
   // reverse
   if (!e && cudaMemsetAsync(LN[0], 0, FB, c->st) != cudaSuccess) e = SPH_ERR_CUDA;
@@ -1264,10 +1258,10 @@ extern "C" int sph_step_adjoint(sph_ctx* c, double dt, int n_iter, const double*
     CF<double> ub;
     // the iteration's Ubar, coefficients and sweep solutions
     e = prepare(c, b, iter, &ub, Sk);
-    if (!e) e = run_rhs(c, b, ub, cf_of(iter ? Sk : un), iter, dt, src, has, mf_of(b.Rb));
-    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(XS[0]), 0, cf_of(Sk), mf_of(Sk), 1);
-    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(XS[0]), mf_of(XS[1]), 0, cf_of(Sk), mf_of(Sk), 1);
-    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(XS[1]), mf_of(XS[2]), 0, cf_of(Sk), mf_of(Sk), 1);
+    if (!e) e = run_rhs(c, b, ub, iter, dt, src, has, mf_of(b.Rb));
+    if (!e) e = run_sweep(c, b, 0, dt, ub, cf_of(b.Rb), mf_of(XS[0]), 0, cf_of(Sk), mf_of(Sk));
+    if (!e) e = run_sweep(c, b, 1, dt, ub, cf_of(XS[0]), mf_of(XS[1]), 0, cf_of(Sk), mf_of(Sk));
+    if (!e) e = run_sweep(c, b, 2, dt, ub, cf_of(XS[1]), mf_of(XS[2]), 0, cf_of(Sk), mf_of(Sk));
     // transposed solves, phi first
     if (!e) e = run_sweep_T(c, 2, dt, ub, cf_of(LB), mf_of(MU[2]));
     if (!e) e = run_sweep_T(c, 1, dt, ub, cf_of(MU[2]), mf_of(MU[1]));

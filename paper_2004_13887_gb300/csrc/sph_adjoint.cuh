@@ -10,7 +10,7 @@
 //   dJ/db = lambda - mu_r + g/2,  dJ/da = mu_r + g/2,
 //   g = grad over Ubar of  <mu_r, R(Ubar)> - sum_d <mu_d, A_d(Ubar) x_d>
 // (the x_d and mu_d held fixed).  The transposed solves are the line solvers of
-// sph.cu with TR = true.  g is taken here by reverse-mode differentiation of the
+// sph_fp64_lines.cuh with TR = true.  g is taken here by reverse-mode differentiation of the
 // same row functions the forward kernels run (rhs_c_at, rhs_u_at,
 // assemble_block, scalar_row, coef_at), instantiated on the tape value `ad`: each
 // thread evaluates the rows of one location, recording every operation on a
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(128) k_adj_rhs(AdjArgs A, int kind) {
     RowsOut out;
     ad psi;
     if (kind == 0) {
-      rhs_c_at<2>(ga, g, A.P, c, ub, none, noned, noned, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
+      rhs_c_at<2>(ga, A.P, c, ub, none, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
       psi = out.f[0].v * w0 + out.f[4].v * w4;
     } else if (kind == 1) {
       rhs_u_at<2, 0>(ga, A.P, c, ub, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);

@@ -67,7 +67,7 @@ struct RhsTab {
   Par P;
   Coef<float> c;
   CF<float> ub, ul, Dv;
-  CF<double> un, uk, src;
+  CF<double> src;
   MF<float> Rout;
   float tau;
   int hasD;
@@ -79,10 +79,6 @@ struct LineTab {
   int ng1;    // line groups of the first transverse kind (the scalar launch)
   int pad;
 };
-
-// Never read: rhs_c_at takes the FP64 grid for the FP64 kernels' div(Ubar),
-// which the FP32 instantiation does not form.
-__device__ Geo<double> g_unused_gd;
 
 // dst = src for a descriptor (8-byte words, the whole block), then a barrier
 template <typename T>
@@ -170,9 +166,9 @@ __global__ void __launch_bounds__(128, FUSED_MINB_RHSC) k_rhs_c_f(const RhsTab* 
     if (p.k >= g.np || p.j >= g.nt || p.i >= g.nr) continue;
     const int t = IC(g, p.i, p.j, p.k);
     if (inner)
-      rhs_c_at<0>(g, g_unused_gd, A.P, A.c, A.ub, A.ul, A.un, A.uk, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
+      rhs_c_at<0>(g, A.P, A.c, A.ub, A.ul, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
     else
-      rhs_c_at<1>(g, g_unused_gd, A.P, A.c, A.ub, A.ul, A.un, A.uk, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
+      rhs_c_at<1>(g, A.P, A.c, A.ub, A.ul, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
   }
 }
 
@@ -429,7 +425,7 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
         memset(&R, 0, sizeof R);
         R.g = B.g; R.P = c->P; R.c = B.c;
         R.ub = cf5(B.Ub); R.ul = cf5(B.UbLo); R.Dv = cf5(B.Db);
-        R.un = cf5(un); R.uk = cf5(uk); R.src = cf5(c->src);
+        R.src = cf5(c->src);
         R.Rout = mf5(B.Rb);
         R.tau = (float)dt;
         R.hasD = it;

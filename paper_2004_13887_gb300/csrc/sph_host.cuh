@@ -9,6 +9,7 @@
 
 #include "../../include/sph.h"
 #include "sph_kernels.cuh"
+#include "sph_fp64_tab.cuh"
 
 // Device buffers of one precision.
 template <typename R>
@@ -46,7 +47,9 @@ struct sph_ctx {
   Bufs<double> d64;      // FP64 metric/background tables always; bulk buffers in FP64 mode
   Bufs<float> d32;       // bulk buffers in mixed mode
   double* rows64;        // FP64 mode: the line rows the right-hand side stores for the sweeps
-  Rows64 rows;           // pointers into rows64 (all null in mixed mode)
+  f64::Rows rows;        // pointers into rows64 (all null in mixed mode)
+  double* tab64;         // FP64 mode: the metric tables of its kernels
+  f64::Tabs tabs;        // pointers into tab64
   long long launches;
   long unknowns[5];
   // per-kernel timing
@@ -109,11 +112,23 @@ struct sph_batch {
   int fstreams;            // side streams created
 };
 
+// The launches of the FP64 mode's stages (sph_fp64.cu), on the context's stream
+// (f64_rhs: the momentum rows on its side streams): the metric tables, the
+// coefficients at Ubar, the right-hand side (which stores the line rows), the
+// line rows along one direction alone, and a sweep on stored rows.
+void f64_tables(sph_ctx* c);
+void f64_coef(sph_ctx* c, CF<double> ub);
+void f64_rhs(sph_ctx* c, CF<double> ub, CF<double> D, int hasD, double tau, CF<double> src, int has_src, MF<double> R);
+void f64_rows(sph_ctx* c, CF<double> ub, int dir);
+void f64_lines(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base, MF<double> uk,
+               bool transposed, bool norms);
+
 // frees what sph_batch_capture_fused allocated (sph_batch.cu)
 void batch_fused_free(sph_batch* b);
 #ifdef SPH_CHECKED
-// the bounds counter of the batched kernels' translation unit into h, then zeroed
+// the bounds counters of the other translation units into h, then zeroed
 int bounds_take_batch(int* h);
+int bounds_take_f64(int* h);
 #endif
 
 

@@ -159,10 +159,8 @@ __device__ __forceinline__ bool tile_inner(const G& g) {
 }
 // The FP32 stencil kernels are bound by load latency: full occupancy (16
 // blocks of 128 threads, 32 registers) pays for its few register spills
-// (measured: the right-hand side 17 % faster than at 64 registers).  The FP64
-// instantiations keep their registers: they are bound by the FP64 pipe, and
-// capping them at 128, 96 or 80 registers (up to 6 blocks an SM) left the
-// FP64 right-hand side at 20.8 ms per step.
+// (measured: the right-hand side 17 % faster than at 64 registers).  (The FP64
+// mode has its own stencil kernels, sph_fp64.cuh.)
 #define STENCIL_MINB(R) (sizeof(R) == 4 ? 16 : 1)
 
 // grid of tiles of tj x ti rows of phi points (128 / (tj ti) each) over an
@@ -184,22 +182,6 @@ __global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_coef(Geo<R> g, Par P, 
   int t = IC(g, i, j, k);
   if (inner) coef_at<0>(g, P, ub, c, i, j, k, t);
   else coef_at<W ? 2 : 1>(g, P, ub, c, i, j, k, t);
-}
-
-// div(Ubar) at centre (i,j,k), in FP64 from U^n and U^k (Ubar = (U^n+U^k)/2).
-__device__ __forceinline__ double div_ubar(const Geo<double>& g, const CF<double>& un, const CF<double>& uk, int i,
-                                           int j, int k) {
-  const double *ur0 = un.f[1], *ur1 = uk.f[1], *ut0 = un.f[2], *ut1 = uk.f[2], *up0 = un.f[3], *up1 = uk.f[3];
-  int a0 = IRf(g, i, j, k), a1 = IRf(g, i + 1, j, k);
-  int b0 = ITf(g, i, j, k), b1 = ITf(g, i, j + 1, k);
-  int kp = g.per ? wrapk(g, k + 1) : k + 1;
-  int c0 = IPf(g, i, j, k), c1 = IPf(g, i, j, kp);
-  double ir = g.irc[i], is = g.isc[j];
-  double f0 = g.rf[i] * g.rf[i], f1 = g.rf[i + 1] * g.rf[i + 1];
-  double dr_ = (f1 * (ur0[a1] + ur1[a1]) - f0 * (ur0[a0] + ur1[a0])) * ir * ir * g.idr;
-  double dt_ = (g.sf[j + 1] * (ut0[b1] + ut1[b1]) - g.sf[j] * (ut0[b0] + ut1[b0])) * ir * is * g.idth;
-  double dp_ = ((up0[c1] + up1[c1]) - (up0[c0] + up1[c0])) * ir * is * g.idph;
-  return 0.5 * (dr_ + dt_ + dp_);
 }
 
 // div(Ubar) at centre (i,j,k) in FP32 mode, from the pair (hi = Ubar, lo) of the
@@ -249,69 +231,12 @@ __device__ __forceinline__ R div_ubar_of(const Geo<R>& g, const CF<R>& ub, int i
   return dr_ + dt_ + dp_;
 }
 
-// Line rows of the FP64 mode.  The right-hand side evaluates, at every unknown,
-// the rows of D_r, D_theta and D_phi at Ubar -- the same rows each sweep's line
-// matrix I + tau/2 D_d is assembled from.  In the FP64 mode the arithmetic, not
-// memory, bounds the step, so the right-hand side stores the rows it has formed
-// and the sweeps read them instead of forming them again (45 doubles a cell).
-//   c[d]: 12 planes over the centres, the p- and T-rows of D_d: p-row wp0, wp2,
-//         wT0, wT1, wT2, v0, v1 (wp1 is zero: advection has no diagonal); T-row
-//         wT0, wT1, wT2, v0, v1; v_q = a gd_q + wv_q (the u_d couplings);
-//   f[d]: 5 planes over the d-faces, the normal-velocity row of D_d (wp0, wp1,
-//         wu0, wu1, wu2);
-//   s[c]: 6 planes over the c-faces, the rows of velocity component c along its
-//         two transverse directions in increasing order (3 weights each).
-// NoRows (every other caller) stores nothing.
-struct NoRows { static constexpr bool on = false; };
-struct Rows64 {
-  static constexpr bool on = true;
-  double* c[3];
-  double* f[3];
-  double* s[3];
-  long nc, nf[3];  // centres; faces of each kind
-};
-// slot of direction d among the transverse directions of component cc
-__host__ __device__ constexpr int trans_slot(int cc, int d) { return d < cc ? d : d - 1; }
-
-template <typename RowsT, typename R>
-__device__ __forceinline__ void rows_put_c(const RowsT& o, int d, int isT, int t, const RowC<R>& w) {
-  if constexpr (RowsT::on && std::is_same<R, double>::value) {
-    double* p = o.c[d] + t;
-    const long n = o.nc;
-    if (!isT) {
-      p[0] = w.wp[0]; p[n] = w.wp[2]; p[2 * n] = w.wT[0]; p[3 * n] = w.wT[1]; p[4 * n] = w.wT[2];
-      p[5 * n] = w.a * w.gd[0] + w.wv[0]; p[6 * n] = w.a * w.gd[1] + w.wv[1];
-    } else {
-      p[7 * n] = w.wT[0]; p[8 * n] = w.wT[1]; p[9 * n] = w.wT[2];
-      p[10 * n] = w.a * w.gd[0] + w.wv[0]; p[11 * n] = w.a * w.gd[1] + w.wv[1];
-    }
-  }
-}
-template <typename RowsT, typename R>
-__device__ __forceinline__ void rows_put_f(const RowsT& o, int d, int t, const R* wp, const R* wu) {
-  if constexpr (RowsT::on && std::is_same<R, double>::value) {
-    double* p = o.f[d] + t;
-    const long n = o.nf[d];
-    p[0] = wp[0]; p[n] = wp[1]; p[2 * n] = wu[0]; p[3 * n] = wu[1]; p[4 * n] = wu[2];
-  }
-}
-template <typename RowsT, typename R>
-__device__ __forceinline__ void rows_put_s(const RowsT& o, int cc, int d, int t, const R* w) {
-  if constexpr (RowsT::on && std::is_same<R, double>::value) {
-    const long n = o.nf[cc];
-    double* p = o.s[cc] + 3 * trans_slot(cc, d) * n + t;
-    p[0] = w[0]; p[n] = w[1]; p[2 * n] = w[2];
-  }
-}
-
 // R = -(U^k - U^n) - tau (N(Ubar) + G - S) for the p- and T-rows: one thread per
-// centre; written to Rout.f[0][t], Rout.f[4][t] (a field pair, or the adjoint's
-// slots).
-template <int CIJ, typename R, typename Out, typename RowsT = NoRows>
-__device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Geo<double>& gd, const Par& P, const Coef<R>& c,
-                                         const CF<R>& ub, const CF<R>& ul, const CF<double>& un, const CF<double>& uk,
-                                         const CF<R>& D, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const Out& Rout, int i, int j, int k, int t, const RowsT& rows = RowsT()) {
+// centre; written to Rout.f[0][t], Rout.f[4][t].
+template <int CIJ, typename R, typename Out>
+__device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Par& P, const Coef<R>& c,
+                                         const CF<R>& ub, const CF<R>& ul, const CF<R>& D, int hasD, const CF<double>& src, int has_src, R tau,
+                                         const Out& Rout, int i, int j, int k, int t) {
   const auto Pp = ub.f[0];
   const auto UR = ub.f[1];
   const auto UT = ub.f[2];
@@ -335,20 +260,17 @@ __device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Geo<double>& gd,
     else { uv[0] = vp<CIJ>(g, UP, i, j, k); uv[1] = vp<CIJ>(g, UP, i, j, k + 1); }
     RowC<R> w;
     row_c(g, P, c, d, 0, i, j, k, w);
-    rows_put_c(rows, d, 0, t, w);
     accp += w.wp[0] * pv[0] + w.wp[2] * pv[2] + w.wT[0] * Tv[0] + w.wT[1] * Tv[1] + w.wT[2] * Tv[2]
           + w.wv[0] * uv[0] + w.wv[1] * uv[1];
     if (d == 0) accp += w.adv * g.dbgp[i] - w.dif * g.lapT[i];
     ap = w.a;
     row_c(g, P, c, d, 1, i, j, k, w);
-    rows_put_c(rows, d, 1, t, w);
     accT += w.wT[0] * Tv[0] + w.wT[1] * Tv[1] + w.wT[2] * Tv[2] + w.wv[0] * uv[0] + w.wv[1] * uv[1];
     if (d == 0) accT += w.adv * g.dbgT[i] - w.dif * g.lapT[i];
     aT = w.a;
   }
   R divu;
   if constexpr (is_f32<R>) divu = div_ubar_ff(g, ub, ul, i, j, k);
-  else if constexpr (std::is_same<R, double>::value) divu = div_ubar(gd, un, uk, i, j, k);
   else divu = div_ubar_of(g, ub, i, j, k);
   // Cross terms of the viscous dissipation: the centred derivative sums
   // d_r u_t + d_t u_r / r, d_r u_p + d_p u_r / (r sin), d_t u_p / r + d_p u_t / (r sin)
@@ -368,36 +290,26 @@ __device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Geo<double>& gd,
   Rout.f[4][t] = -d4 - tau * NT;
 }
 
-// one block per tile.  FP64: at least SPH_RHSC64_MINB blocks of 128 threads
-// per SM (the compiler would otherwise take ~190 registers a thread for the
-// centre rows it keeps live until their stores, leaving two blocks per SM).
-#ifndef SPH_RHSC64_MINB
-#define SPH_RHSC64_MINB 4
-#endif
+// one block per tile
 template <typename R, bool W>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? STENCIL_MINB(R) : SPH_RHSC64_MINB) k_rhs_c(Geo<R> g, Geo<double> gd, Par P, Coef<R> c, CF<R> ub, CF<R> ul,
-                                               CF<double> un, CF<double> uk, CF<R> D, int hasD, CF<double> src,
-                                               int has_src, R tau, MF<R> Rout, Rows64 rows) {
+__global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_c(Geo<R> g, Par P, Coef<R> c, CF<R> ub, CF<R> ul, CF<R> D,
+                                                                int hasD, CF<double> src, int has_src, R tau,
+                                                                MF<R> Rout) {
   int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
       i = blockIdx.z * blockDim.z + threadIdx.z;
   bool inner = tile_inner(g) && !g.hasw;  // with wall data every tile takes the checked path
   if (k >= g.np || j >= g.nt || i >= g.nr) return;
   int t = IC(g, i, j, k);
-  if constexpr (std::is_same<R, double>::value) {  // the FP64 mode stores its line rows
-    if (inner) rhs_c_at<0>(g, gd, P, c, ub, ul, un, uk, D, hasD, src, has_src, tau, Rout, i, j, k, t, rows);
-    else rhs_c_at<W ? 2 : 1>(g, gd, P, c, ub, ul, un, uk, D, hasD, src, has_src, tau, Rout, i, j, k, t, rows);
-  } else {
-    if (inner) rhs_c_at<0>(g, gd, P, c, ub, ul, un, uk, D, hasD, src, has_src, tau, Rout, i, j, k, t);
-    else rhs_c_at<W ? 2 : 1>(g, gd, P, c, ub, ul, un, uk, D, hasD, src, has_src, tau, Rout, i, j, k, t);
-  }
+  if (inner) rhs_c_at<0>(g, P, c, ub, ul, D, hasD, src, has_src, tau, Rout, i, j, k, t);
+  else rhs_c_at<W ? 2 : 1>(g, P, c, ub, ul, D, hasD, src, has_src, tau, Rout, i, j, k, t);
 }
 
 // R for the momentum row of component D on its faces: one thread per face
 // (zero on wall faces, which are not unknowns); written to Rout.f[1 + D][t].
-template <int CIJ, int D, typename R, typename Out, typename RowsT = NoRows>
+template <int CIJ, int D, typename R, typename Out>
 __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Coef<R>& c, const CF<R>& ub,
                                          const CF<R>& Dv, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const Out& Rout, int i, int j, int k, int t, const RowsT& rows = RowsT()) {
+                                         const Out& Rout, int i, int j, int k, int t) {
   const auto Pp = ub.f[0];
   const auto UR = ub.f[1];
   const auto UT = ub.f[2];
@@ -407,14 +319,11 @@ __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Co
   R acc;
   if (D == 0) {
     row_f(g, P, c, UR, 0, i, j, k, wp, wu);
-    rows_put_f(rows, 0, t, wp, wu);
     acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i - 1, j, k))
         + wu[0] * UR[IRf(g, i - 1, j, k)] + wu[1] * UR[t] + wu[2] * UR[IRf(g, i + 1, j, k)];
     row_s<CIJ>(g, P, c, ub, 0, 1, i, j, k, w);
-    rows_put_s(rows, 0, 1, t, w);
     acc += w[0] * vr<CIJ>(g, UR, i, j - 1, k) + w[1] * UR[t] + w[2] * vr<CIJ>(g, UR, i, j + 1, k);
     row_s<CIJ>(g, P, c, ub, 0, 2, i, j, k, w);
-    rows_put_s(rows, 0, 2, t, w);
     acc += w[0] * vr<CIJ>(g, UR, i, j, k - 1) + w[1] * UR[t] + w[2] * vr<CIJ>(g, UR, i, j, k + 1);
     // hydrostatic part: (1/rho_f) d p_ref/dr + g = (1 - b) e + g b, b = 1 - rho_ref,f / rho_f
     int c0 = IC(g, i - 1, j, k), c1 = IC(g, i, j, k);
@@ -438,14 +347,11 @@ __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Co
   } else if (D == 1) {
     R ir = g.irc[i];
     row_f(g, P, c, UT, 1, i, j, k, wp, wu);
-    rows_put_f(rows, 1, t, wp, wu);
     acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i, j - 1, k))
         + wu[0] * UT[ITf(g, i, j - 1, k)] + wu[1] * UT[t] + wu[2] * UT[ITf(g, i, j + 1, k)];
     row_s<CIJ>(g, P, c, ub, 1, 0, i, j, k, w);
-    rows_put_s(rows, 1, 0, t, w);
     acc += w[0] * vt<CIJ>(g, UT, i - 1, j, k) + w[1] * UT[t] + w[2] * vt<CIJ>(g, UT, i + 1, j, k);
     row_s<CIJ>(g, P, c, ub, 1, 2, i, j, k, w);
-    rows_put_s(rows, 1, 2, t, w);
     acc += w[0] * vt<CIJ>(g, UT, i, j, k - 1) + w[1] * UT[t] + w[2] * vt<CIJ>(g, UT, i, j, k + 1);
     R isfj = g.isf[j], cfj = g.cf[j], cotf = g.cotf[j];
     R irh = sdiv(R(2), rho_at(g, c, i, j - 1, k) + rho_at(g, c, i, j, k));
@@ -469,14 +375,11 @@ __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Co
   } else {
     R ir = g.irc[i], is = g.isc[j], cot = g.cotc[j];
     row_f(g, P, c, UP, 2, i, j, k, wp, wu);
-    rows_put_f(rows, 2, t, wp, wu);
     acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i, j, k - 1))
         + wu[0] * vp<CIJ>(g, UP, i, j, k - 1) + wu[1] * UP[t] + wu[2] * vp<CIJ>(g, UP, i, j, k + 1);
     row_s<CIJ>(g, P, c, ub, 2, 0, i, j, k, w);
-    rows_put_s(rows, 2, 0, t, w);
     acc += w[0] * vp<CIJ>(g, UP, i - 1, j, k) + w[1] * UP[t] + w[2] * vp<CIJ>(g, UP, i + 1, j, k);
     row_s<CIJ>(g, P, c, ub, 2, 1, i, j, k, w);
-    rows_put_s(rows, 2, 1, t, w);
     acc += w[0] * vp<CIJ>(g, UP, i, j - 1, k) + w[1] * UP[t] + w[2] * vp<CIJ>(g, UP, i, j + 1, k);
     R s = g.sc[j], cj = g.cc[j];
     R irh = sdiv(R(2), rho_at(g, c, i, j, k - 1) + rho_at(g, c, i, j, k));
@@ -507,7 +410,7 @@ __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Co
 // one block per tile of faces; zero on wall faces, which are not unknowns
 template <typename R, int D, bool W>
 __global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_u(Geo<R> g, Par P, Coef<R> c, CF<R> ub, CF<R> Dv, int hasD,
-                                               CF<double> src, int has_src, R tau, MF<R> Rout, Rows64 rows) {
+                                               CF<double> src, int has_src, R tau, MF<R> Rout) {
   int nj = g.nt + (D == 1), nk = D == 2 ? g.npf : g.np;
   int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
       i = blockIdx.z * blockDim.z + threadIdx.z;
@@ -516,13 +419,8 @@ __global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_u(Geo<R> g, Par P,
   int t = (i * nj + j) * nk + k;
   bool wall = D == 0 ? (i == 0 || i == g.nr) : D == 1 ? (j == 0 || j == g.nt) : (!g.per && (k == 0 || k == g.np));
   if (wall) { Rout.f[1 + D][t] = R(0); return; }
-  if constexpr (std::is_same<R, double>::value) {  // the FP64 mode stores its line rows
-    if (inner) rhs_u_at<0, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t, rows);
-    else rhs_u_at<W ? 2 : 1, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t, rows);
-  } else {
-    if (inner) rhs_u_at<0, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
-    else rhs_u_at<W ? 2 : 1, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
-  }
+  if (inner) rhs_u_at<0, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
+  else rhs_u_at<W ? 2 : 1, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
 }
 
 // ------------------------------------------------------------ line solvers
@@ -631,7 +529,6 @@ struct SweepArgs {
   int a0[3], nb[3], b0[3];
   double* acc;            // 5 sums of squares (mode 1)
   int* flag;
-  Rows64 rows;            // FP64 mode: the line rows the right-hand side stored
 };
 
 // Per-thread sums of squares of the increments, per field (the iteration
@@ -1121,354 +1018,6 @@ __global__ void __launch_bounds__(128) k_sweep(SweepArgs<R> S) {
     for (int f = 0; f < 5; f++) {
       double v = ss.warp_total(f);
       if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(S.acc + f, v);
-    }
-  }
-}
-
-// ------------------------------------------------- two-sided line solvers
-// Walled (non-cyclic) lines, forward sweeps: two threads per line, one
-// eliminating downwards from the first cell, the other upwards from the last
-// (block Thomas "burning at both ends"): the same block operations as the
-// one-sided solver above in two dependent chains of half the length, so twice
-// the threads for the same arithmetic.  Lanes 0-15 of a warp take the top side
-// of 16 lines, lanes 16-31 the bottom side of the same lines (partner = lane ^ 16).
-//   top (s = 0), cells 0 .. h-1 (h = ceil(n/2)):  S_m = B_m - A_m E_{m-1},
-//     E_m = S_m^{-1} C_m, g_m = S_m^{-1} (r_m - A_m g_{m-1}),  x_m = g_m - E_m x_{m+1};
-//   bottom (s = 1), cells n-1 .. h, the roles of A and C swapped:
-//     S_m = B_m - C_m E_{m+1}, E_m = S_m^{-1} A_m, g_m = S_m^{-1} (r_m - C_m g_{m+1}),
-//     x_m = g_m - E_m x_{m-1}.
-// At the meeting cells h-1 and h each side solves for its own boundary value,
-// (I - E_o E_p) x_o = g_o - E_o g_p, with the partner's (E_p, g_p) from a
-// shuffle (the same instructions on both sides), then substitutes outwards.
-// Every lane runs the same instructions: a lane past the last line works on
-// the last line and stores nothing; a singular pivot sets the flag and carries
-// NaN on, so that no lane leaves the shuffles early.
-constexpr int SWEEP2_LINES = 16;  // lines per warp
-
-template <typename R>
-__device__ __forceinline__ void inv3_or_nan(const R* S, R* I, int* bad) {
-  if (!inv3(S, I)) {
-    *bad |= FLAG_SINGULAR;
-#pragma unroll
-    for (int q = 0; q < 9; q++) I[q] = R(NAN);
-  }
-}
-
-// Block m of (I + h D_d) on a walled line from the stored rows: rc the 12 centre
-// values of the p- and T-rows, rf the 5 values of the normal-velocity row on
-// face m + 1 (m < n - 1); the same entries and wall folds as assemble_pts.
-template <typename R>
-__device__ __forceinline__ void assemble_rows(const R* rc, const R* rf, int n, int m, R h, R* A, R* B, R* C) {
-#pragma unroll
-  for (int q = 0; q < 9; q++) { A[q] = R(0); B[q] = R(0); C[q] = R(0); }
-  A[0] = h * rc[0]; A[1] = h * rc[2]; A[2] = h * rc[5];
-  B[1] = h * rc[3]; B[2] = h * rc[6];
-  C[0] = h * rc[1]; C[1] = h * rc[4];
-  A[4] = h * rc[7]; A[5] = h * rc[10];
-  B[4] = h * rc[8]; B[5] = h * rc[11];
-  C[4] = h * rc[9];
-  if (m < n - 1) {
-    A[8] = h * rf[2];
-    B[6] = h * rf[0]; B[8] = h * rf[3];
-    C[6] = h * rf[1]; C[8] = h * rf[4];
-  }
-  B[0] += R(1); B[4] += R(1); B[8] += R(1);
-  if (m == 0) {
-    B[0] += A[0]; B[1] += A[1]; B[3] += A[3]; B[4] += A[4];
-#pragma unroll
-    for (int q = 0; q < 9; q++) A[q] = R(0);
-  }
-  if (m == n - 1) {
-    B[0] += C[0]; B[1] += C[1]; B[3] += C[3]; B[4] += C[4];
-#pragma unroll
-    for (int q = 0; q < 9; q++) C[q] = R(0);
-    B[2] = R(0); B[5] = R(0);
-    A[8] = R(0); B[6] = R(0); B[7] = R(0); B[8] = R(1);
-  }
-}
-
-template <typename R, int D, bool ROWS>
-__device__ void block_line2(const SweepArgs<R>& S, int line, bool valid, int a, int b, int side, SqSum<R>& ss,
-                            int* bad) {
-  const Geo<R>& g = S.g;
-  constexpr int d = D;
-  const int n = d == 0 ? g.nr : d == 1 ? g.nt : g.np;
-  const int nl = S.nl[0];
-  R* scr = S.scr + S.scr_off[0];
-  constexpr int W = 12;
-  const int h = (n + 1) / 2;
-  const int cnt = side ? n - h : h;  // cells of this side (the bottom side of a one-cell line has none)
-  auto cell = [&](int s) { return side ? n - 1 - s : s; };
-  CPt<R> cqn;
-  FPt<R> fqn;
-  R rcn[ROWS ? 12 : 1], rfn[ROWS ? 5 : 1];
-  R r0n = R(0), r4n = R(0), run = R(0);
-  auto fetch = [&](int m) {
-    int i, j, k, fi, fj, fk;
-    line_pos(d, a, b, m, i, j, k);
-    const int ic = IC(g, i, j, k);
-    if constexpr (ROWS) {
-      const R* pc = S.rows.c[d] + ic;
-#pragma unroll
-      for (int q = 0; q < 12; q++) rcn[q] = pc[q * S.rows.nc];
-    } else {
-      cqn = load_c(S.c, d, ic);
-      fqn = {R(1), R(1), R(0)};
-    }
-    run = R(0);
-    if (m < n - 1) {
-      next_face(d, n, m, i, j, k, fi, fj, fk);
-      const int fx = face_idx(g, d, fi, fj, fk);
-      if constexpr (ROWS) {
-        const R* pf = S.rows.f[d] + fx;
-#pragma unroll
-        for (int q = 0; q < 5; q++) rfn[q] = pf[q * S.rows.nf[d]];
-      } else {
-        fqn = load_f(g, S.c, S.ub.f[1 + d], d, fi, fj, fk);
-      }
-      run = S.rhs.f[1 + d][fx];
-    }
-    r0n = S.rhs.f[0][ic];
-    r4n = S.rhs.f[4][ic];
-  };
-  R E[9], gv[3];
-#pragma unroll
-  for (int q = 0; q < 9; q++) E[q] = R(0);
-  gv[0] = gv[1] = gv[2] = R(0);
-  if (cnt > 0) fetch(cell(0));
-  for (int s = 0; s < cnt; s++) {
-    const int m = cell(s);
-    int i, j, k;
-    line_pos(d, a, b, m, i, j, k);
-    R A[9], B[9], C[9];
-    R rr[3] = {r0n, r4n, run};
-    if constexpr (ROWS) {
-      R rc[12], rf[5];
-#pragma unroll
-      for (int q = 0; q < 12; q++) rc[q] = rcn[q];
-#pragma unroll
-      for (int q = 0; q < 5; q++) rf[q] = rfn[q];
-      if (s + 1 < cnt) fetch(cell(s + 1));
-      assemble_rows(rc, rf, n, m, S.h, A, B, C);
-    } else {
-      const CPt<R> cq = cqn;
-      const FPt<R> fq = fqn;
-      if (s + 1 < cnt) fetch(cell(s + 1));
-      int fi, fj, fk;
-      next_face(d, n, m, i, j, k, fi, fj, fk);
-      assemble_pts(g, S.P, cq, fq, d, n, 0, m, i, j, fi, fj, S.h, A, B, C);
-    }
-    // L couples to the cell already eliminated, U to the next one
-    R L[9], U[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) { L[q] = side ? C[q] : A[q]; U[q] = side ? A[q] : C[q]; }
-    R Sm[9], y[3];
-#pragma unroll
-    for (int r = 0; r < 3; r++) {
-#pragma unroll
-      for (int q = 0; q < 3; q++)
-        Sm[r * 3 + q] = B[r * 3 + q] - (L[r * 3] * E[q] + L[r * 3 + 1] * E[3 + q] + L[r * 3 + 2] * E[6 + q]);
-      y[r] = rr[r] - (L[r * 3] * gv[0] + L[r * 3 + 1] * gv[1] + L[r * 3 + 2] * gv[2]);
-    }
-    R Si[9];
-    inv3_or_nan(Sm, Si, bad);
-#pragma unroll
-    for (int r = 0; r < 3; r++) {
-#pragma unroll
-      for (int q = 0; q < 3; q++) E[r * 3 + q] = Si[r * 3] * U[q] + Si[r * 3 + 1] * U[3 + q] + Si[r * 3 + 2] * U[6 + q];
-      gv[r] = Si[r * 3] * y[0] + Si[r * 3 + 1] * y[1] + Si[r * 3 + 2] * y[2];
-    }
-    if (s + 1 < cnt && valid) {
-      R* sp = scr + m * W * nl + line;
-#pragma unroll
-      for (int q = 0; q < 9; q++) sp[q * nl] = E[q];
-#pragma unroll
-      for (int q = 0; q < 3; q++) sp[(9 + q) * nl] = gv[q];
-    }
-  }
-  // the meeting cells: the partner's last factors (zero for the empty bottom
-  // side of a one-cell line, which leaves x = g on the top side)
-  R Ep[9], gp[3];
-#pragma unroll
-  for (int q = 0; q < 9; q++) Ep[q] = __shfl_xor_sync(0xffffffffu, E[q], 16);
-#pragma unroll
-  for (int q = 0; q < 3; q++) gp[q] = __shfl_xor_sync(0xffffffffu, gv[q], 16);
-  R Mm[9], rhs[3], Mi[9], xs[3];
-#pragma unroll
-  for (int r = 0; r < 3; r++) {
-#pragma unroll
-    for (int q = 0; q < 3; q++)
-      Mm[r * 3 + q] = (r == q ? R(1) : R(0)) - (E[r * 3] * Ep[q] + E[r * 3 + 1] * Ep[3 + q] + E[r * 3 + 2] * Ep[6 + q]);
-    rhs[r] = gv[r] - (E[r * 3] * gp[0] + E[r * 3 + 1] * gp[1] + E[r * 3 + 2] * gp[2]);
-  }
-  inv3_or_nan(Mm, Mi, bad);
-#pragma unroll
-  for (int r = 0; r < 3; r++) xs[r] = Mi[r * 3] * rhs[0] + Mi[r * 3 + 1] * rhs[1] + Mi[r * 3 + 2] * rhs[2];
-  // substitution outwards from the meeting cell; the factors of the next cell
-  // out are loaded before the current one is stored
-  R En[9], gn[3];
-  if (cnt >= 2) {
-    const R* sp = scr + cell(cnt - 2) * W * nl + line;
-#pragma unroll
-    for (int q = 0; q < 9; q++) En[q] = sp[q * nl];
-#pragma unroll
-    for (int q = 0; q < 3; q++) gn[q] = sp[(9 + q) * nl];
-  }
-  for (int s = cnt - 1; s >= 0; s--) {
-    const int m = cell(s);
-    if (s < cnt - 1) {
-      R E_[9], g_[3];
-#pragma unroll
-      for (int q = 0; q < 9; q++) E_[q] = En[q];
-#pragma unroll
-      for (int q = 0; q < 3; q++) g_[q] = gn[q];
-      if (s >= 1) {
-        const R* sp = scr + cell(s - 1) * W * nl + line;
-#pragma unroll
-        for (int q = 0; q < 9; q++) En[q] = sp[q * nl];
-#pragma unroll
-        for (int q = 0; q < 3; q++) gn[q] = sp[(9 + q) * nl];
-      }
-      R xn[3];
-#pragma unroll
-      for (int r = 0; r < 3; r++) xn[r] = g_[r] - (E_[r * 3] * xs[0] + E_[r * 3 + 1] * xs[1] + E_[r * 3 + 2] * xs[2]);
-#pragma unroll
-      for (int q = 0; q < 3; q++) xs[q] = xn[q];
-    }
-    if (valid) {
-      int i, j, k;
-      line_pos(d, a, b, m, i, j, k);
-      int ic = IC(g, i, j, k);
-      put(S, 0, ic, xs[0], ss, bad);
-      put(S, 4, ic, xs[1], ss, bad);
-      int fi = i, fj = j, fk = k;
-      if (m < n - 1) {
-        if (d == 0) fi = m + 1; else if (d == 1) fj = m + 1; else fk = m + 1;
-        put(S, 1 + d, face_idx(g, d, fi, fj, fk), xs[2], ss, bad);
-      } else {
-        if (d == 0) fi = n; else if (d == 1) fj = n; else fk = n;
-        put_wall(S, 1 + d, face_idx(g, d, fi, fj, fk));
-        int gi = i, gj = j, gk = k;
-        if (d == 0) gi = 0; else if (d == 1) gj = 0; else gk = 0;
-        put_wall(S, 1 + d, face_idx(g, d, gi, gj, gk));
-      }
-    }
-  }
-}
-
-// The scalar (transverse-component) lines the same way: Thomas from both ends,
-// (1 - e_o e_p) x_o = g_o - e_o g_p at the meeting cells.
-template <typename R, int D, int KIND, bool ROWS>
-__device__ void scalar_line2(const SweepArgs<R>& S, int line, bool valid, int a, int b, int side, SqSum<R>& ss,
-                             int* bad) {
-  const Geo<R>& g = S.g;
-  constexpr int d = D, kind = KIND;
-  const int cc = trans_comp(d, kind);
-  const int n = d == 0 ? g.nr : d == 1 ? g.nt : g.np;
-  const int nl = S.nl[kind];
-  R* scr = S.scr + S.scr_off[kind];
-  const R* rhs = S.rhs.f[1 + cc];
-  const int h = (n + 1) / 2;
-  const int cnt = side ? n - h : h;
-  auto cell = [&](int s) { return side ? n - 1 - s : s; };
-  SPt<R> qn;
-  R wn[3];
-  R rn = R(0);
-  auto fetch = [&](int m) {
-    int i, j, k;
-    line_pos(d, a, b, m, i, j, k);
-    const int fx = face_idx(g, cc, i, j, k);
-    if constexpr (ROWS) {
-      const long nfc = S.rows.nf[cc];
-      const R* ps = S.rows.s[cc] + 3 * trans_slot(cc, d) * nfc + fx;
-      wn[0] = ps[0]; wn[1] = ps[nfc]; wn[2] = ps[2 * nfc];
-    } else {
-      qn = load_s<2>(g, S.c, S.ub, cc, d, i, j, k);
-    }
-    rn = rhs[fx];
-  };
-  R e = R(0), gy = R(0);
-  if (cnt > 0) fetch(cell(0));
-  for (int s = 0; s < cnt; s++) {
-    const int m = cell(s);
-    int i, j, k;
-    line_pos(d, a, b, m, i, j, k);
-    const R r = rn;
-    R w[3];
-    if constexpr (ROWS) {
-      w[0] = wn[0]; w[1] = wn[1]; w[2] = wn[2];
-      if (s + 1 < cnt) fetch(cell(s + 1));
-    } else {
-      const SPt<R> q = qn;
-      if (s + 1 < cnt) fetch(cell(s + 1));
-      row_sw(g, S.P, q, cc, d, i, j, w);
-    }
-    R am = S.h * w[0], bm = R(1) + S.h * w[1], cm = S.h * w[2];
-    if (m == 0) { bm -= am; am = R(0); }
-    if (m == n - 1) { bm -= cm; cm = R(0); }
-    const R lo = side ? cm : am, up = side ? am : cm;
-    R den = bm - lo * e;
-    if (den == R(0) || !isfinite(den)) *bad |= FLAG_SINGULAR;
-    R iden = sdiv(R(1), den);
-    e = up * iden;
-    gy = (r - lo * gy) * iden;
-    if (s + 1 < cnt && valid) {
-      R* sp = scr + m * 3 * nl + line;
-      sp[0] = e;
-      sp[nl] = gy;
-    }
-  }
-  const R ep = __shfl_xor_sync(0xffffffffu, e, 16), gp = __shfl_xor_sync(0xffffffffu, gy, 16);
-  R x = sdiv(gy - e * gp, R(1) - e * ep);
-  R en = R(0), gn = R(0);
-  if (cnt >= 2) {
-    const int mm = cell(cnt - 2);
-    en = scr[mm * 3 * nl + line];
-    gn = scr[mm * 3 * nl + nl + line];
-  }
-  for (int s = cnt - 1; s >= 0; s--) {
-    const int m = cell(s);
-    if (s < cnt - 1) {
-      const R e_ = en, g_ = gn;
-      if (s >= 1) {
-        const int mm = cell(s - 1);
-        en = scr[mm * 3 * nl + line];
-        gn = scr[mm * 3 * nl + nl + line];
-      }
-      x = g_ - e_ * x;
-    }
-    if (valid) {
-      int i, j, k;
-      line_pos(d, a, b, m, i, j, k);
-      scalar_put(S, cc, i, j, k, x, ss, bad);
-    }
-  }
-}
-
-// one warp per 16 lines of one kind (blockIdx.y): lanes l and l + 16 share a line
-template <typename R, int D, bool ROWS>
-__global__ void __launch_bounds__(128) k_sweep2(SweepArgs<R> S) {
-  const int kind = blockIdx.y;
-  const int nl = S.nl[kind];
-  const int lane = threadIdx.x & 31;
-  const int base = (blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / 2;  // first line of the warp
-  if (base >= nl) return;  // the whole warp: no line of this kind left
-  const int side = lane >> 4;
-  const int l0 = base + (lane & (SWEEP2_LINES - 1));
-  const bool valid = l0 < nl;
-  const int line = valid ? l0 : nl - 1;
-  SqSum<R> ss;
-  int bad = 0;
-  int a = (int)(line / S.nb[kind]) + S.a0[kind];
-  int b = (int)(line % S.nb[kind]) + S.b0[kind];
-  if (kind == 0) block_line2<R, D, ROWS>(S, line, valid, a, b, side, ss, &bad);
-  else if (kind == 1) scalar_line2<R, D, 1, ROWS>(S, line, valid, a, b, side, ss, &bad);
-  else scalar_line2<R, D, 2, ROWS>(S, line, valid, a, b, side, ss, &bad);
-  if (bad) atomicOr(S.flag, bad);
-  if (S.update) {
-    for (int f = 0; f < 5; f++) {
-      double v = ss.warp_total(f);
-      if (lane == 0 && v != 0.0) atomicAdd(S.acc + f, v);
     }
   }
 }
