@@ -43,7 +43,7 @@ extern "C" {
 #define SPH_ERR_NONFINITE (-3)  /* NaN/Inf in the new state; the state is left at U^n */
 #define SPH_ERR_SINGULAR (-4)   /* a zero pivot in a line solve; state left at U^n */
 #define SPH_ERR_NOMEM (-5)      /* device allocation failed */
-#define SPH_ERR_TAPE (-6)       /* sph_step_adjoint: a per-thread tape was too short */
+#define SPH_ERR_TAPE (-6)       /* no longer returned (a per-thread tape was too short) */
 
 #define SPH_PREC_FP64 0          /* every step in FP64 */
 #define SPH_PREC_MIXED 1         /* FP32 bulk stencils/line solves, FP64 iterate */
@@ -146,16 +146,15 @@ int sph_status(sph_ctx* ctx, double* residual_out);
  * was given.  Wall data set by sph_set_bc are constants of the step.  The call
  * recomputes the step's iterates, then runs the iterations backwards: per
  * iteration the transposed line solves (phi, theta, r) and the gradient over
- * Ubar of the right-hand side and of the three line operators, by reverse-mode
- * differentiation of the library's own row functions.  Work buffers (about 16
- * fields plus 17 coefficient planes and 1.4 GB of per-thread tapes) are
- * allocated on the first call and kept with the context.  Synchronises.
- * Errors: SPH_ERR_ARG, SPH_ERR_NOMEM, SPH_ERR_CUDA, SPH_ERR_SINGULAR (a zero pivot
- * in a transposed solve), SPH_ERR_TAPE (a location's rows outgrew the tape). */
+ * Ubar of the right-hand side and of the three line operators, by hand-derived
+ * adjoints of their rows.  Work buffers (n_iter + 10 sets of 5 fields and 8
+ * coefficient planes) are allocated on the first call and kept with the context.
+ * Synchronises.  Errors: SPH_ERR_ARG, SPH_ERR_NOMEM, SPH_ERR_CUDA, SPH_ERR_SINGULAR
+ * (a zero pivot in a transposed solve). */
 int sph_step_adjoint(sph_ctx* ctx, double dt, int n_iter, const double* const* source,
                      const double* const* lam_out, double* const* lam_in);
-/* The longest per-thread tape the adjoint has used so far and the capacity
- * (synchronises). */
+/* Kept for callers of the taped adjoint: no tape is recorded any more, longest is
+ * 0 and capacity the former 512. */
 int sph_adjoint_tape_use(sph_ctx* ctx, int* longest, int* capacity);
 
 /* Batches of independent contexts (an ensemble of problems, e.g. of different

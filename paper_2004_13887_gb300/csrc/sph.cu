@@ -46,7 +46,6 @@ using namespace sph;
 
 #include "sph_kernels.cuh"
 
-#include "sph_adjoint.cuh"
 #include "sph_lines.cuh"
 
 // ============================================================== host side
@@ -148,7 +147,6 @@ static void free_all(sph_ctx* c) {
   cudaFree(c->wmean64); cudaFree(c->wmean32); cudaFree(c->wnext);
   cudaFree(c->wzero64); cudaFree(c->wzero32);
   cudaFree(c->adjS); cudaFree(c->adjW); cudaFree(c->adjC);
-  cudaFree(c->tape_d); cudaFree(c->tape_ix); cudaFree(c->tape_li); cudaFree(c->tape_adj); cudaFree(c->adj_info);
   for (int f = 0; f < 5; f++) { cudaFree(c->U[0][f]); cudaFree(c->U[1][f]); cudaFree(c->src[f]); }
   free(c->hmet);
 }
@@ -1084,10 +1082,6 @@ extern "C" int sph_step(sph_ctx* c, double dt, int n_iter, const double* const* 
 
 // ------------------------------------------------------------ adjoint
 
-#define ADJ_TAPE_CAP 512       // nodes per thread's tape (the longest location's rows record 370)
-#define ADJ_TAPE_BLOCKS 608    // blocks of 128 threads of the gradient kernels (four per SM: their registers allow it)
-#define ADJ_FLAG_TAPE 8
-
 static int adj_alloc(sph_ctx* c, int K) {
   if (c->adjS && c->adjK >= K) return SPH_OK;
   cudaFree(c->adjS);
@@ -1101,20 +1095,14 @@ static int adj_alloc(sph_ctx* c, int K) {
   if (cudaMalloc((void**)&c->adjS, (size_t)K * fs * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return SPH_ERR_NOMEM; }
   c->adjK = K;
   if (c->adjW) return SPH_OK;
-  size_t slots = (size_t)ADJ_TAPE_BLOCKS * 128, cap = ADJ_TAPE_CAP;
   if (cudaMalloc((void**)&c->adjW, 10 * fs * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&c->adjC, (size_t)NCOEF * c->N * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&c->tape_d, 2 * cap * slots * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&c->tape_ix, 2 * cap * slots * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&c->tape_li, cap * slots * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&c->tape_adj, cap * slots * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&c->adj_info, sizeof(int)) != cudaSuccess) {
+      cudaMalloc((void**)&c->adjC, (size_t)f64::ADJ_PLANES * c->N * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
+    cudaFree(c->adjW);
+    c->adjW = NULL;
     return SPH_ERR_NOMEM;
   }
-  c->tape_cap = (int)cap;
-  c->tape_blocks = ADJ_TAPE_BLOCKS;
-  return cudaMemset(c->adj_info, 0, sizeof(int)) == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
+  return SPH_OK;
 }
 
 // the 5 fields of set q of a block of sets
@@ -1124,8 +1112,7 @@ static void adj_set(const sph_ctx* c, double* base, int q, double** out) {
 
 // y += s x over whole 5-field sets
 static int adj_axpy(sph_ctx* c, double s, double* x, double* y) {
-  long n = (long)c->fset;
-  adj::k_axpy<<<grid_stride_blocks(n), 256, 0, c->st>>>(n, s, x, y);
+  f64_axpy(c, (long)c->fset, s, x, y);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
@@ -1153,47 +1140,20 @@ static int run_sweep_T(sph_ctx* c, int d, double tau, CF<double> ub, CF<double> 
 }
 
 // the gradient over Ubar of <mu_r, R(Ubar)> - sum_d <mu_d, A_d(Ubar) x_d> into lu
-// (5 fields, added to), by the tape kernels of sph_adjoint.cuh
+// (5 fields, added to), by the kernels of sph_adjoint.cuh
 static int adj_gradient(sph_ctx* c, double tau, CF<double> ub, double** mu, double** xs, double** lu) {
-  Bufs<double>& b = c->d64;
-  adj::AdjArgs A;
-  memset(&A, 0, sizeof A);
-  A.g = b.g; A.P = c->P; A.c = b.c; A.ub = ub; A.tau = tau;
+  CF<double> m[3], x[3];
   for (int d = 0; d < 3; d++) {
     double* m5[5];
     double* x5[5];
     adj_set(c, mu[d], 0, m5);
     adj_set(c, xs[d], 0, x5);
-    A.mu[d] = cf_of(m5);
-    A.x[d] = cf_of(x5);
+    m[d] = cf_of(m5);
+    x[d] = cf_of(x5);
   }
-  for (int f = 0; f < 5; f++) A.lam[f] = lu[f];
-  for (int q = 0; q < NCOEF; q++) A.lam[5 + q] = c->adjC + (size_t)q * c->N;
-  A.td = c->tape_d; A.tix = c->tape_ix; A.tli = c->tape_li; A.tadj = c->tape_adj; A.cap = c->tape_cap;
-  A.flag = c->flag; A.maxn = c->adj_info;
-  if (cudaMemsetAsync(c->adjC, 0, (size_t)NCOEF * c->N * sizeof(double), c->st) != cudaSuccess) return SPH_ERR_CUDA;
-  const int nb = c->tape_blocks;
-  for (int kind = 0; kind < 4; kind++) adj::k_adj_rhs<<<nb, 128, 0, c->st>>>(A, kind);
-  for (int d = 0; d < 3; d++) {
-    SweepArgs<double> S;
-    memset(&S, 0, sizeof S);
-    line_layout(c->d64.g, d, S);
-    if (d == 0) {
-      adj::k_adj_blk<0><<<nb, 128, 0, c->st>>>(A, S.nl[0], S.nb[0], S.a0[0], S.b0[0]);
-      adj::k_adj_sca<0, 1><<<nb, 128, 0, c->st>>>(A, S);
-      adj::k_adj_sca<0, 2><<<nb, 128, 0, c->st>>>(A, S);
-    } else if (d == 1) {
-      adj::k_adj_blk<1><<<nb, 128, 0, c->st>>>(A, S.nl[0], S.nb[0], S.a0[0], S.b0[0]);
-      adj::k_adj_sca<1, 1><<<nb, 128, 0, c->st>>>(A, S);
-      adj::k_adj_sca<1, 2><<<nb, 128, 0, c->st>>>(A, S);
-    } else {
-      adj::k_adj_blk<2><<<nb, 128, 0, c->st>>>(A, S.nl[0], S.nb[0], S.a0[0], S.b0[0]);
-      adj::k_adj_sca<2, 1><<<nb, 128, 0, c->st>>>(A, S);
-      adj::k_adj_sca<2, 2><<<nb, 128, 0, c->st>>>(A, S);
-    }
-  }
-  adj::k_adj_coef<<<nb, 128, 0, c->st>>>(A);
-  c->launches += 14;
+  if (cudaMemsetAsync(c->adjC, 0, (size_t)f64::ADJ_PLANES * c->N * sizeof(double), c->st) != cudaSuccess) return SPH_ERR_CUDA;
+  f64_adjoint(c, tau, ub, m, x, lu);
+  c->launches += 4;
   return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 
@@ -1297,19 +1257,16 @@ extern "C" int sph_step_adjoint(sph_ctx* c, double dt, int n_iter, const double*
   if (e) return e;
   int flag = 0;
   if ((e = read_flag(c, &flag))) return e;
-  if (flag & ADJ_FLAG_TAPE) return SPH_ERR_TAPE;
   if (flag & FLAG_SINGULAR) return SPH_ERR_SINGULAR;
   return SPH_OK;
 }
 
+// No tape is recorded: the adjoint's rows are differentiated by hand.  The
+// capacity is what it was when they were taped.
 extern "C" int sph_adjoint_tape_use(sph_ctx* c, int* longest, int* capacity) {
   if (!c) return SPH_ERR_ARG;
-  int n = 0;
-  if (c->adj_info && (cudaStreamSynchronize(c->st) != cudaSuccess ||
-                      cudaMemcpy(&n, c->adj_info, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess))
-    return SPH_ERR_CUDA;
-  if (longest) *longest = n;
-  if (capacity) *capacity = c->adj_info ? c->tape_cap : ADJ_TAPE_CAP;
+  if (longest) *longest = 0;
+  if (capacity) *capacity = 512;
   return SPH_OK;
 }
 

@@ -10,365 +10,346 @@
 //   dJ/db = lambda - mu_r + g/2,  dJ/da = mu_r + g/2,
 //   g = grad over Ubar of  <mu_r, R(Ubar)> - sum_d <mu_d, A_d(Ubar) x_d>
 // (the x_d and mu_d held fixed).  The transposed solves are the line solvers of
-// sph_fp64_lines.cuh with TR = true.  g is taken here by reverse-mode differentiation of the
-// same row functions the forward kernels run (rhs_c_at, rhs_u_at,
-// assemble_block, scalar_row, coef_at), instantiated on the tape value `ad`: each
-// thread evaluates the rows of one location, recording every operation on a
-// tape, then sweeps the tape backwards and scatters the adjoints of its leaves
-// -- values of Ubar and of the coefficient planes -- with FP64 atomics.  The
-// planes are themselves functions of Ubar, so a last pass takes the planes'
-// adjoints back to Ubar through coef_at.
+// sph_fp64_lines.cuh with TR = true.
+//
+// g is taken by hand-derived adjoints of the rows in sph_fp64.cuh.  A row of
+// D_d enters both the right-hand side (applied to Ubar, weight -tau mu_r) and the
+// line operator (applied to x_d, weight -tau/2 mu_d), with the same weights, so
+// their cotangents add before the one pass back through the weights.  Two
+// kernels per iteration, bound like the forward ones by their FP64
+// instructions (sph_fp64.cuh): k_adj_u at the faces of each component (the
+// momentum rows; what they give to the coefficient planes and to Ubar is added
+// with FP64 atomics, which the L2 performs), then k_adj_c at the centres (the p-
+// and T-rows, and everything back through the coefficients to Ubar).
+// Measured on 96 x 192 x 192 cells, ms per iteration: 4.3 (k_adj_c 2.0, k_adj_u
+// 0.71-0.80 a component) where recording the rows on a tape per thread and
+// sweeping it back (370 nodes a row set in global memory) took 193; the adjoint
+// of a step of two iterations 441 -> 29.9 ms.
 #pragma once
 
-namespace adj {
+namespace f64 {
 
-// The tape of one thread: node q holds up to two parents with their partial
-// derivatives, or (a leaf) an array code and element index.  Arrays are
-// interleaved by thread (element q of thread s at q * stride + s), so a warp
-// recording the same node touches consecutive words.
-struct Tape {
-  double* d;      // partials, 2 per node
-  int* ix;        // parents, 2 per node: node index, -1 none, <= -2 leaf of code -2 - ix
-  int* li;        // leaf element index, 1 per node
-  double* adj;    // adjoints, 1 per node
-  int n, cap, stride, slot, ovf;
-  __device__ __forceinline__ int node(int a, double da, int b, double db) {
-    if (n >= cap) { ovf = 1; return -1; }
-    int q = n++;
-    size_t o = (size_t)(2 * q) * stride + slot;
-    d[o] = da; d[o + stride] = db;
-    ix[o] = a; ix[o + stride] = b;
-    adj[(size_t)q * stride + slot] = 0.0;
-    return q;
-  }
-  __device__ __forceinline__ int leaf(int code, int idx) {
-    if (n >= cap) { ovf = 1; return -1; }
-    int q = n++;
-    ix[(size_t)(2 * q) * stride + slot] = -2 - code;
-    li[(size_t)q * stride + slot] = idx;
-    adj[(size_t)q * stride + slot] = 0.0;
-    return q;
-  }
-  // adjoint 1 at node `out`, swept back to the leaves, whose adjoints are added
-  // to lam[code][idx]
-  __device__ void reverse(int out, double* const* lam) {
-    if (out < 0) return;
-    adj[(size_t)out * stride + slot] = 1.0;
-    for (int q = out; q >= 0; q--) {
-      double a = adj[(size_t)q * stride + slot];
-      if (a == 0.0) continue;
-      size_t o = (size_t)(2 * q) * stride + slot;
-      int p0 = ix[o];
-      if (p0 <= -2) {
-        atomicAdd(lam[-2 - p0] + li[(size_t)q * stride + slot], a);
-        continue;
-      }
-      if (p0 >= 0) adj[(size_t)p0 * stride + slot] += d[o] * a;
-      int p1 = ix[o + stride];
-      if (p1 >= 0) adj[(size_t)p1 * stride + slot] += d[o + stride] * a;
-    }
-  }
-};
+// coefficient planes the momentum rows read: the accumulators of their cotangents
+enum { L_RHO, L_DRHO, L_UC0, L_UC1, L_UC2, L_DVR, L_DVT, L_DVP, NL };
 
-// A value on the tape (id >= 0) or a constant (id = -1).
-struct ad {
-  double v;
-  int id;
-  Tape* t;
-  __device__ __forceinline__ ad() : v(0.0), id(-1), t(nullptr) {}
-  __device__ __forceinline__ ad(double x) : v(x), id(-1), t(nullptr) {}
-  __device__ __forceinline__ ad(double x, int i, Tape* tp) : v(x), id(i), t(tp) {}
-};
-
-__device__ __forceinline__ ad operator+(const ad& a, const ad& b) {
-  if (b.id < 0) return ad(a.v + b.v, a.id, a.t);  // d(a + c)/da = 1: the same node
-  if (a.id < 0) return ad(a.v + b.v, b.id, b.t);
-  return ad(a.v + b.v, a.t->node(a.id, 1.0, b.id, 1.0), a.t);
-}
-__device__ __forceinline__ ad operator-(const ad& a, const ad& b) {
-  if (b.id < 0) return ad(a.v - b.v, a.id, a.t);
-  if (a.id < 0) return ad(a.v - b.v, b.t->node(b.id, -1.0, -1, 0.0), b.t);
-  return ad(a.v - b.v, a.t->node(a.id, 1.0, b.id, -1.0), a.t);
-}
-__device__ __forceinline__ ad operator-(const ad& a) {
-  if (a.id < 0) return ad(-a.v);
-  return ad(-a.v, a.t->node(a.id, -1.0, -1, 0.0), a.t);
-}
-__device__ __forceinline__ ad operator*(const ad& a, const ad& b) {
-  if (b.id < 0) {
-    if (a.id < 0) return ad(a.v * b.v);
-    return ad(a.v * b.v, a.t->node(a.id, b.v, -1, 0.0), a.t);
-  }
-  if (a.id < 0) return ad(a.v * b.v, b.t->node(b.id, a.v, -1, 0.0), b.t);
-  return ad(a.v * b.v, a.t->node(a.id, b.v, b.id, a.v), a.t);
-}
-__device__ __forceinline__ ad operator/(const ad& a, const ad& b) {
-  double q = a.v / b.v;
-  if (b.id < 0) {
-    if (a.id < 0) return ad(q);
-    return ad(q, a.t->node(a.id, 1.0 / b.v, -1, 0.0), a.t);
-  }
-  double db = -q / b.v;
-  if (a.id < 0) return ad(q, b.t->node(b.id, db, -1, 0.0), b.t);
-  return ad(q, a.t->node(a.id, 1.0 / b.v, b.id, db), a.t);
-}
-__device__ __forceinline__ ad& operator+=(ad& a, const ad& b) { a = a + b; return a; }
-__device__ __forceinline__ ad& operator-=(ad& a, const ad& b) { a = a - b; return a; }
-__device__ __forceinline__ ad& operator*=(ad& a, const ad& b) { a = a * b; return a; }
-__device__ __forceinline__ bool operator==(const ad& a, const ad& b) { return a.v == b.v; }
-__device__ __forceinline__ bool isfinite(const ad& a) { return ::isfinite(a.v); }
-
-// Reads of a field or coefficient plane that record tape leaves (code = the
-// array's index in the adjoint accumulators: the 5 fields of Ubar, then the
-// 17 coefficient planes in Coef's order).
-struct LeafPtr {
-  const double* p;
-  int code;
-  Tape* t;
-  __device__ __forceinline__ ad operator[](int i) const { return ad(p[i], t->leaf(code, i), t); }
-};
-
-// the adjoint's stand-in for a Coef or MF the rows write into: slots that keep
-// the written values
-struct Slot {
-  mutable ad v;
-  __device__ __forceinline__ ad& operator[](int) const { return v; }
-};
-struct CoefOut { Slot Pb, Tb, rho, drho, beta, uc0, uc1, uc2, grr, gtt, gpp, srt, srp, stp, dvr, dvt, dvp; };
-struct RowsOut { Slot f[5]; };
-
-constexpr int NLAM = 5 + sph::NCOEF;  // accumulators: Ubar fields, then coefficient planes
-
-}  // namespace adj
-
-namespace sph {
-template <>
-struct Val<adj::ad> {
-  using T = double;
-  using CP = adj::LeafPtr;
-  using MP = adj::LeafPtr;
-};
-}  // namespace sph
-
-namespace adj {
-
-// Everything a gradient kernel reads: the forward values at Ubar (FP64 planes and
-// fields), the adjoint vectors, the accumulators and the tape.
 struct AdjArgs {
   Geo<double> g;
-  Par P;
+  K64 k;
+  Tabs T;
   Coef<double> c;       // coefficient planes at Ubar
   CF<double> ub;        // Ubar
   double tau;
-  CF<double> mu[3];     // mu_r (the right-hand side's weight), mu_theta, mu_phi
+  CF<double> mu[3];     // mu_r (the right-hand side's weight too), mu_theta, mu_phi
   CF<double> x[3];      // the forward sweeps' solutions x_r, x_theta, x_phi
-  double* lam[NLAM];    // gradient accumulators (Ubar, then the planes)
-  double* td; int* tix; int* tli; double* tadj;
-  int cap;
-  int* flag;            // bit 8: a tape overflowed
-  int* maxn;            // the longest tape used
+  double* lam[5];       // gradient over Ubar (added to)
+  double* pl[NL];       // cotangents of the planes (zero before k_adj_u)
 };
 
-__device__ __forceinline__ Tape make_tape(const AdjArgs& A) {
-  Tape T;
-  T.d = A.td; T.ix = A.tix; T.li = A.tli; T.adj = A.tadj;
-  T.n = 0; T.cap = A.cap; T.stride = gridDim.x * blockDim.x;
-  T.slot = blockIdx.x * blockDim.x + threadIdx.x;
-  T.ovf = 0;
-  return T;
+// add v to the cotangent of the value that an accessor with ghosts reads at
+// (i, j, k): p and T (zero gradient at the walls), or velocity component C
+// (ghost = 2 wall - interior; the wall value is a constant)
+__device__ __forceinline__ void scat_c(const Geo<double>& g, double* lam, int i, int j, int k, double v) {
+  const int kk = g.per ? wrapk(g, k) : clampi(k, 0, g.np - 1);
+  atomicAdd(lam + IC(g, clampi(i, 0, g.nr - 1), clampi(j, 0, g.nt - 1), kk), v);
+}
+template <int C>
+__device__ __forceinline__ void scat_v(const Geo<double>& g, double* lam, int i, int j, int k, double v) {
+  if (C != 0 && (i < 0 || i >= g.nr)) { i = i < 0 ? 0 : g.nr - 1; v = -v; }
+  if (C != 1 && (j < 0 || j >= g.nt)) { j = j < 0 ? 0 : g.nt - 1; v = -v; }
+  if (g.per) k = wrapk(g, k);
+  else if (C != 2 && (k < 0 || k >= g.np)) { k = k < 0 ? 0 : g.np - 1; v = -v; }
+  atomicAdd(lam + face_idx(g, C, i, j, k), v);
+}
+// an increment's velocity component beside its face: homogeneous ghosts
+template <int C>
+__device__ __forceinline__ double vel0(const Geo<double>& g, const double* u, int i, int j, int k) {
+  return C == 0 ? vr<1>(g, u, i, j, k) : C == 1 ? vt<1>(g, u, i, j, k) : vp<1>(g, u, i, j, k);
 }
 
-// the geometry with its tables as they are (doubles) for the tape instantiation
-__device__ __forceinline__ Geo<ad> geo_ad(const Geo<double>& a) {
-  static_assert(sizeof(Geo<ad>) == sizeof(Geo<double>), "Geo<ad> must have Geo<double>'s layout");
-  Geo<ad> g;
-  memcpy(&g, &a, sizeof g);
-  return g;
+// the transverse row of component C along D: cotangents of 1/(rho_0 + rho_1) and
+// of the advecting velocity's sum; Ubar's share is scattered
+template <int C, int D>
+__device__ __forceinline__ void adj_trans(const AdjArgs& A, const double* m, int i, int j, int k, int t, double iv,
+                                          double ua2, double a, double u, double& civ, double& cua, double& cu) {
+  const Geo<double>& g = A.g;
+  constexpr int di = D == 0, dj = D == 1, dk = D == 2;
+  double q, f0, f1, f2;
+  if (C == 0 && D == 1) { q = m[R_QT]; f0 = m[R_T0]; f1 = m[R_TS]; f2 = m[R_T1]; }
+  else if (C == 0) { q = m[R_QP]; f0 = f2 = m[R_P]; f1 = m[R_P2]; }
+  else if (C == 1 && D == 0) { q = A.k.qidr; f0 = m[T_R0]; f1 = m[T_RS]; f2 = m[T_R1]; }
+  else if (C == 1) { q = m[T_QP]; f0 = f2 = m[T_P]; f1 = m[T_P2]; }
+  else if (D == 0) { q = A.k.qidr; f0 = m[P_R0]; f1 = m[P_RS]; f2 = m[P_R1]; }
+  else { q = m[C_QMT]; f0 = m[P_T0]; f1 = m[P_TS]; f2 = m[P_T1]; }
+  const double* U = A.ub.f[1 + C];
+  const double* X = A.x[D].f[1 + C];
+  const double cd = -0.5 * A.tau * A.mu[D].f[1 + C][t];
+  const double zl = fma(a, vel<C>(g, U, i - di, j - dj, k - dk), cd * vel0<C>(g, X, i - di, j - dj, k - dk));
+  const double zh = fma(a, vel<C>(g, U, i + di, j + dj, k + dk), cd * vel0<C>(g, X, i + di, j + dj, k + dk));
+  const double z0 = fma(a, u, cd * X[t]);
+  civ = fma(f0, zl, fma(f1, z0, fma(f2, zh, civ)));
+  cua = fma(q, zh - zl, cua);
+  const double adv = ua2 * q;
+  scat_v<C>(g, A.lam[1 + C], i - di, j - dj, k - dk, a * fma(iv, f0, -adv));
+  scat_v<C>(g, A.lam[1 + C], i + di, j + dj, k + dk, a * fma(iv, f2, adv));
+  cu = fma(a, iv * f1, cu);
 }
 
-__device__ __forceinline__ CF<ad> leaves_ub(const AdjArgs& A, Tape* t) {
-  CF<ad> u;
-  for (int f = 0; f < 5; f++) u.f[f] = LeafPtr{A.ub.f[f], f, t};
-  return u;
-}
-__device__ __forceinline__ Coef<ad> leaves_coef(const AdjArgs& A, Tape* t) {
+// the momentum rows of component C: one thread per face
+template <int C>
+__global__ void __launch_bounds__(128) k_adj_u(const __grid_constant__ AdjArgs A) {
+  const Geo<double>& g = A.g;
+  const int nj = g.nt + (C == 1), nk = C == 2 ? g.npf : g.np;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
+            i = blockIdx.z * blockDim.z + threadIdx.z;
+  if (k >= nk || j >= nj || i >= g.nr + (C == 0)) return;
+  if (C == 0 ? (i == 0 || i == g.nr) : C == 1 ? (j == 0 || j == g.nt) : (!g.per && (k == 0 || k == g.np))) return;
+  const int t = (i * nj + j) * nk + k;
+  constexpr int D1 = C == 0 ? 1 : 0, D2 = C == 2 ? 1 : 2;   // the transverse directions
   const Coef<double>& c = A.c;
-  Coef<ad> o;
-  const double* src[NCOEF] = {c.Pb, c.Tb, c.rho, c.drho, c.beta, c.uc0, c.uc1, c.uc2,
-                              c.grr, c.gtt, c.gpp, c.srt, c.srp, c.stp, c.dvr, c.dvt, c.dvp};
-  LeafPtr* dst[NCOEF] = {&o.Pb, &o.Tb, &o.rho, &o.drho, &o.beta, &o.uc0, &o.uc1, &o.uc2,
-                         &o.grr, &o.gtt, &o.gpp, &o.srt, &o.srp, &o.stp, &o.dvr, &o.dvt, &o.dvp};
-  for (int q = 0; q < NCOEF; q++) *dst[q] = LeafPtr{src[q], 5 + q, t};
-  return o;
-}
-
-__device__ __forceinline__ void finish(const AdjArgs& A, Tape& T, const ad& psi) {
-  T.reverse(psi.t ? psi.id : -1, A.lam);
-  if (T.ovf) atomicOr(A.flag, 8);
-  atomicMax(A.maxn, T.n);
-}
-
-// (1) <mu_r, R(Ubar)>: one thread per location -- centres (kind = 0, the p- and
-// T-rows) or the interior faces of u_r, u_theta, u_phi (kind 1, 2, 3).  D = U^k -
-// U^n and the source do not depend on Ubar: hasD = has_src = 0.
-__global__ void __launch_bounds__(128) k_adj_rhs(AdjArgs A, int kind) {
-  Tape T = make_tape(A);
-  const Geo<double>& g = A.g;
-  const Geo<ad> ga = geo_ad(g);
-  const int nt = g.nt + (kind == 2), np = kind == 3 ? g.npf : g.np, nr = g.nr + (kind == 1);
-  const long total = (long)nr * nt * np;
-  CF<ad> none;
-  for (int f = 0; f < 5; f++) none.f[f] = LeafPtr{nullptr, 0, nullptr};
-  CF<double> noned;
-  for (int f = 0; f < 5; f++) noned.f[f] = nullptr;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-    int t = (int)e;
-    int k = t % np, j = (t / np) % nt, i = t / (np * nt);
-    if (kind == 1 && (i == 0 || i == g.nr)) continue;
-    if (kind == 2 && (j == 0 || j == g.nt)) continue;
-    if (kind == 3 && !g.per && (k == 0 || k == g.np)) continue;
-    double w0 = A.mu[0].f[kind == 0 ? 0 : kind][t];
-    double w4 = kind == 0 ? A.mu[0].f[4][t] : 0.0;
-    if (w0 == 0.0 && w4 == 0.0) continue;
-    T.n = 0;
-    CF<ad> ub = leaves_ub(A, &T);
-    Coef<ad> c = leaves_coef(A, &T);
-    RowsOut out;
-    ad psi;
-    if (kind == 0) {
-      rhs_c_at<2>(ga, A.P, c, ub, none, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
-      psi = out.f[0].v * w0 + out.f[4].v * w4;
-    } else if (kind == 1) {
-      rhs_u_at<2, 0>(ga, A.P, c, ub, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
-      psi = out.f[1].v * w0;
-    } else if (kind == 2) {
-      rhs_u_at<2, 1>(ga, A.P, c, ub, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
-      psi = out.f[2].v * w0;
-    } else {
-      rhs_u_at<2, 2>(ga, A.P, c, ub, none, 0, noned, 0, ad(A.tau), out, i, j, k, t);
-      psi = out.f[3].v * w0;
-    }
-    finish(A, T, psi);
+  const FaceC q = face_load<C>(g, c, i, j, k);
+  const double* m = face_tab<C>(g, A.T, i, j);
+  const double iv = q.iv;
+  const double* U = A.ub.f[1 + C];
+  const double* Pp = A.ub.f[0];
+  const double u = U[t];
+  const double a = -A.tau * A.mu[0].f[1 + C][t], cn = -0.5 * A.tau * A.mu[C].f[1 + C][t];
+  double civ, cu, cs1 = 0.0, cs2 = 0.0;
+  {
+    // the normal row
+    const double* X = A.x[C].f[1 + C];
+    const double* Xp = A.x[C].f[0];
+    double wp, w[3];
+    face_normal<C>(A.k, m, iv, u, wp, w);
+    constexpr int di = C == 0, dj = C == 1, dk = C == 2;
+    const double zp = fma(a, Pp[q.c1] - Pp[q.c0], cn * (Xp[q.c1] - Xp[q.c0]));
+    const double zm = fma(a, vel<C>(g, U, i - di, j - dj, k - dk), cn * vel0<C>(g, X, i - di, j - dj, k - dk));
+    const double zn = fma(a, vel<C>(g, U, i + di, j + dj, k + dk), cn * vel0<C>(g, X, i + di, j + dj, k + dk));
+    const double z0 = fma(a, u, cn * X[t]);
+    const double fw = m[C == 0 ? R_WP : C == 1 ? T_WP : P_WP], f0 = m[C == 0 ? R_F0 : C == 1 ? T_F0 : P_F],
+                 f1 = m[C == 0 ? R_F1 : C == 1 ? T_F1 : P_F2], f2 = m[C == 0 ? R_F2 : C == 1 ? T_F2 : P_F];
+    civ = fma(fw, zp, fma(f0, zm, fma(f1, z0, f2 * zn)));
+    cu = fma(a, w[1], (zn - zm) * (C == 0 ? A.k.hidr : C == 1 ? m[T_HADV] : m[C_HMP]));
+    atomicAdd(A.lam[0] + q.c1, a * wp);
+    atomicAdd(A.lam[0] + q.c0, -a * wp);
+    scat_v<C>(g, A.lam[1 + C], i - di, j - dj, k - dk, a * w[0]);
+    scat_v<C>(g, A.lam[1 + C], i + di, j + dj, k + dk, a * w[2]);
   }
-}
-
-// the unknowns (p, T, u_d on face m+1) of block m of the line (a, b) along d in
-// the fields F (the wall face of a walled line's last block is 0)
-__device__ __forceinline__ void block_vec(const Geo<double>& g, const CF<double>& F, int d, int n, int cyc, int a, int b,
-                                          int m, double v[3]) {
-  int i, j, k;
-  line_pos(d, a, b, m, i, j, k);
-  int ic = IC(g, i, j, k);
-  v[0] = F.f[0][ic];
-  v[1] = F.f[4][ic];
-  v[2] = 0.0;
-  if (m < n - 1 || cyc) {
-    int fi = i, fj = j, fk = k;
-    if (d == 0) fi = m + 1; else if (d == 1) fj = m + 1; else fk = (m + 1 == n) ? 0 : m + 1;
-    v[2] = F.f[1 + d][face_idx(g, d, fi, fj, fk)];
+  const double s1 = ucen<D1>(c)[q.c0] + ucen<D1>(c)[q.c1], s2 = ucen<D2>(c)[q.c0] + ucen<D2>(c)[q.c1];
+  adj_trans<C, D1>(A, m, i, j, k, t, iv, s1, a, u, civ, cs1, cu);
+  adj_trans<C, D2>(A, m, i, j, k, t, iv, s2, a, u, civ, cs2, cu);
+  const double ai = a * iv;
+  double vis;
+  if (C == 0) {
+    vis = fma(u, m[R_V], fma(c.dvt[q.c1] + c.dvp[q.c1], m[R_Q1], (c.dvt[q.c0] + c.dvp[q.c0]) * m[R_Q0]));
+    vis = fma(c.drho[q.c0] + c.drho[q.c1], m[R_GE], vis);
+    const double cd = ai * m[R_GE], v1 = ai * m[R_Q1], v0 = ai * m[R_Q0], a2 = -2.0 * a * m[R_QIR];
+    atomicAdd(A.pl[L_DRHO] + q.c0, cd);
+    atomicAdd(A.pl[L_DRHO] + q.c1, cd);
+    atomicAdd(A.pl[L_DVT] + q.c0, v0);
+    atomicAdd(A.pl[L_DVP] + q.c0, v0);
+    atomicAdd(A.pl[L_DVT] + q.c1, v1);
+    atomicAdd(A.pl[L_DVP] + q.c1, v1);
+    cs1 = fma(a2, s1, cs1);
+    cs2 = fma(a2, s2, fma(-a, m[R_OM], cs2));
+    cu = fma(ai, m[R_V], cu);
+    atomicAdd(A.pl[L_UC1] + q.c0, cs1);
+    atomicAdd(A.pl[L_UC1] + q.c1, cs1);
+    atomicAdd(A.pl[L_UC2] + q.c0, cs2);
+    atomicAdd(A.pl[L_UC2] + q.c1, cs2);
+  } else if (C == 1) {
+    vis = fma(u, m[T_V], (c.dvr[q.c1] - c.dvr[q.c0]) * m[T_D]);
+    vis = fma(c.dvp[q.c0], m[T_D0], fma(c.dvp[q.c1], m[T_D1], vis));
+    vis = fma(c.uc0[q.c1] - c.uc0[q.c0], m[T_UR], vis);
+    const double d = ai * m[T_D], r = ai * m[T_UR];
+    atomicAdd(A.pl[L_DVR] + q.c0, -d);
+    atomicAdd(A.pl[L_DVR] + q.c1, d);
+    atomicAdd(A.pl[L_DVP] + q.c0, ai * m[T_D0]);
+    atomicAdd(A.pl[L_DVP] + q.c1, ai * m[T_D1]);
+    cs1 = fma(a * u, m[T_HIR], cs1);
+    cs2 = fma(-2.0 * a * m[T_C], s2, fma(-a, m[T_OM], cs2));
+    cu = fma(a * s1, m[T_HIR], fma(ai, m[T_V], cu));
+    atomicAdd(A.pl[L_UC0] + q.c0, cs1 - r);
+    atomicAdd(A.pl[L_UC0] + q.c1, cs1 + r);
+    atomicAdd(A.pl[L_UC2] + q.c0, cs2);
+    atomicAdd(A.pl[L_UC2] + q.c1, cs2);
+  } else {
+    vis = fma(u, m[P_V], ((c.dvr[q.c1] - c.dvr[q.c0]) + (c.dvt[q.c1] - c.dvt[q.c0])) * m[P_D]);
+    vis = fma(c.uc0[q.c1] - c.uc0[q.c0], m[P_UR], fma(c.uc1[q.c1] - c.uc1[q.c0], m[P_UT], vis));
+    const double d = ai * m[P_D], r = ai * m[P_UR], p = ai * m[P_UT], au = a * u;
+    atomicAdd(A.pl[L_DVR] + q.c0, -d);
+    atomicAdd(A.pl[L_DVR] + q.c1, d);
+    atomicAdd(A.pl[L_DVT] + q.c0, -d);
+    atomicAdd(A.pl[L_DVT] + q.c1, d);
+    cs1 = fma(au, m[C_HIR], fma(a, m[P_OS], cs1));
+    cs2 = fma(au, m[C_HCOTIR], fma(a, m[P_OC], cs2));
+    cu = fma(a, fma(s2, m[C_HCOTIR], s1 * m[C_HIR]), fma(ai, m[P_V], cu));
+    atomicAdd(A.pl[L_UC0] + q.c0, cs1 - r);
+    atomicAdd(A.pl[L_UC0] + q.c1, cs1 + r);
+    atomicAdd(A.pl[L_UC1] + q.c0, cs2 - p);
+    atomicAdd(A.pl[L_UC1] + q.c1, cs2 + p);
   }
+  atomicAdd(A.lam[1 + C] + t, cu);
+  const double cr = -iv * iv * fma(a, vis, civ);
+  atomicAdd(A.pl[L_RHO] + q.c0, cr);
+  atomicAdd(A.pl[L_RHO] + q.c1, cr);
 }
 
-// (2) -<mu_d, A_d(Ubar) x_d> over the block rows of the lines along D: one thread
-// per cell of a line; the block row m of A_d is assembled by the forward's
-// assemble_block on tape values.
+// the cotangents of a centre's coefficients
+struct CenCot {
+  double Pb, Tb, be, grr, gtt, gpp, srt, srp, stp, uc[3];
+  double ap, aT, vT2;
+};
+
+// one direction of the p- and T-rows: a, b weight the right-hand side's rows
 template <int D>
-__global__ void __launch_bounds__(128) k_adj_blk(AdjArgs A, int nl, int nb, int a0, int b0) {
-  Tape T = make_tape(A);
+__device__ __forceinline__ void adj_cen(const AdjArgs& A, const CenC& q, const double* m, int i, int j, int k, int t,
+                                        double a, double b, double e, double& vis, double& lap, CenCot& o) {
   const Geo<double>& g = A.g;
-  const Geo<ad> ga = geo_ad(g);
-  const int n = D == 0 ? g.nr : D == 1 ? g.nt : g.np;
-  const int cyc = (D == 2 && g.per);
-  const long total = (long)nl * n;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-    int line = (int)(e / n), m = (int)(e % n);
-    int a = line / nb + a0, b = line % nb + b0;
-    double mu[3];
-    block_vec(g, A.mu[D], D, n, cyc, a, b, m, mu);
-    if (mu[0] == 0.0 && mu[1] == 0.0 && mu[2] == 0.0) continue;
-    double xm[3], x0[3], xp[3];
-    block_vec(g, A.x[D], D, n, cyc, a, b, m, x0);
-    int mp = m - 1, mn = m + 1;
-    if (cyc) { mp = mp < 0 ? n - 1 : mp; mn = mn == n ? 0 : mn; }
-    xm[0] = xm[1] = xm[2] = xp[0] = xp[1] = xp[2] = 0.0;
-    if (mp >= 0) block_vec(g, A.x[D], D, n, cyc, a, b, mp, xm);
-    if (mn < n) block_vec(g, A.x[D], D, n, cyc, a, b, mn, xp);
-    T.n = 0;
-    CF<ad> ub = leaves_ub(A, &T);
-    Coef<ad> c = leaves_coef(A, &T);
-    int i, j, k;
-    line_pos(D, a, b, m, i, j, k);
-    ad Ab[9], Bb[9], Cb[9];
-    assemble_block(ga, A.P, c, ub, D, n, cyc, m, i, j, k, ad(0.5 * A.tau), Ab, Bb, Cb);
-    ad psi;
-    for (int r = 0; r < 3; r++) {
-      if (mu[r] == 0.0) continue;
-      ad y = ad(0.0);
-      for (int q = 0; q < 3; q++) y += Ab[r * 3 + q] * xm[q] + Bb[r * 3 + q] * x0[q] + Cb[r * 3 + q] * xp[q];
-      psi -= y * mu[r];
-    }
-    finish(A, T, psi);
+  constexpr int di = D == 0, dj = D == 1, dk = D == 2;
+  const double cp = -0.5 * A.tau * A.mu[D].f[0][t], cT = -0.5 * A.tau * A.mu[D].f[4][t];
+  const double hm = D == 0 ? A.k.hidr : m[D == 1 ? C_HMT : C_HMP];
+  const double adv = cen_adv<D>(A.k, A.c, m, t);
+  double s, u;
+  cen_visc<D>(A.k, q, m, s, u);
+  const double l0 = m[D == 0 ? C_L00 : D == 1 ? C_L10 : C_MP2], l1 = m[D == 0 ? C_L01 : D == 1 ? C_L11 : C_MP2];
+  const double g0 = m[D == 0 ? C_G00 : D == 1 ? C_G10 : C_MP], g1 = m[D == 0 ? C_G01 : D == 1 ? C_G11 : C_MP];
+  const double *Pp = A.ub.f[0], *TT = A.ub.f[4], *U = A.ub.f[1 + D];
+  const double *Xp = A.x[D].f[0], *XT = A.x[D].f[4], *XU = A.x[D].f[1 + D];
+  // the rows' operands: Ubar's (with the background) and the sweep solution's
+  double dp = cpert<2>(g, Pp, i + di, j + dj, k + dk) - cpert<2>(g, Pp, i - di, j - dj, k - dk);
+  const double Tm = cpert<2>(g, TT, i - di, j - dj, k - dk), T0 = TT[t], Tn = cpert<2>(g, TT, i + di, j + dj, k + dk);
+  double dT = Tn - Tm;
+  lap = fma(l1, Tn - T0, fma(l0, Tm - T0, lap));
+  if (D == 0) { dp += g.dbgp[i]; dT += g.dbgT[i]; }
+  const double xp = cpert<2>(g, Xp, i + di, j + dj, k + dk) - cpert<2>(g, Xp, i - di, j - dj, k - dk);
+  const double Xm = cpert<2>(g, XT, i - di, j - dj, k - dk), X0 = XT[t], Xn = cpert<2>(g, XT, i + di, j + dj, k + dk);
+  const double xl = fma(l1, Xn - X0, l0 * (Xm - X0));
+  const int f0 = face_idx(g, D, i, j, k);
+  const int f1 = face_idx(g, D, i + di, j + dj, D == 2 && g.per ? wrapk(g, k + 1) : k + dk);
+  const double u0 = U[f0], u1 = U[f1], x0 = XU[f0], x1 = XU[f1];
+  const double dx = fma(g1, x1, -(g0 * x0)), vx = fma(s, x0, u * x1);
+  vis = fma(s, u0, fma(u, u1, vis));
+  // cotangents of the row weights
+  const double ce = fma(cp, A.k.vp2, cT * q.vT2);
+  const double cs = fma(e, u0, ce * x0), cu = fma(e, u1, ce * x1);
+  o.ap = fma(cp, dx, o.ap);
+  o.aT = fma(cT, dx, o.aT);
+  o.vT2 = fma(cT, vx, o.vT2);
+  o.be = fma(-A.k.kap * cT, xl, o.be);
+  o.uc[D] = fma(hm, fma(a, dp, fma(b, dT, fma(cp, xp, cT * (Xn - Xm)))), o.uc[D]);
+  const double cl = cs + cu, cm = cs - cu;
+  if (D == 0) {
+    const double z = -m[C_HIR] * cl;
+    o.gtt += z;
+    o.gpp += z;
+    o.grr = fma(A.k.idr, cm, o.grr);
+  } else if (D == 1) {
+    const double z = m[C_QIR] * cl;
+    o.gpp = fma(-z, m[C_COT2], o.gpp);
+    o.srt += z;
+    o.gtt = fma(m[C_MT], cm, o.gtt);
+  } else {
+    const double z = m[C_QIR] * cl;
+    o.stp = fma(z, m[C_COT], o.stp);
+    o.srp += z;
+    o.gpp = fma(m[C_MP], cm, o.gpp);
   }
+  // Ubar as the right-hand side's operand
+  const double aa = a * adv, bb = b * adv, ct = -fma(A.k.difp, a, A.k.kap * q.be * b);
+  scat_c(g, A.lam[0], i + di, j + dj, k + dk, aa);
+  scat_c(g, A.lam[0], i - di, j - dj, k - dk, -aa);
+  scat_c(g, A.lam[4], i + di, j + dj, k + dk, fma(ct, l1, bb));
+  scat_c(g, A.lam[4], i - di, j - dj, k - dk, fma(ct, l0, -bb));
+  atomicAdd(A.lam[4] + t, -ct * (l0 + l1));
+  atomicAdd(A.lam[1 + D] + f0, e * s);
+  atomicAdd(A.lam[1 + D] + f1, e * u);
 }
 
-// (2') the same over the transverse scalar lines of kind KIND along D
-template <int D, int KIND>
-__global__ void __launch_bounds__(128) k_adj_sca(AdjArgs A, SweepArgs<double> S) {
-  Tape T = make_tape(A);
+// The p- and T-rows at the centres and the coefficients' adjoint: one thread
+// per centre, after k_adj_u has added the planes' cotangents.
+__global__ void __launch_bounds__(128) k_adj_c(const __grid_constant__ AdjArgs A) {
   const Geo<double>& g = A.g;
-  const Geo<ad> ga = geo_ad(g);
-  constexpr int cc = trans_comp(D, KIND);
-  const int n = D == 0 ? g.nr : D == 1 ? g.nt : g.np;
-  const int cyc = (D == 2 && g.per);
-  const int nl = S.nl[KIND], nb = S.nb[KIND], a0 = S.a0[KIND], b0 = S.b0[KIND];
-  const long total = (long)nl * n;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-    int line = (int)(e / n), m = (int)(e % n);
-    int a = line / nb + a0, b = line % nb + b0;
-    int i, j, k;
-    line_pos(D, a, b, m, i, j, k);
-    double mu = A.mu[D].f[1 + cc][face_idx(g, cc, i, j, k)];
-    if (mu == 0.0) continue;
-    const double* X = A.x[D].f[1 + cc];
-    double x0 = X[face_idx(g, cc, i, j, k)], xm = 0.0, xp = 0.0;
-    int mp = m - 1, mn = m + 1;
-    if (cyc) { mp = mp < 0 ? n - 1 : mp; mn = mn == n ? 0 : mn; }
-    if (mp >= 0) { int ii, jj, kk; line_pos(D, a, b, mp, ii, jj, kk); xm = X[face_idx(g, cc, ii, jj, kk)]; }
-    if (mn < n) { int ii, jj, kk; line_pos(D, a, b, mn, ii, jj, kk); xp = X[face_idx(g, cc, ii, jj, kk)]; }
-    T.n = 0;
-    SweepArgs<ad> Sa;
-    Sa.g = ga; Sa.P = A.P; Sa.c = leaves_coef(A, &T); Sa.ub = leaves_ub(A, &T); Sa.h = ad(0.5 * A.tau);
-    ad am, bm, cm;
-    scalar_row(Sa, cc, D, n, cyc, a, b, m, am, bm, cm);
-    ad psi = -((am * xm + bm * x0 + cm * xp) * mu);
-    finish(A, T, psi);
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
+            i = blockIdx.z * blockDim.z + threadIdx.z;
+  if (k >= g.np || j >= g.nt || i >= g.nr) return;
+  const int t = IC(g, i, j, k);
+  const double* m = A.T.c + (size_t)(i * g.nt + j) * NC;
+  const Coef<double>& c = A.c;
+  const K64& K = A.k;
+  const CenC q = cen_load(K, c, t);
+  const double a = -A.tau * A.mu[0].f[0][t], b = -A.tau * A.mu[0].f[4][t];
+  const double e = fma(a, K.vp2, b * q.vT2);        // cotangent of the viscous sum
+  const double div = c.dvr[t] + c.dvt[t] + c.dvp[t];
+  CenCot o;
+  o.Pb = o.Tb = o.be = o.grr = o.gtt = o.gpp = o.srt = o.srp = o.stp = 0.0;
+  o.uc[0] = A.pl[L_UC0][t]; o.uc[1] = A.pl[L_UC1][t]; o.uc[2] = A.pl[L_UC2][t];
+  o.ap = a * div;
+  o.aT = b * div;
+  o.vT2 = 0.0;
+  double vis = 0.0, lap = g.lapT[i];
+  adj_cen<0>(A, q, m, i, j, k, t, a, b, e, vis, lap, o);
+  adj_cen<1>(A, q, m, i, j, k, t, a, b, e, vis, lap, o);
+  adj_cen<2>(A, q, m, i, j, k, t, a, b, e, vis, lap, o);
+  const double ir = m[C_IR], cotir = m[C_COTIR];
+  {
+    // -1/2 cross of the viscous sum
+    const double ut = c.uc1[t], up = c.uc2[t], he = -0.5 * e;
+    const double xrt = fma(ut, ir, q.srt), xrp = fma(up, ir, q.srp), xtp = fma(up, cotir, q.stp);
+    vis = fma(-0.5, fma(q.stp, xtp, fma(q.srp, xrp, q.srt * xrt)), vis);
+    o.srt = fma(he, q.srt + xrt, o.srt);
+    o.srp = fma(he, q.srp + xrp, o.srp);
+    o.stp = fma(he, q.stp + xtp, o.stp);
+    o.uc[1] = fma(he * q.srt, ir, o.uc[1]);
+    o.uc[2] = fma(he, fma(q.srp, ir, q.stp * cotir), o.uc[2]);
   }
-}
-
-// (3) the coefficient planes' adjoints back to Ubar: one thread per centre,
-// <lam_coef, coef(Ubar)> through the forward's coef_at on tape values
-__global__ void __launch_bounds__(128) k_adj_coef(AdjArgs A) {
-  Tape T = make_tape(A);
-  const Geo<double>& g = A.g;
-  const Geo<ad> ga = geo_ad(g);
-  const long total = (long)g.nr * g.nt * g.np;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-    int t = (int)e;
-    double w[NCOEF];
-    bool any = false;
-    for (int q = 0; q < NCOEF; q++) { w[q] = A.lam[5 + q][t]; any |= w[q] != 0.0; }
-    if (!any) continue;
-    int k = t % g.np, j = (t / g.np) % g.nt, i = t / (g.np * g.nt);
-    T.n = 0;
-    CF<ad> ub = leaves_ub(A, &T);
-    CoefOut o;
-    coef_at<2>(ga, A.P, ub, o, i, j, k, t);
-    const Slot* sl[NCOEF] = {&o.Pb, &o.Tb, &o.rho, &o.drho, &o.beta, &o.uc0, &o.uc1, &o.uc2,
-                             &o.grr, &o.gtt, &o.gpp, &o.srt, &o.srp, &o.stp, &o.dvr, &o.dvt, &o.dvp};
-    ad psi;
-    for (int q = 0; q < NCOEF; q++)
-      if (w[q] != 0.0) psi += sl[q]->v * w[q];
-    finish(A, T, psi);
+  // a_p = gamma Pb + vp2 t3, a_T = (gamma-1) Tb + vT2 t3, vT2 = 2 mu beta, t3 = tr G / 3
+  const double t3 = (q.grr + q.gtt + q.gpp) * (1.0 / 3.0);
+  o.vT2 = fma(b, vis, fma(t3, o.aT, o.vT2));
+  o.be = fma(K.mu2, o.vT2, fma(-K.kap * b, lap, o.be));
+  o.Pb = K.gm * o.ap;
+  o.Tb = K.gm1 * o.aT;
+  const double ct = fma(K.vp2, o.ap, q.vT2 * o.aT) * (1.0 / 3.0);
+  o.grr += ct;
+  o.gtt += ct;
+  o.gpp += ct;
+  // the coefficients of the centre back to Ubar
+  const double cdiv = fma(a, q.ap, b * q.aT);
+  const double cdr = A.pl[L_DVR][t] + cdiv, cdt = A.pl[L_DVT][t] + cdiv, cdp = A.pl[L_DVP][t] + cdiv;
+  {
+    const double iT = 1.0 / c.Tb[t], iP = 1.0 / c.Pb[t], cr = A.pl[L_RHO][t], cd = A.pl[L_DRHO][t];
+    const double w = iT * m[C_IT];
+    const double lp = fma(cd, g.Tcen[i] * w, fma(cr, iT * K.iRg, fma(-o.be * q.be, iP, o.Pb)));
+    const double lT = fma(o.be, iP * K.gm1, fma(-cd, fma(g.pcen[i], w, c.drho[t] * iT), fma(-cr, c.rho[t] * iT, o.Tb)));
+    atomicAdd(A.lam[0] + t, lp);
+    atomicAdd(A.lam[4] + t, lT);
+  }
+  const double cur = 0.5 * fma(ir, o.gtt + o.gpp, o.uc[0]);
+  const double cut = 0.5 * fma(cotir, o.gpp, fma(-ir, o.srt, o.uc[1]));
+  const double cup = 0.5 * fma(-ir, o.srp, fma(-cotir, o.stp, o.uc[2]));
+  const double zr = K.idr * (o.grr + cdr), zt = m[C_MT] * (o.gtt + cdt), zp = m[C_MP] * (o.gpp + cdp);
+  const int kp = g.per ? wrapk(g, k + 1) : k + 1;
+  atomicAdd(A.lam[1] + IRf(g, i, j, k), fma(-m[C_E00], cdr, cur - zr));
+  atomicAdd(A.lam[1] + IRf(g, i + 1, j, k), fma(m[C_E01], cdr, cur + zr));
+  atomicAdd(A.lam[2] + ITf(g, i, j, k), fma(-m[C_E10], cdt, cut - zt));
+  atomicAdd(A.lam[2] + ITf(g, i, j + 1, k), fma(m[C_E11], cdt, cut + zt));
+  atomicAdd(A.lam[3] + IPf(g, i, j, k), cup - zp);
+  atomicAdd(A.lam[3] + IPf(g, i, j, kp), cup + zp);
+  const double qt = m[C_QMT], qp = m[C_QMP], qr = K.qidr;
+  const double rt = qr * o.srt, tr = qt * o.srt, rp = qr * o.srp, pr = qp * o.srp, tp = qt * o.stp, pt = qp * o.stp;
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    scat_v<1>(g, A.lam[2], i + 1, j + s, k, rt);
+    scat_v<1>(g, A.lam[2], i - 1, j + s, k, -rt);
+    scat_v<0>(g, A.lam[1], i + s, j + 1, k, tr);
+    scat_v<0>(g, A.lam[1], i + s, j - 1, k, -tr);
+    scat_v<2>(g, A.lam[3], i + 1, j, k + s, rp);
+    scat_v<2>(g, A.lam[3], i - 1, j, k + s, -rp);
+    scat_v<0>(g, A.lam[1], i + s, j, k + 1, pr);
+    scat_v<0>(g, A.lam[1], i + s, j, k - 1, -pr);
+    scat_v<2>(g, A.lam[3], i, j + 1, k + s, tp);
+    scat_v<2>(g, A.lam[3], i, j - 1, k + s, -tp);
+    scat_v<1>(g, A.lam[2], i, j + s, k + 1, pt);
+    scat_v<1>(g, A.lam[2], i, j + s, k - 1, -pt);
   }
 }
 
@@ -377,4 +358,4 @@ __global__ void k_axpy(long n, double s, const double* __restrict__ x, double* _
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) y[e] += s * x[e];
 }
 
-}  // namespace adj
+}  // namespace f64

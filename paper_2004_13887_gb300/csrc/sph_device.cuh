@@ -26,26 +26,9 @@
 
 namespace sph {
 
-// Value-type traits of the row templates.  R is the kernels' bulk type (float
-// or double) or the adjoint's tape value: T is the type of the metric tables and
-// of the grid spacings, CP what a row reads a field or a coefficient plane
-// through, MP what the coefficient stage writes a plane through.  For float and
-// double these are the plain types and pointers; the adjoint specialises them
-// (tables stay double, reads record tape leaves).
-template <typename R>
-struct Val {
-  using T = R;
-  using CP = const R*;
-  using MP = R*;
-};
-template <typename R> using TabT = typename Val<R>::T;
-// whether R is the FP32 bulk type (the mixed mode's pair arithmetic) or an
-// FP64 value (double, or the adjoint's tape value on doubles)
-template <typename R> constexpr bool is_f32 = std::is_same<R, float>::value;
-
 template <typename R>
 struct Geo {
-  using T = TabT<R>;
+  using T = R;
   int nr, nt, np, npf, per;
   T dr, dth, dph, idr, idth, idph;
   // metric tables: centres rc[nr], faces rf[nr+1]; theta centres/faces
@@ -181,7 +164,7 @@ __device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, f
 
 template <typename R>
 struct Coef {  // per cell centre, frozen at Ubar
-  using MP = typename Val<R>::MP;
+  using MP = R*;
   MP Pb, Tb, rho, drho, beta, uc0, uc1, uc2;
   MP grr, gtt, gpp, srt, srp, stp;  // G_rr, G_tt, G_pp, G_rt+G_tr, G_rp+G_pr, G_tp+G_pt
   // the three parts of div(Ubar) at the centre, (1/r^2) d_r (r^2 u_r),
@@ -191,7 +174,7 @@ struct Coef {  // per cell centre, frozen at Ubar
 };
 constexpr int NCOEF = 17;
 
-template <typename R> struct CF { typename Val<R>::CP f[5]; };
+template <typename R> struct CF { const R* f[5]; };
 template <typename R> struct MF { R* f[5]; };
 
 // 32-bit flat indices: the host refuses grids whose arrays (and line-solve
@@ -311,7 +294,7 @@ __device__ __forceinline__ R rho_at(const Geo<R>& g, const Coef<R>& c, int i, in
 // data) and the periodic wrap (only used for the components tangential to phi);
 // elsewhere the face average with all checks.
 template <int CC, typename R>
-__device__ __forceinline__ R ucen(const Geo<R>& g, const typename Val<R>::CP& plane, int i, int j, int k) {
+__device__ __forceinline__ R ucen(const Geo<R>& g, const R* plane, int i, int j, int k) {
   if (k < 0 || k >= g.np) {
     if (g.per) k = wrapk(g, k);
     else return -plane[IC(g, i, j, k < 0 ? 0 : g.np - 1)];
@@ -468,7 +451,7 @@ template <typename R>
 struct FPt { R rho0, rho1, ub; };
 
 template <typename R>
-__device__ __forceinline__ FPt<R> load_f(const Geo<R>& g, const Coef<R>& c, const typename Val<R>::CP& ubd, int d, int i,
+__device__ __forceinline__ FPt<R> load_f(const Geo<R>& g, const Coef<R>& c, const R* ubd, int d, int i,
                                          int j, int k) {
   FPt<R> q;
   if (d == 0) {
@@ -518,7 +501,7 @@ __device__ __forceinline__ void row_fw(const Geo<R>& g, const Par& P, const FPt<
 }
 
 template <typename R>
-__device__ __forceinline__ void row_f(const Geo<R>& g, const Par& P, const Coef<R>& c, const typename Val<R>::CP& ubd, int d, int i,
+__device__ __forceinline__ void row_f(const Geo<R>& g, const Par& P, const Coef<R>& c, const R* ubd, int d, int i,
                                       int j, int k, R wp[2], R wu[3]) {
   row_fw(g, P, load_f(g, c, ubd, d, i, j, k), d, i, j, wp, wu);
 }

@@ -11,6 +11,7 @@
 #include "sph_host.cuh"
 #include "sph_fp64.cuh"
 #include "sph_fp64_lines.cuh"
+#include "sph_adjoint.cuh"
 
 // what the FP64 mode's coefficient and right-hand-side kernels take
 static f64::Args args64(sph_ctx* c, CF<double> ub) {
@@ -95,6 +96,26 @@ void f64_lines(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int 
   else if (c->d64.g.per) SPH_LINES64(2, true);
   else SPH_LINES64(2, false);
 #undef SPH_LINES64
+}
+
+void f64_adjoint(sph_ctx* c, double tau, CF<double> ub, const CF<double>* mu, const CF<double>* x, double* const* lam) {
+  static_assert(f64::NL == f64::ADJ_PLANES, "the accumulators of k_adj_u");
+  const Geo<double>& g = c->d64.g;
+  f64::AdjArgs A;
+  memset(&A, 0, sizeof A);
+  A.g = g; A.k = f64::consts_of(g, c->P); A.T = c->tabs; A.c = c->d64.c; A.ub = ub; A.tau = tau;
+  for (int d = 0; d < 3; d++) { A.mu[d] = mu[d]; A.x[d] = x[d]; }
+  for (int f = 0; f < 5; f++) A.lam[f] = lam[f];
+  for (int q = 0; q < f64::NL; q++) A.pl[q] = c->adjC + (size_t)q * c->N;
+  f64::k_adj_u<0><<<tile_grid(g.np, g.nt, g.nr + 1), TILE_BLOCK, 0, c->st>>>(A);
+  f64::k_adj_u<1><<<tile_grid(g.np, g.nt + 1, g.nr), TILE_BLOCK, 0, c->st>>>(A);
+  f64::k_adj_u<2><<<tile_grid(g.npf, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
+  f64::k_adj_c<<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
+}
+
+void f64_axpy(sph_ctx* c, long n, double s, const double* x, double* y) {
+  const long b = (n + 255) / 256;
+  f64::k_axpy<<<(unsigned)(b < 16L * c->nsm ? b : 16L * c->nsm), 256, 0, c->st>>>(n, s, x, y);
 }
 
 #ifdef SPH_CHECKED

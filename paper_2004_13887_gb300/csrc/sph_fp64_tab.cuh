@@ -65,6 +65,7 @@ struct Rows {
   long nc, nf[3];  // centres; faces of each kind
 };
 constexpr int ROWS_C = 5, ROWS_F = 4, ROWS_S = 6;
+constexpr int ADJ_PLANES = 8;   // coefficient planes whose cotangents the adjoint accumulates
 // slot of direction d among the transverse directions of component cc
 __host__ __device__ constexpr int trans_slot(int cc, int d) { return d < cc ? d : d - 1; }
 

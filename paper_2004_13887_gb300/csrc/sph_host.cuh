@@ -83,13 +83,7 @@ struct sph_ctx {
   size_t foff[5];         // offsets of the fields in a set
   double* adjS;           // U^{n+1,k}, k < adjK
   double* adjW;           // 10 sets: lam_n, lam, mu_r, mu_theta, mu_phi, x_r, x_theta, x_phi, lam_Ubar, spare
-  double* adjC;           // the coefficient planes' accumulators (17 planes)
-  double* tape_d;
-  int* tape_ix;
-  int* tape_li;
-  double* tape_adj;
-  int* adj_info;          // longest tape used
-  int tape_cap, tape_blocks;
+  double* adjC;           // the coefficient planes' accumulators (f64::ADJ_PLANES of them)
 };
 
 #define SPH_FUSED_STREAMS 8
@@ -122,6 +116,10 @@ void f64_rhs(sph_ctx* c, CF<double> ub, CF<double> D, int hasD, double tau, CF<d
 void f64_rows(sph_ctx* c, CF<double> ub, int dir);
 void f64_lines(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base, MF<double> uk,
                bool transposed, bool norms);
+// the step adjoint's gradient over Ubar into lam (added to; adjC zeroed before),
+// and y += s x
+void f64_adjoint(sph_ctx* c, double tau, CF<double> ub, const CF<double>* mu, const CF<double>* x, double* const* lam);
+void f64_axpy(sph_ctx* c, long n, double s, const double* x, double* y);
 
 // frees what sph_batch_capture_fused allocated (sph_batch.cu)
 void batch_fused_free(sph_batch* b);

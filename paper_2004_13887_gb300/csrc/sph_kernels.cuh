@@ -99,10 +99,9 @@ __global__ void k_cvt_in(long n, const double* __restrict__ a, R* __restrict__ o
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += s) o[t] = (R)a[t];
 }
 
-// The coefficients of centre (i, j, k) (flat index t) into c: the planes of a
-// Coef (k_coef), or the adjoint's slots for the same values.
-template <int CIJ, typename R, typename Out>
-__device__ __forceinline__ void coef_at(const Geo<R>& g, const Par& P, const CF<R>& ub, const Out& c, int i, int j,
+// The coefficients of centre (i, j, k) (flat index t) into the planes of c.
+template <int CIJ, typename R>
+__device__ __forceinline__ void coef_at(const Geo<R>& g, const Par& P, const CF<R>& ub, const Coef<R>& c, int i, int j,
                                         int k, int t) {
   const auto UR = ub.f[1];
   const auto UT = ub.f[2];
@@ -215,28 +214,12 @@ __device__ __forceinline__ float div_ubar_ff(const Geo<float>& g, const CF<float
   return sh + sl;
 }
 
-// div(Ubar) at centre (i,j,k) from Ubar itself (the adjoint's evaluation: the
-// FP64 kernels form it from U^n and U^k, the same value up to rounding)
-template <typename R>
-__device__ __forceinline__ R div_ubar_of(const Geo<R>& g, const CF<R>& ub, int i, int j, int k) {
-  int a0 = IRf(g, i, j, k), a1 = IRf(g, i + 1, j, k);
-  int b0 = ITf(g, i, j, k), b1 = ITf(g, i, j + 1, k);
-  int kp = g.per ? wrapk(g, k + 1) : k + 1;
-  int c0 = IPf(g, i, j, k), c1 = IPf(g, i, j, kp);
-  auto ir = g.irc[i], is = g.isc[j];
-  auto f0 = g.rf[i] * g.rf[i], f1 = g.rf[i + 1] * g.rf[i + 1];
-  R dr_ = (f1 * ub.f[1][a1] - f0 * ub.f[1][a0]) * (ir * ir * g.idr);
-  R dt_ = (g.sf[j + 1] * ub.f[2][b1] - g.sf[j] * ub.f[2][b0]) * (ir * is * g.idth);
-  R dp_ = (ub.f[3][c1] - ub.f[3][c0]) * (ir * is * g.idph);
-  return dr_ + dt_ + dp_;
-}
-
 // R = -(U^k - U^n) - tau (N(Ubar) + G - S) for the p- and T-rows: one thread per
 // centre; written to Rout.f[0][t], Rout.f[4][t].
-template <int CIJ, typename R, typename Out>
+template <int CIJ, typename R>
 __device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Par& P, const Coef<R>& c,
                                          const CF<R>& ub, const CF<R>& ul, const CF<R>& D, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const Out& Rout, int i, int j, int k, int t) {
+                                         const MF<R>& Rout, int i, int j, int k, int t) {
   const auto Pp = ub.f[0];
   const auto UR = ub.f[1];
   const auto UT = ub.f[2];
@@ -269,9 +252,7 @@ __device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Par& P, const Co
     if (d == 0) accT += w.adv * g.dbgT[i] - w.dif * g.lapT[i];
     aT = w.a;
   }
-  R divu;
-  if constexpr (is_f32<R>) divu = div_ubar_ff(g, ub, ul, i, j, k);
-  else divu = div_ubar_of(g, ub, i, j, k);
+  const R divu = div_ubar_ff(g, ub, ul, i, j, k);
   // Cross terms of the viscous dissipation: the centred derivative sums
   // d_r u_t + d_t u_r / r, d_r u_p + d_p u_r / (r sin), d_t u_p / r + d_p u_t / (r sin)
   // of the centre-averaged velocities.  k_coef forms the same sums minus the
@@ -306,10 +287,10 @@ __global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_c(Geo<R> g, Par P,
 
 // R for the momentum row of component D on its faces: one thread per face
 // (zero on wall faces, which are not unknowns); written to Rout.f[1 + D][t].
-template <int CIJ, int D, typename R, typename Out>
+template <int CIJ, int D, typename R>
 __device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Coef<R>& c, const CF<R>& ub,
                                          const CF<R>& Dv, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const Out& Rout, int i, int j, int k, int t) {
+                                         const MF<R>& Rout, int i, int j, int k, int t) {
   const auto Pp = ub.f[0];
   const auto UR = ub.f[1];
   const auto UT = ub.f[2];
