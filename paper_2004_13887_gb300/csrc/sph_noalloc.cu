@@ -18,6 +18,7 @@
 #include "../../include/sph.h"
 
 #define NOALLOC_MAX_DEVICES 64
+#define SPLIT_LINES 8192
 
 static __device__ __align__(256) double g_noalloc_scratch[(size_t)SPH_NOALLOC_MAX_BLOCKS * 12];
 
@@ -100,6 +101,79 @@ __global__ void k_block_thomas_noalloc(int nlines, int n, const double* __restri
   }
 }
 
+// Few lines: 16 lanes per line, two lines per warp.  A FP64 instruction of a warp
+// takes 64 cycles of its SM quarter however many lanes are active, so one
+// thread per line leaves a serial chain of ~120 of them per block on a few
+// warps.  Here lane 4 r + q holds element (r, q) of [C'_m | d'_m] (3 x 4; lanes 12-15
+// repeat row 2) and every product of the same elimination, in the same order,
+// is one element per lane, its operands exchanged by shuffles: 17 FP64
+// instructions a block.  1024 lines of 128 blocks: 685 -> 154 us.
+__device__ __forceinline__ double from(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+__global__ void __launch_bounds__(32) k_block_thomas_split(int nlines, int n, const double* __restrict__ A,
+                                                           const double* __restrict__ B, const double* __restrict__ C,
+                                                           const double* __restrict__ d, double* __restrict__ x,
+                                                           double* __restrict__ scr) {
+  const int lane = threadIdx.x, g0 = lane & 16, e = lane & 15, q = e & 3, r = e >> 2 < 3 ? e >> 2 : 2;
+  const int l0 = blockIdx.x * 2 + (lane >> 4);
+  const bool valid = l0 < nlines;
+  const long l = valid ? l0 : nlines - 1;
+  // element (a, b) of the 3 x 3 (or 3 x 4) array spread over the line's lanes
+  auto at = [&](double v, int a, int b) { return from(v, g0 + 4 * a + b); };
+  const int r1 = (r + 1) % 3, r2 = (r + 2) % 3, q3 = q < 3 ? q : 0, q1 = (q3 + 1) % 3, q2 = (q3 + 2) % 3;
+  double an[3], cn[3], bn;
+  auto fetch = [&](int m) {
+    const long b = l * n + m;
+#pragma unroll
+    for (int z = 0; z < 3; z++) {
+      an[z] = m > 0 ? A[9 * b + 3 * r + z] : 0.0;
+      cn[z] = q < 3 && m < n - 1 ? C[9 * b + 3 * z + q] : 0.0;
+    }
+    bn = q < 3 ? B[9 * b + 3 * r + q] : d[3 * b + r];
+  };
+  bool bad = false;
+  double v = 0.0;   // element (r, q) of [C' | d'] of the block before
+  fetch(0);
+  for (int m = 0; m < n; m++) {
+    const double a0 = an[0], a1 = an[1], a2 = an[2], c0 = cn[0], c1 = cn[1], c2 = cn[2];
+    double t = bn;
+    if (m + 1 < n) fetch(m + 1);
+    if (m > 0) t = t - fma(a2, at(v, 2, q), fma(a1, at(v, 1, q), a0 * at(v, 0, q)));
+    // adj(S): element (r, q) is the cofactor of (q, r), column q's rows r1, r2 ... of S
+    const double s11 = at(t, q1, r1), s22 = at(t, q2, r2), s12 = at(t, q1, r2), s21 = at(t, q2, r1);
+    const double adj = fma(s11, s22, -(s12 * s21));
+    const double det = fma(at(t, 0, 2), at(adj, 2, 0), fma(at(t, 0, 1), at(adj, 1, 0), at(t, 0, 0) * at(adj, 0, 0)));
+    const unsigned hi = (unsigned)__double2hiint(det) & 0x7fffffffu;
+    if (hi >= 0x7ff00000u || (hi | (unsigned)__double2loint(det)) == 0u) bad = true;   // zero or non-finite pivot
+    const double u0 = q < 3 ? c0 : 0.0, u1 = q < 3 ? c1 : 0.0, u2 = q < 3 ? c2 : 0.0;
+    const double y0 = at(t, 0, 3), y1 = at(t, 1, 3), y2 = at(t, 2, 3);
+    const double w = fma(at(adj, r, 2), q < 3 ? u2 : y2, fma(at(adj, r, 1), q < 3 ? u1 : y1, at(adj, r, 0) * (q < 3 ? u0 : y0)));
+    v = w * (1.0 / det);
+    if (m < n - 1 && valid && e < 12) scr[(l * n + m) * 12 + e] = v;
+  }
+  __syncwarp();
+  double xs[3];
+#pragma unroll
+  for (int z = 0; z < 3; z++) xs[z] = at(v, z, 3);
+  double en[4];
+  auto back = [&](int m) {
+    const double* s = scr + (l * n + m) * 12 + 4 * r;
+#pragma unroll
+    for (int z = 0; z < 4; z++) en[z] = s[z];
+  };
+  if (n >= 2) back(n - 2);
+  for (int m = n - 1; m >= 0; m--) {
+    if (m < n - 1) {
+      const double e0 = en[0], e1 = en[1], e2 = en[2], gq = en[3];
+      if (m > 0) back(m - 1);
+      const double mine = gq - fma(e2, xs[2], fma(e1, xs[1], e0 * xs[0]));
+#pragma unroll
+      for (int z = 0; z < 3; z++) xs[z] = at(mine, z, 0);
+    }
+    if (valid && q == 0 && e < 12) x[3 * (l * n + m) + r] = bad ? NAN : r == 0 ? xs[0] : r == 1 ? xs[1] : xs[2];
+  }
+}
+
 // Per-device set-up, with that device current: the device address of the array.
 static int noalloc_setup(int dev) {
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return SPH_ERR_ARG;
@@ -119,8 +193,16 @@ extern "C" int sph_block_thomas_noalloc(int nlines, int n, const double* A, cons
   int e = noalloc_setup(dev);
   if (e != SPH_OK) return e;
   cudaStream_t st = (cudaStream_t)stream;
-  int threads = 128;
-  int blocks = (nlines + threads - 1) / threads;
-  k_block_thomas_noalloc<<<blocks, threads, 0, st>>>(nlines, n, A, B, C, d, x, s_scratch[dev]);
+  // the lane-split form needs 17 FP64 instructions a block on nlines / 2 warps,
+  // one thread per line about 120 on nlines / 32, over the 608 SM quarters: the
+  // split's time grows with the lines once they fill the quarters (1216 lines)
+  // and reaches the other's at about 8192
+  if (nlines <= SPLIT_LINES) {
+    k_block_thomas_split<<<(nlines + 1) / 2, 32, 0, st>>>(nlines, n, A, B, C, d, x, s_scratch[dev]);
+  } else {
+    int threads = 32;
+    int blocks = (nlines + threads - 1) / threads;
+    k_block_thomas_noalloc<<<blocks, threads, 0, st>>>(nlines, n, A, B, C, d, x, s_scratch[dev]);
+  }
   return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
