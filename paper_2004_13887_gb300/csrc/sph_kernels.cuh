@@ -478,10 +478,11 @@ __device__ __forceinline__ void assemble_pts(const Geo<R>& g, const Par& P, cons
   }
 }
 
-// face m+1 of cell m on a line along d (wrapping to 0 on a cyclic line)
-__device__ __forceinline__ void next_face(int d, int n, int m, int i, int j, int k, int& fi, int& fj, int& fk) {
+// face m+1 of cell m on a line along d (wrapping to 0 on a cyclic line; the wall
+// face n of a walled one)
+__device__ __forceinline__ void next_face(int d, int n, int cyc, int m, int i, int j, int k, int& fi, int& fj, int& fk) {
   fi = i; fj = j; fk = k;
-  if (d == 0) fi = m + 1; else if (d == 1) fj = m + 1; else fk = (m + 1 == n) ? 0 : m + 1;
+  if (d == 0) fi = m + 1; else if (d == 1) fj = m + 1; else fk = (cyc && m + 1 == n) ? 0 : m + 1;
 }
 
 // Assemble block m of (I + h D_d) on a line; h = tau/2.
@@ -491,7 +492,7 @@ __device__ void assemble_block(const Geo<R>& g, const Par& P, const Coef<R>& c, 
   CPt<R> cq = load_c(c, d, IC(g, i, j, k));
   FPt<R> fq = {R(1), R(1), R(0)};
   int fi, fj, fk;
-  next_face(d, n, m, i, j, k, fi, fj, fk);
+  next_face(d, n, cyc, m, i, j, k, fi, fj, fk);
   if (m < n - 1 || cyc) fq = load_f(g, c, ub.f[1 + d], d, fi, fj, fk);
   assemble_pts(g, P, cq, fq, d, n, cyc, m, i, j, fi, fj, h, A, B, C);
 }
@@ -656,7 +657,7 @@ __device__ void block_line(const SweepArgs<R>& S, int line, int a, int b, SqSum<
     fqn = {R(1), R(1), R(0)};
     run = R(0);
     if (m < n - 1 || cyc) {
-      next_face(d, n, m, i, j, k, fi, fj, fk);
+      next_face(d, n, cyc, m, i, j, k, fi, fj, fk);
       fqn = load_f(g, S.c, S.ub.f[1 + d], d, fi, fj, fk);
       run = S.rhs.f[1 + d][face_idx(g, d, fi, fj, fk)];
     }
@@ -689,7 +690,7 @@ __device__ void block_line(const SweepArgs<R>& S, int line, int a, int b, SqSum<
       rr[2 * NR] = run;
       if (m + 1 < n) fetch(m + 1);
       int fi, fj, fk;
-      next_face(d, n, m, i, j, k, fi, fj, fk);
+      next_face(d, n, cyc, m, i, j, k, fi, fj, fk);
       assemble_pts(g, S.P, cq, fq, d, n, cyc, m, i, j, fi, fj, S.h, A, B, C);
     }
     if (cyc) {

@@ -285,7 +285,7 @@ __device__ __forceinline__ void stage_block(const SweepArgs<float>& S, float* sm
   if (D == 1) { cpa4(sm + 5 * FS + si, C.srt + ic); sm[6 * FS + si] = 0.f; }
   if (D == 2) { cpa4(sm + 5 * FS + si, C.srp + ic); cpa4(sm + 6 * FS + si, C.stp + ic); }
   int fi, fj, fk;
-  next_face(D, n, c, i, j, k, fi, fj, fk);
+  next_face(D, n, cyc, c, i, j, k, fi, fj, fk);
   int f = face_idx(g, D, fi, fj, fk);
   cpa4(sm + 7 * FS + si, S.ub.f[1 + D] + f);
   if (c < n - 1 || cyc) cpa4(sm + 10 * FS + si, S.rhs.f[1 + D] + f);
@@ -419,7 +419,7 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
       int si = sidx<P, L, CB>(w, m);
       int i, j, k, fi, fj, fk;
       line_pos(D, a, b, m, i, j, k);
-      next_face(D, n, m, i, j, k, fi, fj, fk);
+      next_face(D, n, cyc, m, i, j, k, fi, fj, fk);
       float ufn = sm[7 * FS + si];
       CPt<float> cq;
       cq.Pb = th.Pb; cq.Tb = th.Tb; cq.beta = th.beta;
@@ -589,7 +589,7 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
       S.x.f[0][ic] = sm[si];
       S.x.f[4][ic] = sm[FS + si];
       int fi, fj, fk;
-      next_face(D, n, c, i, j, k, fi, fj, fk);
+      next_face(D, n, cyc, c, i, j, k, fi, fj, fk);
       S.x.f[1 + D][face_idx(g, D, fi, fj, fk)] = (c < n - 1 || cyc) ? sm[2 * FS + si] : 0.f;
       if (c == 0 && !cyc) {
         int wi = i, wj = j, wk = k;
@@ -610,7 +610,7 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
       line_pos(D, G.a, G.bb + lw, c, i, j, k);
       ic[q] = IC(g, i, j, k);
       int fi, fj, fk;
-      next_face(D, n, c, i, j, k, fi, fj, fk);
+      next_face(D, n, cyc, c, i, j, k, fi, fj, fk);
       iu[q] = face_idx(g, D, fi, fj, fk);
       if (c == 0 && !cyc) {
         int wi = i, wj = j, wk = k;
