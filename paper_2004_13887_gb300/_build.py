@@ -10,9 +10,10 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libsph.so")
 LIB_CHECKED = os.path.join(HERE, "libsph_checked.so")   # bounds-checked debug build (SPH_CHECKED)
-SOURCES = ["sph.cu", "sph_fp64.cu", "sph_batch.cu", "sph_noalloc.cu", "sph_schur.cu"]
+SOURCES = ["sph.cu", "sph_fp64.cu", "sph_lines2.cu", "sph_stencil32.cu", "sph_batch.cu", "sph_noalloc.cu", "sph_schur.cu"]
 HEADERS = ["sph_device.cuh", "sph_kernels.cuh", "sph_host.cuh", "sph_lines.cuh", "sph_fp64.cuh", "sph_fp64_tab.cuh",
-           "sph_fp64_lines.cuh", "sph_blk3.cuh", "sph_adjoint.cuh"]
+           "sph_fp64_lines.cuh", "sph_blk3.cuh", "sph_lines2.cuh",
+           "sph_lines2_kernels.cuh", "sph_stencil32.cuh", "sph_adjoint.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

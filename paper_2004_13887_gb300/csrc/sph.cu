@@ -46,7 +46,6 @@ using namespace sph;
 
 #include "sph_kernels.cuh"
 
-#include "sph_lines.cuh"
 
 // ============================================================== host side
 
@@ -100,12 +99,13 @@ extern "C" long long sph_launch_count(const sph_ctx* ctx) { return ctx ? ctx->la
 
 extern "C" int sph_bounds_report(int* first) {
 #ifdef SPH_CHECKED
-  int h[5] = {0, 0, 0, 0, 0}, z[5] = {0, 0, 0, 0, 0}, o[2][5];
+  int h[5] = {0, 0, 0, 0, 0}, z[5] = {0, 0, 0, 0, 0}, o[4][5];
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpyFromSymbol(h, g_bounds, sizeof h) != cudaSuccess ||
       cudaMemcpyToSymbol(g_bounds, z, sizeof z) != cudaSuccess || bounds_take_batch(o[0]) != SPH_OK ||
-      bounds_take_f64(o[1]) != SPH_OK)
+      bounds_take_f64(o[1]) != SPH_OK || bounds_take_lines2(o[2]) != SPH_OK ||
+      bounds_take_s32(o[3]) != SPH_OK)
     return SPH_ERR_CUDA;
-  for (int u = 0; u < 2; u++) {
+  for (int u = 0; u < 4; u++) {
     if (h[0] == 0)
       for (int q = 1; q < 5; q++) h[q] = o[u][q];
     h[0] += o[u][0];
@@ -143,7 +143,7 @@ static void free_all(sph_ctx* c) {
   if (c->efork) cudaEventDestroy(c->efork);
   bufs_free(c->d64);
   bufs_free(c->d32);
-  cudaFree(c->bg); cudaFree(c->acc); cudaFree(c->flag); cudaFree(c->rows64); cudaFree(c->tab64);
+  cudaFree(c->bg); cudaFree(c->acc); cudaFree(c->flag); cudaFree(c->rows64); cudaFree(c->tab64); cudaFree(c->tab32); cudaFree(c->tab32s);
   cudaFree(c->wmean64); cudaFree(c->wmean32); cudaFree(c->wnext);
   cudaFree(c->wzero64); cudaFree(c->wzero32);
   cudaFree(c->adjS); cudaFree(c->adjW); cudaFree(c->adjC);
@@ -277,6 +277,7 @@ static int upload_background(sph_ctx* c, const double* pref, const double* Tref)
   if (e == SPH_OK && c->prec == SPH_PREC_MIXED) e = upload_tables(c, c->d32, c->hmet, der, nr);
   if (e == SPH_OK && c->tab64) {
     f64_tables(c);
+    if (c->tab32s) s32_tables(c);
     if (cudaGetLastError() != cudaSuccess) e = SPH_ERR_CUDA;
   }
   free(der);
@@ -353,6 +354,10 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
     free(c->hmet); free(c); return SPH_ERR_ARG;
   }
   int mixed = c->prec == SPH_PREC_MIXED;
+  for (int d = 0; d < 3 && mixed; d++) {   // (these kernels index their scratch with size_t)
+    const size_t need = lines2_scratch(g, d);
+    if (nscr < need) nscr = need;
+  }
   c->nscr = nscr;
   int err = bufs_alloc(c->d64, c->nmet, nr, c->nf, c->N, nscr, !mixed);
   if (err == SPH_OK && mixed) err = bufs_alloc(c->d32, c->nmet, nr, c->nf, c->N, nscr, 1);
@@ -367,10 +372,9 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
                         !cuda_ok(cudaMalloc((void**)&c->flag, sizeof(int)))))
     err = SPH_ERR_NOMEM;
   if (err == SPH_OK && !mixed) {
-    // the line rows of the FP64 mode and the tables of its kernels
+    // the line rows of the FP64 mode
     const size_t rc = f64::ROWS_C * (size_t)c->N, rf = f64::ROWS_F, rs = f64::ROWS_S;
-    if (!cuda_ok(cudaMalloc((void**)&c->rows64, (3 * rc + (rf + rs) * (c->nf[1] + c->nf[2] + c->nf[3])) * sizeof(double))) ||
-        !cuda_ok(cudaMalloc((void**)&c->tab64, f64::tabs_doubles(nr, nt) * sizeof(double)))) {
+    if (!cuda_ok(cudaMalloc((void**)&c->rows64, (3 * rc + (rf + rs) * (c->nf[1] + c->nf[2] + c->nf[3])) * sizeof(double)))) {
       err = SPH_ERR_NOMEM;
     } else {
       double* p = c->rows64;
@@ -381,8 +385,15 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
         c->rows.f[d] = p; p += rf * c->nf[1 + d];
         c->rows.s[d] = p; p += rs * c->nf[1 + d];
       }
-      c->tabs = f64::tabs_of(c->tab64, nr, nt);
     }
+  }
+  if (err == SPH_OK) {
+    if (!cuda_ok(cudaMalloc((void**)&c->tab64, f64::tabs_doubles(nr, nt) * sizeof(double))) ||
+        (mixed && (!cuda_ok(cudaMalloc((void**)&c->tab32s, s32_tab_floats(nr, nt) * sizeof(float))) ||
+                   !cuda_ok(cudaMalloc((void**)&c->tab32, lines2_tab_floats(nr, nt) * sizeof(float))))))
+      err = SPH_ERR_NOMEM;
+    else
+      c->tabs = f64::tabs_of(c->tab64, nr, nt);
   }
   if (err != SPH_OK) { cudaGetLastError(); free_all(c); free(c); return err; }
   if (!cuda_ok(cudaMemset(c->bg, 0, 2 * (size_t)(nr + 2) * sizeof(double))) || !cuda_ok(cudaMemset(c->flag, 0, sizeof(int))))
@@ -418,6 +429,10 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
   free(zb); free(tb);
   if (err != SPH_OK) { free_all(c); free(c); return err; }
   if (mixed && (err = lines_prepare(c)) != SPH_OK) { free_all(c); free(c); return err; }
+  if (mixed) {
+    lines2_tables(c);
+    if (cudaGetLastError() != cudaSuccess) { free_all(c); free(c); return SPH_ERR_CUDA; }
+  }
   if (cudaEventCreateWithFlags(&c->efork, cudaEventDisableTiming) != cudaSuccess) err = SPH_ERR_CUDA;
   for (int q = 0; q < 3 && !err; q++)
     if (cudaStreamCreateWithFlags(&c->aux[q], cudaStreamNonBlocking) != cudaSuccess ||
@@ -643,6 +658,16 @@ static int grid_stride_blocks(long n) {
   return (int)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b));
 }
 
+static int lines2_use(const sph_ctx* c, int d);
+
+// whether some sweep of the mixed mode takes the one-thread-per-line solver,
+// which reads the planes Pb, Tb, beta
+static int thomas_used(const sph_ctx* c) {
+  for (int d = 0; d < 3; d++)
+    if (c->line_solver == SPH_LINES_THOMAS || (!lines_ok(c, d) && !lines2_use(c, d))) return 1;
+  return 0;
+}
+
 // Ubar into the bulk buffer (FP64 mode at k = 0: U^n itself); coefficients
 template <typename R>
 static int prepare(sph_ctx* c, Bufs<R>& b, int have_iter, CF<R>* ub_out, double* const* ukp = nullptr) {
@@ -666,11 +691,8 @@ static int prepare(sph_ctx* c, Bufs<R>& b, int have_iter, CF<R>* ub_out, double*
     ub = cf_of(b.Ub);
   }
   k_begin(c, SPH_K_COEF);
-  const Geo<double>& gg = c->d64.g;
-  if constexpr (sizeof(R) == sizeof(double)) {
-    f64_coef(c, ub);
-  } else if (b.g.hasw) k_coef<R, true><<<tile_grid(gg.np, gg.nt, gg.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, ub, b.c);
-  else k_coef<R, false><<<tile_grid(gg.np, gg.nt, gg.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, ub, b.c);
+  if constexpr (sizeof(R) == sizeof(double)) f64_coef(c, ub);
+  else s32_coef(c, ub, thomas_used(c));
   if (launch_ok(c)) return SPH_ERR_CUDA;
   *ub_out = ub;
   return SPH_OK;
@@ -693,35 +715,15 @@ static int join_aux(sph_ctx* c, int n) {
   return SPH_OK;
 }
 
-// The right-hand side stage: centre rows on the context's stream, the
-// momentum rows of the three components on side streams, concurrently (timed
-// as one stage).
-template <bool W>
-static void launch_rhs32(sph_ctx* c, Bufs<float>& b, CF<float> ub, CF<float> ul, CF<float> Dv, int hasD, float tr,
-                         CF<double> src, int has_src, MF<float> Rout) {
-  const Geo<double>& g = c->d64.g;
-  k_rhs_c<float, W><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(b.g, c->P, b.c, ub, ul, Dv, hasD, src,
-                                                                           has_src, tr, Rout);
-  k_rhs_u<float, 0, W><<<tile_grid(g.np, g.nt, g.nr + 1), TILE_BLOCK, 0, c->aux[0]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                      has_src, tr, Rout);
-  k_rhs_u<float, 1, W><<<tile_grid(g.np, g.nt + 1, g.nr), TILE_BLOCK, 0, c->aux[1]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                      has_src, tr, Rout);
-  k_rhs_u<float, 2, W><<<tile_grid(g.npf, g.nt, g.nr), TILE_BLOCK, 0, c->aux[2]>>>(b.g, c->P, b.c, ub, Dv, hasD, src,
-                                                                                   has_src, tr, Rout);
-}
-
+// The right-hand side stage: centre rows on the context's stream, the momentum
+// rows of the three components on side streams, concurrently (timed as one
+// stage).  The FP64 kernels also store the line rows the sweeps read.
 template <typename R>
 static int run_rhs(sph_ctx* c, Bufs<R>& b, CF<R> ub, int hasD, double tau, CF<double> src, int has_src, MF<R> Rout) {
-  CF<R> Dv = cf_of(b.Db);  // U^k - U^n from the averaging stage (zero, and not read, when hasD = 0)
   k_begin(c, SPH_K_RHS);
   if (fork_aux(c, 3)) return SPH_ERR_CUDA;
-  if constexpr (sizeof(R) == sizeof(double)) {
-    f64_rhs(c, ub, Dv, hasD, tau, src, has_src, Rout);   // also stores the line rows the sweeps read
-  } else {
-    CF<float> ul = cf_of(b.UbLo);  // velocity remainders of Ubar
-    if (b.g.hasw) launch_rhs32<true>(c, b, ub, ul, Dv, hasD, (float)tau, src, has_src, Rout);
-    else launch_rhs32<false>(c, b, ub, ul, Dv, hasD, (float)tau, src, has_src, Rout);
-  }
+  if constexpr (sizeof(R) == sizeof(double)) f64_rhs(c, ub, cf_of(b.Db), hasD, tau, src, has_src, Rout);
+  else s32_rhs(c, ub, hasD, tau, src, has_src, Rout);
   if (join_aux(c, 3)) return SPH_ERR_CUDA;
   c->launches += 3;  // launch_ok counts the fourth
   return launch_ok(c);
@@ -862,6 +864,25 @@ static int run_lines_d(sph_ctx* c, SweepArgs<float>& S, int n) {
 template <typename R>
 static constexpr int sweep_block() { return sizeof(R) == sizeof(double) ? 32 : 128; }
 
+// Whether the many-lines solver (sph_lines2.cuh) takes the sweep along d of the
+// mixed mode (with the default line solver).  Lengths the partitioned solver
+// takes: r and theta with enough lines to fill the SMs (measured at 5 to 50 us
+// a sweep's launch, many-lines against partitioned: r, 4096 lines of 16 cells 14.3
+// vs 13.8 us, 8192 of 32 22 vs 26, 16384 of 64 49 vs 63; theta, 8192 lines of 128
+// 74 vs 70, 9216 of 192 114 vs 109, 16384 of 192 144 vs 181; 32768 of 256 376 vs
+// 496; phi 740 + 220 vs 345 + 195: not taken).  Other lengths, where the
+// alternative is one thread a line: any direction from 1024 lines (30 x 60 x 60:
+// 20 vs 43, 31 vs 87, 48 vs 176 us; 100 x 200 x 200: 165 vs 247, 188 vs 437, 350 vs
+// 1268); fewer lines gain little and keep the one-sided elimination, the more
+// accurate one on long stiff lines (512 cells: 6.6e-6 vs 1.1e-5).
+static int lines2_use(const sph_ctx* c, int d) {
+  if (c->line_solver != SPH_LINES_PARTITIONED) return 0;
+  const Geo<double>& g = c->d64.g;
+  const long lines = d == 2 ? (long)g.nr * g.nt : (long)(d == 0 ? g.nt : g.nr) * g.np;
+  if (!lines_ok(c, d)) return lines >= LINES2_MIN_OTHER;
+  return d < 2 && lines >= LINES2_MIN;
+}
+
 // The FP64 sweep along d on the rows the right-hand side (or f64_rows) stored;
 // transposed: the adjoint's.  norms: accumulate the squares of the increments.
 static int run_lines64(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base,
@@ -882,6 +903,16 @@ static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> 
   S.rhs = rhs; S.x = x; S.update = update; S.base = base; S.uk = uk;
   S.scr = b.scr; S.acc = c->acc; S.flag = c->flag;
   line_layout(c->d64.g, d, S);
+  if constexpr (sizeof(R) == sizeof(float)) {
+    if (lines2_use(c, d)) {
+      k_begin(c, SPH_K_SWEEP_R + d);
+      if (fork_aux(c, 1)) return SPH_ERR_CUDA;
+      lines2_run(c, d, tau, ub, rhs, x, update, norms, base, uk, c->aux[0]);
+      if (join_aux(c, 1)) return SPH_ERR_CUDA;
+      c->launches++;
+      return launch_ok(c);
+    }
+  }
   if (sizeof(R) == sizeof(float) && c->line_solver != SPH_LINES_THOMAS && lines_ok(c, d)) {
     SweepArgs<float>& Sf = *reinterpret_cast<SweepArgs<float>*>(&S);
     const Geo<double>& g = c->d64.g;

@@ -24,7 +24,6 @@
 
 #include "../../include/sph.h"
 #include "sph_kernels.cuh"
-#include "sph_lines.cuh"
 #include "sph_host.cuh"
 
 namespace fused {
@@ -47,30 +46,17 @@ constexpr int TILES = FUSED_TILES;
 #ifndef FUSED_MINB_COEF
 #define FUSED_MINB_COEF 10
 #endif
-#ifndef FUSED_MINB_RHSC
-#define FUSED_MINB_RHSC 8
-#endif
-#ifndef FUSED_MINB_RHSU
-#define FUSED_MINB_RHSU 16
+#ifndef FUSED_MINB_RHS
+#define FUSED_MINB_RHS 10
 #endif
 
 struct CoefTab {
-  Geo<float> g;
-  Par P;
-  CF<float> ub;
-  Coef<float> c;
+  s32::Args A;
   Tile t;
 };
 
 struct RhsTab {
-  Geo<float> g;
-  Par P;
-  Coef<float> c;
-  CF<float> ub, ul, Dv;
-  CF<double> src;
-  MF<float> Rout;
-  float tau;
-  int hasD;
+  s32::Args A;
   Tile t[4];  // centres (p, T rows), then the faces of u_r, u_theta, u_phi
 };
 
@@ -136,62 +122,35 @@ __global__ void __launch_bounds__(256) k_avg_f(const AvgArgs<float>* tab, const 
   }
 }
 
-// the coefficient stage (k_coef) over the tiles of every problem
+// the coefficient stage over the tiles of every problem
 __global__ void __launch_bounds__(128, FUSED_MINB_COEF) k_coef_f(const CoefTab* tab, const int2* map) {
-  __shared__ CoefTab A;
+  __shared__ CoefTab S;
   const int2 m = map[blockIdx.x];
-  load_args(A, tab[m.x]);
-  const Geo<float>& g = A.g;
-  const int b1 = min(m.y + TILES, A.t.n);
+  load_args(S, tab[m.x]);
+  const Geo<float>& g = S.A.g;
+  const int b1 = min(m.y + TILES, S.t.n);
   for (int b = m.y; b < b1; b++) {
-    const Pt p = point_of(A.t, b);
-    const bool inner = tile_inner_at(g, p.i0, p.j0, A.t.ti, A.t.tj);
+    const Pt p = point_of(S.t, b);
+    const bool inner = tile_inner_at(g, p.i0, p.j0, S.t.ti, S.t.tj);
     if (p.k >= g.np || p.j >= g.nt || p.i >= g.nr) continue;
     const int t = IC(g, p.i, p.j, p.k);
-    if (inner) coef_at<0>(g, A.P, A.ub, A.c, p.i, p.j, p.k, t);
-    else coef_at<1>(g, A.P, A.ub, A.c, p.i, p.j, p.k, t);
+    if (inner) s32::coef<0>(S.A, p.i, p.j, p.k, t);
+    else s32::coef<1>(S.A, p.i, p.j, p.k, t);
   }
 }
 
-// the p- and T-rows of the right-hand side (k_rhs_c) over every problem
-__global__ void __launch_bounds__(128, FUSED_MINB_RHSC) k_rhs_c_f(const RhsTab* tab, const int2* map) {
-  __shared__ RhsTab A;
+// the right-hand side over every problem: map = (problem, kind * 2^28 + first tile),
+// the tiles of a problem's four kinds one after another
+__global__ void __launch_bounds__(128, FUSED_MINB_RHS) k_rhs_f(const RhsTab* tab, const int2* map) {
+  __shared__ RhsTab S;
   const int2 m = map[blockIdx.x];
-  load_args(A, tab[m.x]);
-  const Geo<float>& g = A.g;
-  const int b1 = min(m.y + TILES, A.t[0].n);
-  for (int b = m.y; b < b1; b++) {
-    const Pt p = point_of(A.t[0], b);
-    const bool inner = tile_inner_at(g, p.i0, p.j0, A.t[0].ti, A.t[0].tj);
-    if (p.k >= g.np || p.j >= g.nt || p.i >= g.nr) continue;
-    const int t = IC(g, p.i, p.j, p.k);
-    if (inner)
-      rhs_c_at<0>(g, A.P, A.c, A.ub, A.ul, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
-    else
-      rhs_c_at<1>(g, A.P, A.c, A.ub, A.ul, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
-  }
-}
-
-// the momentum rows of component D (k_rhs_u) over every problem; zero on wall faces
-template <int D>
-__global__ void __launch_bounds__(128, FUSED_MINB_RHSU) k_rhs_u_f(const RhsTab* tab, const int2* map) {
-  __shared__ RhsTab A;
-  const int2 m = map[blockIdx.x];
-  load_args(A, tab[m.x]);
-  const Geo<float>& g = A.g;
-  const Tile& tl = A.t[1 + D];
-  const int nj = g.nt + (D == 1), nk = D == 2 ? g.npf : g.np;
-  const int b1 = min(m.y + TILES, tl.n);
-  for (int b = m.y; b < b1; b++) {
+  load_args(S, tab[m.x]);
+  const int kind = m.y >> 28, b0 = m.y & 0xfffffff;
+  const Tile& tl = S.t[kind];
+  const int b1 = min(b0 + TILES, tl.n);
+  for (int b = b0; b < b1; b++) {
     const Pt p = point_of(tl, b);
-    const bool inner = tile_inner_at(g, p.i0, p.j0, tl.ti, tl.tj);
-    if (p.k >= nk || p.j >= nj || p.i >= g.nr + (D == 0)) continue;
-    const int t = (p.i * nj + p.j) * nk + p.k;
-    const bool wall = D == 0 ? (p.i == 0 || p.i == g.nr) : D == 1 ? (p.j == 0 || p.j == g.nt)
-                                                                  : (!g.per && (p.k == 0 || p.k == g.np));
-    if (wall) A.Rout.f[1 + D][t] = 0.f;
-    else if (inner) rhs_u_at<0, D>(g, A.P, A.c, A.ub, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
-    else rhs_u_at<1, D>(g, A.P, A.c, A.ub, A.Dv, A.hasD, A.src, 0, A.tau, A.Rout, p.i, p.j, p.k, t);
+    s32::rhs_point<false>(S.A, kind, p.i, p.j, p.k, tile_inner_at(S.A.g, p.i0, p.j0, tl.ti, tl.tj));
   }
 }
 
@@ -221,6 +180,33 @@ __global__ void __launch_bounds__(CB / P, 65536 * P / (CB * 48)) k_lines_sca_f(c
   const int ng1 = tab[m.x].ng1;
   if (m.y < ng1) lines::lines_sca<D, P, L, CB, 1>(S, m.y);
   else lines::lines_sca<D, P, L, CB, 2>(S, m.y - ng1);
+}
+
+// The r- (D = 0) and theta-lines (1) of every problem, of any length, 32 lines a
+// block (sph_lines2.cuh): one launch for the block lines and one for the scalar
+// lines over all problems; map = (problem, block of its launch).
+template <int D>
+__global__ void __launch_bounds__(64, LINES2_MINB) k_l2_blk_f(const lines2::Args* tab, const int2* map) {
+  __shared__ lines2::Args S;
+  __shared__ float ex[24][32];
+  __shared__ float rings[2 * lines2::RING][32];
+  const int2 m = map[blockIdx.x];
+  load_args(S, tab[m.x]);
+  int bad = 0;
+  lines2::block_lines<D>(S, ex, rings, m.y, &bad);
+  if (bad) atomicOr(S.flag, bad);
+}
+template <int D>
+__global__ void __launch_bounds__(64) k_l2_sca_f(const lines2::Args* tab, const int2* map) {
+  __shared__ lines2::Args S;
+  __shared__ float ex[4][32];
+  __shared__ float rings[2 * lines2::SRING][32];
+  const int2 m = map[blockIdx.x];
+  load_args(S, tab[m.x]);
+  int bad = 0;
+  if (m.y < S.nb1) lines2::scalar_lines<D, 1>(S, ex, rings, m.y, m.y, &bad);
+  else lines2::scalar_lines<D, 2>(S, ex, rings, m.y - S.nb1, m.y, &bad);
+  if (bad) atomicOr(S.flag, bad);
 }
 
 }  // namespace fused
@@ -397,7 +383,7 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
   // ---- stencil stages
   std::vector<fused::CoefTab> coef(n);
   std::vector<fused::RhsTab> rhs[2][2];
-  std::vector<int2> mcoef, mrhs[4];
+  std::vector<int2> mcoef, mrhs;
   std::vector<double*> accs(n);
   for (int p = 0; p < 2; p++)
     for (int it = 0; it < 2; it++) {
@@ -423,12 +409,8 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
         }
         fused::RhsTab& R = rhs[p][it][q];
         memset(&R, 0, sizeof R);
-        R.g = B.g; R.P = c->P; R.c = B.c;
-        R.ub = cf5(B.Ub); R.ul = cf5(B.UbLo); R.Dv = cf5(B.Db);
-        R.src = cf5(c->src);
-        R.Rout = mf5(B.Rb);
-        R.tau = (float)dt;
-        R.hasD = it;
+        s32_fill(c, cf5(B.Ub), dt, &R.A);
+        R.A.hasD = it;
       }
     int nb[5];
     fused::Tile tc = tile_of(c, g.np, g.nt, g.nr, &nb[0]);
@@ -436,7 +418,8 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
                          tile_of(c, g.npf, g.nt, g.nr, &nb[3])};
     fused::CoefTab& C = coef[q];
     memset(&C, 0, sizeof C);
-    C.g = B.g; C.P = c->P; C.ub = cf5(B.Ub); C.c = B.c; C.t = tc;
+    s32_fill(c, cf5(B.Ub), dt, &C.A);
+    C.t = tc;
     for (int p = 0; p < 2; p++)
       for (int it = 0; it < 2; it++) {
         fused::RhsTab& R = rhs[p][it][q];
@@ -444,9 +427,9 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
         for (int d = 0; d < 3; d++) R.t[1 + d] = tu[d];
       }
     // a block per fused::TILES consecutive tiles of the problem
-    for (int k = 0; k < nb[0]; k += fused::TILES) { mcoef.push_back(make_int2(q, k)); mrhs[0].push_back(make_int2(q, k)); }
-    for (int d = 0; d < 3; d++)
-      for (int k = 0; k < nb[1 + d]; k += fused::TILES) mrhs[1 + d].push_back(make_int2(q, k));
+    for (int k = 0; k < nb[0]; k += fused::TILES) mcoef.push_back(make_int2(q, k));
+    for (int d = 0; d < 4; d++)
+      for (int k = 0; k < nb[d]; k += fused::TILES) mrhs.push_back(make_int2(q, (d << 28) + k));
     for (int f = 0; f < 5; f++) {
       const long pairs = (long)c->nf[f] >> 1;
       for (long s = 0; s < pairs || (s == 0 && pairs == 0); s += 1024)
@@ -457,8 +440,31 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
   std::vector<Layout> lay;
   std::vector<fused::LineTab> ltab[64][2][2];   // per layout (at most 3 x 15 exist)
   std::vector<int2> lmb[64], lms[64];
-  for (int d = 0; d < 3; d++)
+  // r and theta: lines of any length in one pair of launches where the batch has
+  // enough of them to fill the SMs, as for a single problem (lines2_use)
+  bool two[3] = {false, false, false};
+  std::vector<lines2::Args> l2tab[2];
+  std::vector<int2> l2b[2], l2s[2];
+  for (int d = 0; d < 2; d++) {
+    long lines = 0;
     for (int q = 0; q < n; q++) {
+      const Geo<double>& g = b->c[q]->d64.g;
+      lines += (long)(d == 0 ? g.nt : g.nr) * g.np;
+    }
+    two[d] = lines >= LINES2_MIN;
+    for (int q = 0; q < n && two[d]; q++) {
+      sph_ctx* c = b->c[q];
+      Bufs<float>& B = c->d32;
+      lines2::Args A;
+      int nb0, ns;
+      lines2_fill(c, d, dt, cf5(B.Ub), cf5(d == 1 ? B.X1 : B.Rb), mf5(d == 1 ? B.Rb : B.X1), &A, &nb0, &ns);
+      l2tab[d].push_back(A);
+      for (int k = 0; k < nb0; k++) l2b[d].push_back(make_int2(q, k));
+      for (int k = 0; k < ns; k++) l2s[d].push_back(make_int2(q, k));
+    }
+  }
+  for (int d = 0; d < 3; d++)
+    for (int q = 0; q < n && !two[d]; q++) {
       sph_ctx* c = b->c[q];
       const Geo<double>& g = c->d64.g;
       const int len = d == 0 ? g.nr : d == 1 ? g.nt : g.np;
@@ -513,8 +519,9 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
       orhs[p][it] = blob.put(rhs[p][it]);
     }
   const size_t ocoef = blob.put(coef), omavg = blob.put(mavg), omcoef = blob.put(mcoef), oacc = blob.put(accs);
-  size_t omrhs[4];
-  for (int k = 0; k < 4; k++) omrhs[k] = blob.put(mrhs[k]);
+  const size_t omrhs = blob.put(mrhs);
+  size_t ol2[2], ol2b[2], ol2s[2];
+  for (int d = 0; d < 2; d++) { ol2[d] = blob.put(l2tab[d]); ol2b[d] = blob.put(l2b[d]); ol2s[d] = blob.put(l2s[d]); }
   for (size_t z = 0; z < lay.size(); z++) {
     for (int p = 0; p < 2; p++)
       for (int it = 0; it < 2; it++) lay[z].tab[p][it] = blob.put(ltab[z][p][it]);
@@ -533,7 +540,6 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
   long long nk = 0;
   if (cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SPH_ERR_CUDA;
   int err = SPH_OK;
-  const int nrc = (int)mrhs[0].size();
   for (int s = 0; s < steps && !err; s++) {
     const int p = s & 1;
     for (int it = 0; it < n_iter && !err; it++) {
@@ -544,17 +550,28 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
                                                                 (const int2*)(base + omcoef));
       nk += 2;
       const fused::RhsTab* rt = (const fused::RhsTab*)(base + orhs[p][il]);
-      if ((err = ffork(b, 3))) break;
-      fused::k_rhs_c_f<<<nrc, 128, 0, b->st>>>(rt, (const int2*)(base + omrhs[0]));
-      fused::k_rhs_u_f<0><<<(unsigned)mrhs[1].size(), 128, 0, b->fst[0]>>>(rt, (const int2*)(base + omrhs[1]));
-      fused::k_rhs_u_f<1><<<(unsigned)mrhs[2].size(), 128, 0, b->fst[1]>>>(rt, (const int2*)(base + omrhs[2]));
-      fused::k_rhs_u_f<2><<<(unsigned)mrhs[3].size(), 128, 0, b->fst[2]>>>(rt, (const int2*)(base + omrhs[3]));
-      nk += 4;
-      if ((err = fjoin(b, 3))) break;
+      fused::k_rhs_f<<<(unsigned)mrhs.size(), 128, 0, b->st>>>(rt, (const int2*)(base + omrhs));
+      nk++;
       for (int d = 0; d < 3 && !err; d++) {
         if (d == 2 && it == n_iter - 1) {
           fused::k_zero_acc_f<<<(5 * n + 255) / 256, 256, 0, b->st>>>((double* const*)(base + oacc), n);
           nk++;
+        }
+        if (two[d]) {
+          if ((err = ffork(b, 1))) break;
+          const lines2::Args* lt = (const lines2::Args*)(base + ol2[d]);
+          const int2 *mb = (const int2*)(base + ol2b[d]), *ms = (const int2*)(base + ol2s[d]);
+          const unsigned nb = (unsigned)l2b[d].size(), ns = (unsigned)l2s[d].size();
+          if (d == 0) {
+            fused::k_l2_blk_f<0><<<nb, 64, 0, b->st>>>(lt, mb);
+            fused::k_l2_sca_f<0><<<ns, 64, 0, b->fst[0]>>>(lt, ms);
+          } else {
+            fused::k_l2_blk_f<1><<<nb, 64, 0, b->st>>>(lt, mb);
+            fused::k_l2_sca_f<1><<<ns, 64, 0, b->fst[0]>>>(lt, ms);
+          }
+          nk += 2;
+          err = fjoin(b, 1);
+          continue;
         }
         int used = 0;
         for (size_t z = 0; z < lay.size(); z++) used += lay[z].d == d ? 2 : 0;

@@ -10,6 +10,9 @@
 #include "../../include/sph.h"
 #include "sph_kernels.cuh"
 #include "sph_fp64_tab.cuh"
+#include "sph_stencil32.cuh"
+#include "sph_lines.cuh"
+#include "sph_lines2.cuh"
 
 // Device buffers of one precision.
 template <typename R>
@@ -48,8 +51,10 @@ struct sph_ctx {
   Bufs<float> d32;       // bulk buffers in mixed mode
   double* rows64;        // FP64 mode: the line rows the right-hand side stores for the sweeps
   f64::Rows rows;        // pointers into rows64 (all null in mixed mode)
-  double* tab64;         // FP64 mode: the metric tables of its kernels
+  double* tab64;         // the metric tables of the FP64 kernels (and the FP32 tables' source)
   f64::Tabs tabs;        // pointers into tab64
+  float* tab32s;         // mixed mode: the tables of the stencil stages (sph_stencil32.cuh)
+  float* tab32;          // mixed mode: the tables of the many-lines sweeps (sph_lines2.cuh)
   long long launches;
   long unknowns[5];
   // per-kernel timing
@@ -116,6 +121,24 @@ void f64_rhs(sph_ctx* c, CF<double> ub, CF<double> D, int hasD, double tau, CF<d
 void f64_rows(sph_ctx* c, CF<double> ub, int dir);
 void f64_lines(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base, MF<double> uk,
                bool transposed, bool norms);
+// The mixed mode's stencil stages (sph_stencil32.cu): floats of their tables, the
+// tables' launch (after f64_tables), the arguments a context's launches share,
+// the coefficients (thermo: with the planes Pb, Tb, beta) and the right-hand side.
+size_t s32_tab_floats(int nr, int nt);
+void s32_tables(sph_ctx* c);
+void s32_fill(const sph_ctx* c, CF<float> ub, double tau, s32::Args* A);
+void s32_coef(sph_ctx* c, CF<float> ub, int thermo);
+void s32_rhs(sph_ctx* c, CF<float> ub, int hasD, double tau, CF<double> src, int has_src, MF<float> R);
+// The sweeps of the mixed mode over many lines (sph_lines2.cu): floats
+// of their tables and of the scratch a direction needs, the tables' launch, a
+// sweep (block lines on the context's stream, scalar lines on st_sca).
+size_t lines2_tab_floats(int nr, int nt);
+size_t lines2_scratch(const Geo<double>& g, int d);
+void lines2_tables(sph_ctx* c);
+void lines2_fill(const sph_ctx* c, int d, double tau, CF<float> ub, CF<float> rhs, MF<float> x, lines2::Args* A, int* nblk,
+                 int* nsca);
+void lines2_run(sph_ctx* c, int d, double tau, CF<float> ub, CF<float> rhs, MF<float> x, int update, int norms,
+                CF<double> base, MF<double> uk, cudaStream_t st_sca);
 // the step adjoint's gradient over Ubar into lam (added to; adjC zeroed before),
 // and y += s x
 void f64_adjoint(sph_ctx* c, double tau, CF<double> ub, const CF<double>* mu, const CF<double>* x, double* const* lam);
@@ -127,6 +150,8 @@ void batch_fused_free(sph_batch* b);
 // the bounds counters of the other translation units into h, then zeroed
 int bounds_take_batch(int* h);
 int bounds_take_f64(int* h);
+int bounds_take_lines2(int* h);
+int bounds_take_s32(int* h);
 #endif
 
 

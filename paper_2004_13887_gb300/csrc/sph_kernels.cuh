@@ -99,55 +99,11 @@ __global__ void k_cvt_in(long n, const double* __restrict__ a, R* __restrict__ o
   for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += s) o[t] = (R)a[t];
 }
 
-// The coefficients of centre (i, j, k) (flat index t) into the planes of c.
-template <int CIJ, typename R>
-__device__ __forceinline__ void coef_at(const Geo<R>& g, const Par& P, const CF<R>& ub, const Coef<R>& c, int i, int j,
-                                        int k, int t) {
-  const auto UR = ub.f[1];
-  const auto UT = ub.f[2];
-  const auto UP = ub.f[3];
-  // thermodynamics from background + perturbation.  The density perturbation
-  // rho - rho_ref = (p' T_ref - (p_ref + pi_inf) T') / (Rg T_ref T) has no
-  // cancellation between large terms, so the bulk type keeps its relative
-  // precision for it.
-  R pref = g.pcen[i], Tref = g.Tcen[i];
-  R pp = ub.f[0][t], Tp = ub.f[4][t];
-  Thermo<R> th = thermo(g, P, i, pp, Tp);
-  R iRg = pick<R>(1.0 / P.Rg, P.iRg_f);
-  R itb = sdiv(R(1), th.Tb);
-  c.Pb[t] = th.Pb;
-  c.Tb[t] = th.Tb;
-  c.rho[t] = th.rho;
-  c.drho[t] = sdiv((pp * Tref - pref * Tp) * itb * iRg, Tref);
-  c.beta[t] = th.beta;
-  R ur = hr<CIJ>(g, UR, i, j, k), ut = ht<CIJ>(g, UT, i, j, k), up = hp<CIJ>(g, UP, i, j, k);
-  c.uc0[t] = ur; c.uc1[t] = ut; c.uc2[t] = up;
-  R ir = g.irc[i], is = g.isc[j], cot = g.cotc[j], h = R(0.5);
-  c.grr[t] = (vr<CIJ>(g, UR, i + 1, j, k) - vr<CIJ>(g, UR, i, j, k)) * g.idr;
-  c.gtt[t] = (vt<CIJ>(g, UT, i, j + 1, k) - vt<CIJ>(g, UT, i, j, k)) * ir * g.idth + ur * ir;
-  c.gpp[t] = (vp<CIJ>(g, UP, i, j, k + 1) - vp<CIJ>(g, UP, i, j, k)) * ir * is * g.idph + ur * ir + ut * cot * ir;
-  R grt = (ht<CIJ>(g, UT, i + 1, j, k) - ht<CIJ>(g, UT, i - 1, j, k)) * h * g.idr;
-  R gtr = (hr<CIJ>(g, UR, i, j + 1, k) - hr<CIJ>(g, UR, i, j - 1, k)) * h * ir * g.idth - ut * ir;
-  R grp = (hp<CIJ>(g, UP, i + 1, j, k) - hp<CIJ>(g, UP, i - 1, j, k)) * h * g.idr;
-  R gpr = (hr<CIJ>(g, UR, i, j, k + 1) - hr<CIJ>(g, UR, i, j, k - 1)) * h * ir * is * g.idph - up * ir;
-  R gtp = (hp<CIJ>(g, UP, i, j + 1, k) - hp<CIJ>(g, UP, i, j - 1, k)) * h * ir * g.idth;
-  R gpt = (ht<CIJ>(g, UT, i, j, k + 1) - ht<CIJ>(g, UT, i, j, k - 1)) * h * ir * is * g.idph - up * cot * ir;
-  c.srt[t] = grt + gtr;
-  c.srp[t] = grp + gpr;
-  c.stp[t] = gtp + gpt;
-  c.dvr[t] = (g.rf[i + 1] * g.rf[i + 1] * UR[IRf(g, i + 1, j, k)] - g.rf[i] * g.rf[i] * UR[IRf(g, i, j, k)]) * ir * ir
-           * g.idr;
-  c.dvt[t] = (g.sf[j + 1] * UT[ITf(g, i, j + 1, k)] - g.sf[j] * UT[ITf(g, i, j, k)]) * ir * is * g.idth;
-  c.dvp[t] = (vp<CIJ>(g, UP, i, j, k + 1) - vp<CIJ>(g, UP, i, j, k)) * ir * is * g.idph;
-}
-
 // The stencil kernels run on tiles of TK x TJ x TI points (phi fastest; 128
 // threads; the shape is set per context, sph_set_tile).  A block takes the
 // fast path when its whole tile has its +-2 neighbourhood in r and theta
-// inside the grid (a uniform choice).  On the 128 x 256 x 256 workload the
-// tile shape made no measurable difference (128x1x1 to 16x4x2 all within 3 %),
-// so the default is one phi row; the ensemble's autotuner picks it per grid
-// shape.
+// inside the grid (a uniform choice).  The default is one phi row; the
+// ensemble's autotuner picks the shape per grid.
 template <typename G>
 __device__ __forceinline__ bool tile_inner_at(const G& g, int i0, int j0, int ti, int tj) {
   return inner_ij(g, i0, j0) && inner_ij(g, i0 + ti - 1, j0 + tj - 1);
@@ -156,12 +112,6 @@ template <typename G>
 __device__ __forceinline__ bool tile_inner(const G& g) {
   return tile_inner_at(g, blockIdx.z * blockDim.z, blockIdx.y * blockDim.y, (int)blockDim.z, (int)blockDim.y);
 }
-// The FP32 stencil kernels are bound by load latency: full occupancy (16
-// blocks of 128 threads, 32 registers) pays for its few register spills
-// (measured: the right-hand side 17 % faster than at 64 registers).  (The FP64
-// mode has its own stencil kernels, sph_fp64.cuh.)
-#define STENCIL_MINB(R) (sizeof(R) == 4 ? 16 : 1)
-
 // grid of tiles of tj x ti rows of phi points (128 / (tj ti) each) over an
 // nk x nj x ni index box
 static dim3 tile_grid_of(int tj, int ti, int nk, int nj, int ni) {
@@ -170,239 +120,6 @@ static dim3 tile_grid_of(int tj, int ti, int nk, int nj, int ni) {
 }
 #define tile_grid(nk, nj, ni) tile_grid_of(c->tile_j, c->tile_i, nk, nj, ni)
 #define TILE_BLOCK dim3(128 / (c->tile_j * c->tile_i), c->tile_j, c->tile_i)
-
-// one block per tile
-template <typename R, bool W>
-__global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_coef(Geo<R> g, Par P, CF<R> ub, Coef<R> c) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
-      i = blockIdx.z * blockDim.z + threadIdx.z;
-  bool inner = tile_inner(g) && !g.hasw;  // with wall data every tile takes the checked path
-  if (k >= g.np || j >= g.nt || i >= g.nr) return;
-  int t = IC(g, i, j, k);
-  if (inner) coef_at<0>(g, P, ub, c, i, j, k, t);
-  else coef_at<W ? 2 : 1>(g, P, ub, c, i, j, k, t);
-}
-
-// div(Ubar) at centre (i,j,k) in FP32 mode, from the pair (hi = Ubar, lo) of the
-// velocity components: each face flux and each difference is carried as a pair,
-// so the cancellation of nearly equal fluxes (and of the three directions
-// against each other) at low Mach number costs no accuracy.
-__device__ __forceinline__ float div_ubar_ff(const Geo<float>& g, const CF<float>& ub, const CF<float>& ul, int i,
-                                             int j, int k) {
-  int a0 = IRf(g, i, j, k), a1 = IRf(g, i + 1, j, k);
-  int b0 = ITf(g, i, j, k), b1 = ITf(g, i, j + 1, k);
-  int kp = g.per ? wrapk(g, k + 1) : k + 1;
-  int c0 = IPf(g, i, j, k), c1 = IPf(g, i, j, kp);
-  float ir = g.irc[i], is = g.isc[j];
-  float h0, l0, h1, l1, dh, dl, th, tl, sh, sl;
-  // r: (rf1^2 u1 - rf0^2 u0) / rc^2 / dr
-  ff_mul(g.rf2h[i + 1], g.rf2l[i + 1], ub.f[1][a1], ul.f[1][a1], h1, l1);
-  ff_mul(g.rf2h[i], g.rf2l[i], ub.f[1][a0], ul.f[1][a0], h0, l0);
-  ff_sub(h1, l1, h0, l0, dh, dl);
-  float cr = ir * ir * g.idr;
-  ff_mul(dh, dl, cr, 0.f, sh, sl);
-  // theta: (sf1 u1 - sf0 u0) / (rc sc dtheta)
-  ff_mul(g.sfh[j + 1], g.sfl[j + 1], ub.f[2][b1], ul.f[2][b1], h1, l1);
-  ff_mul(g.sfh[j], g.sfl[j], ub.f[2][b0], ul.f[2][b0], h0, l0);
-  ff_sub(h1, l1, h0, l0, dh, dl);
-  ff_mul(dh, dl, ir * is * g.idth, 0.f, th, tl);
-  ff_add(sh, sl, th, tl, sh, sl);
-  // phi: (u1 - u0) / (rc sc dphi)
-  ff_sub(ub.f[3][c1], ul.f[3][c1], ub.f[3][c0], ul.f[3][c0], dh, dl);
-  ff_mul(dh, dl, ir * is * g.idph, 0.f, th, tl);
-  ff_add(sh, sl, th, tl, sh, sl);
-  return sh + sl;
-}
-
-// R = -(U^k - U^n) - tau (N(Ubar) + G - S) for the p- and T-rows: one thread per
-// centre; written to Rout.f[0][t], Rout.f[4][t].
-template <int CIJ, typename R>
-__device__ __forceinline__ void rhs_c_at(const Geo<R>& g, const Par& P, const Coef<R>& c,
-                                         const CF<R>& ub, const CF<R>& ul, const CF<R>& D, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const MF<R>& Rout, int i, int j, int k, int t) {
-  const auto Pp = ub.f[0];
-  const auto UR = ub.f[1];
-  const auto UT = ub.f[2];
-  const auto UP = ub.f[3];
-  const auto TT = ub.f[4];
-  R mu = pick<R>(P.mu, P.mu_f), gm = pick<R>(P.gamma, P.gamma_f);
-  R ir = g.irc[i];
-  R accp = R(0), accT = R(0);
-  R ap = R(0), aT = R(0);
-#pragma unroll
-  for (int d = 0; d < 3; d++) {
-    int di = d == 0, dj = d == 1, dk = d == 2;
-    R pv[3], Tv[3], uv[2];
-#pragma unroll
-    for (int s = -1; s <= 1; s++) {
-      pv[s + 1] = cpert<CIJ>(g, Pp, i + s * di, j + s * dj, k + s * dk);
-      Tv[s + 1] = cpert<CIJ>(g, TT, i + s * di, j + s * dj, k + s * dk);
-    }
-    if (d == 0) { uv[0] = UR[IRf(g, i, j, k)]; uv[1] = UR[IRf(g, i + 1, j, k)]; }
-    else if (d == 1) { uv[0] = UT[ITf(g, i, j, k)]; uv[1] = UT[ITf(g, i, j + 1, k)]; }
-    else { uv[0] = vp<CIJ>(g, UP, i, j, k); uv[1] = vp<CIJ>(g, UP, i, j, k + 1); }
-    RowC<R> w;
-    row_c(g, P, c, d, 0, i, j, k, w);
-    accp += w.wp[0] * pv[0] + w.wp[2] * pv[2] + w.wT[0] * Tv[0] + w.wT[1] * Tv[1] + w.wT[2] * Tv[2]
-          + w.wv[0] * uv[0] + w.wv[1] * uv[1];
-    if (d == 0) accp += w.adv * g.dbgp[i] - w.dif * g.lapT[i];
-    ap = w.a;
-    row_c(g, P, c, d, 1, i, j, k, w);
-    accT += w.wT[0] * Tv[0] + w.wT[1] * Tv[1] + w.wT[2] * Tv[2] + w.wv[0] * uv[0] + w.wv[1] * uv[1];
-    if (d == 0) accT += w.adv * g.dbgT[i] - w.dif * g.lapT[i];
-    aT = w.a;
-  }
-  const R divu = div_ubar_ff(g, ub, ul, i, j, k);
-  // Cross terms of the viscous dissipation: the centred derivative sums
-  // d_r u_t + d_t u_r / r, d_r u_p + d_p u_r / (r sin), d_t u_p / r + d_p u_t / (r sin)
-  // of the centre-averaged velocities.  k_coef forms the same sums minus the
-  // metric terms u_t / r, u_p / r, u_p cot / r (S_rt, S_rp, S_tp, with the same
-  // accessors in the same tiles), so they are S + those terms.
-  R srt = c.srt[t], srp = c.srp[t], stp = c.stp[t];
-  R ut = htc<CIJ>(g, c, UT, i, j, k), up = hpc<CIJ>(g, c, UP, i, j, k);
-  R xrt = srt + ut * ir, xrp = srp + up * ir, xtp = stp + up * g.cotc[j] * ir;
-  R cross = srt * xrt + srp * xrp + stp * xtp;
-  accp += -mu * (gm - R(1)) * cross;
-  accT += -mu * c.beta[t] * cross;
-  R Np = ap * divu + accp, NT = aT * divu + accT;
-  if (has_src) { Np -= to_bulk<R>(src.f[0][t]); NT -= to_bulk<R>(src.f[4][t]); }
-  R d0 = hasD ? D.f[0][t] : R(0), d4 = hasD ? D.f[4][t] : R(0);
-  Rout.f[0][t] = -d0 - tau * Np;
-  Rout.f[4][t] = -d4 - tau * NT;
-}
-
-// one block per tile
-template <typename R, bool W>
-__global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_c(Geo<R> g, Par P, Coef<R> c, CF<R> ub, CF<R> ul, CF<R> D,
-                                                                int hasD, CF<double> src, int has_src, R tau,
-                                                                MF<R> Rout) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
-      i = blockIdx.z * blockDim.z + threadIdx.z;
-  bool inner = tile_inner(g) && !g.hasw;  // with wall data every tile takes the checked path
-  if (k >= g.np || j >= g.nt || i >= g.nr) return;
-  int t = IC(g, i, j, k);
-  if (inner) rhs_c_at<0>(g, P, c, ub, ul, D, hasD, src, has_src, tau, Rout, i, j, k, t);
-  else rhs_c_at<W ? 2 : 1>(g, P, c, ub, ul, D, hasD, src, has_src, tau, Rout, i, j, k, t);
-}
-
-// R for the momentum row of component D on its faces: one thread per face
-// (zero on wall faces, which are not unknowns); written to Rout.f[1 + D][t].
-template <int CIJ, int D, typename R>
-__device__ __forceinline__ void rhs_u_at(const Geo<R>& g, const Par& P, const Coef<R>& c, const CF<R>& ub,
-                                         const CF<R>& Dv, int hasD, const CF<double>& src, int has_src, R tau,
-                                         const MF<R>& Rout, int i, int j, int k, int t) {
-  const auto Pp = ub.f[0];
-  const auto UR = ub.f[1];
-  const auto UT = ub.f[2];
-  const auto UP = ub.f[3];
-  R mu = pick<R>(P.mu, P.mu_f), om = pick<R>(P.omega, P.omega_f), h = R(0.5);
-  R wp[2], wu[3], w[3];
-  R acc;
-  if (D == 0) {
-    row_f(g, P, c, UR, 0, i, j, k, wp, wu);
-    acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i - 1, j, k))
-        + wu[0] * UR[IRf(g, i - 1, j, k)] + wu[1] * UR[t] + wu[2] * UR[IRf(g, i + 1, j, k)];
-    row_s<CIJ>(g, P, c, ub, 0, 1, i, j, k, w);
-    acc += w[0] * vr<CIJ>(g, UR, i, j - 1, k) + w[1] * UR[t] + w[2] * vr<CIJ>(g, UR, i, j + 1, k);
-    row_s<CIJ>(g, P, c, ub, 0, 2, i, j, k, w);
-    acc += w[0] * vr<CIJ>(g, UR, i, j, k - 1) + w[1] * UR[t] + w[2] * vr<CIJ>(g, UR, i, j, k + 1);
-    // hydrostatic part: (1/rho_f) d p_ref/dr + g = (1 - b) e + g b, b = 1 - rho_ref,f / rho_f
-    int c0 = IC(g, i - 1, j, k), c1 = IC(g, i, j, k);
-    R rs = c.rho[c0] + c.rho[c1];
-    R bf = sdiv(c.drho[c0] + c.drho[c1], rs);
-    acc += (R(1) - bf) * g.ehyd[i] + pick<R>(P.g, P.g_f) * bf;
-    // D_M
-    R irf = g.irf[i], s = g.sc[j];
-    R irh = sdiv(R(2), rs);
-    R utf = h * (htc<CIJ>(g, c, UT, i - 1, j, k) + htc<CIJ>(g, c, UT, i, j, k));
-    R upf = h * (hpc<CIJ>(g, c, UP, i - 1, j, k) + hpc<CIJ>(g, c, UP, i, j, k));
-    // theta and phi parts of div(Ubar) at the centres i - 1, i
-    R Q[2];
-#pragma unroll
-    for (int q = 0; q < 2; q++) {
-      int cm = IC(g, i - 1 + q, j, k);
-      Q[q] = c.dvt[cm] + c.dvp[cm];
-    }
-    acc += -utf * utf * irf - upf * upf * irf + R(2) * mu * irh * UR[t] * irf * irf - R(2) * om * s * upf
-         - mu * irh * R(1.0 / 3.0) * g.idr * (Q[1] - Q[0]) + mu * irh * irf * (Q[0] + Q[1]);
-  } else if (D == 1) {
-    R ir = g.irc[i];
-    row_f(g, P, c, UT, 1, i, j, k, wp, wu);
-    acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i, j - 1, k))
-        + wu[0] * UT[ITf(g, i, j - 1, k)] + wu[1] * UT[t] + wu[2] * UT[ITf(g, i, j + 1, k)];
-    row_s<CIJ>(g, P, c, ub, 1, 0, i, j, k, w);
-    acc += w[0] * vt<CIJ>(g, UT, i - 1, j, k) + w[1] * UT[t] + w[2] * vt<CIJ>(g, UT, i + 1, j, k);
-    row_s<CIJ>(g, P, c, ub, 1, 2, i, j, k, w);
-    acc += w[0] * vt<CIJ>(g, UT, i, j, k - 1) + w[1] * UT[t] + w[2] * vt<CIJ>(g, UT, i, j, k + 1);
-    R isfj = g.isf[j], cfj = g.cf[j], cotf = g.cotf[j];
-    R irh = sdiv(R(2), rho_at(g, c, i, j - 1, k) + rho_at(g, c, i, j, k));
-    R ubt = UT[t];
-    R upf = h * (hpc<CIJ>(g, c, UP, i, j - 1, k) + hpc<CIJ>(g, c, UP, i, j, k));
-    R vrf = h * (hrc<CIJ>(g, c, UR, i, j - 1, k) + hrc<CIJ>(g, c, UR, i, j, k));
-    // r and phi parts of div(Ubar) at the centres j - 1, j; dpf = the mean of
-    // their d_p u_p (the phi part times r sin)
-    R Dr[2], Dp[2], dpf = R(0);
-#pragma unroll
-    for (int q = 0; q < 2; q++) {
-      int m = j - 1 + q, cm = IC(g, i, m, k);
-      Dr[q] = c.dvr[cm];
-      Dp[q] = c.dvp[cm];
-      dpf += h * Dp[q] * g.rc[i] * g.sc[m];
-    }
-    acc += ubt * vrf * ir - upf * upf * cotf * ir + mu * irh * ubt * ir * ir * isfj * isfj - R(2) * om * cfj * upf
-         - mu * irh * R(1.0 / 3.0) * ir * g.idth * ((Dr[1] - Dr[0]) + (Dp[1] - Dp[0]))
-         - mu * irh * (R(2) * ir * ir * g.idth * (hrc<CIJ>(g, c, UR, i, j, k) - hrc<CIJ>(g, c, UR, i, j - 1, k))
-                       - R(2) * cfj * ir * ir * isfj * isfj * dpf);
-  } else {
-    R ir = g.irc[i], is = g.isc[j], cot = g.cotc[j];
-    row_f(g, P, c, UP, 2, i, j, k, wp, wu);
-    acc = wp[1] * (cpert<CIJ>(g, Pp, i, j, k) - cpert<CIJ>(g, Pp, i, j, k - 1))
-        + wu[0] * vp<CIJ>(g, UP, i, j, k - 1) + wu[1] * UP[t] + wu[2] * vp<CIJ>(g, UP, i, j, k + 1);
-    row_s<CIJ>(g, P, c, ub, 2, 0, i, j, k, w);
-    acc += w[0] * vp<CIJ>(g, UP, i - 1, j, k) + w[1] * UP[t] + w[2] * vp<CIJ>(g, UP, i + 1, j, k);
-    row_s<CIJ>(g, P, c, ub, 2, 1, i, j, k, w);
-    acc += w[0] * vp<CIJ>(g, UP, i, j - 1, k) + w[1] * UP[t] + w[2] * vp<CIJ>(g, UP, i, j + 1, k);
-    R s = g.sc[j], cj = g.cc[j];
-    R irh = sdiv(R(2), rho_at(g, c, i, j, k - 1) + rho_at(g, c, i, j, k));
-    R ubp = UP[t];
-    R vrf = h * (hrc<CIJ>(g, c, UR, i, j, k - 1) + hrc<CIJ>(g, c, UR, i, j, k));
-    R vtf = h * (htc<CIJ>(g, c, UT, i, j, k - 1) + htc<CIJ>(g, c, UT, i, j, k));
-    // r and theta parts of div(Ubar) at the centres k - 1, k (interior faces: real
-    // centres, wrapped on a periodic line)
-    R Dr[2], Dt[2];
-#pragma unroll
-    for (int q = 0; q < 2; q++) {
-      int m = k - 1 + q;
-      if (g.per) m = wrapk(g, m);
-      int cm = IC(g, i, j, m);
-      Dr[q] = c.dvr[cm];
-      Dt[q] = c.dvt[cm];
-    }
-    acc += ubp * vtf * cot * ir + ubp * vrf * ir + mu * irh * ubp * ir * ir * is * is + R(2) * om * (cj * vtf + s * vrf)
-         - mu * irh * R(1.0 / 3.0) * ir * is * g.idph * ((Dr[1] - Dr[0]) + (Dt[1] - Dt[0]))
-         - mu * irh * (R(2) * ir * ir * is * g.idph * (hrc<CIJ>(g, c, UR, i, j, k) - hrc<CIJ>(g, c, UR, i, j, k - 1))
-                       + R(2) * cj * ir * ir * is * is * g.idph * (htc<CIJ>(g, c, UT, i, j, k) - htc<CIJ>(g, c, UT, i, j, k - 1)));
-  }
-  if (has_src) acc -= to_bulk<R>(src.f[1 + D][t]);
-  R dd = hasD ? Dv.f[1 + D][t] : R(0);
-  Rout.f[1 + D][t] = -dd - tau * acc;
-}
-
-// one block per tile of faces; zero on wall faces, which are not unknowns
-template <typename R, int D, bool W>
-__global__ void __launch_bounds__(128, STENCIL_MINB(R)) k_rhs_u(Geo<R> g, Par P, Coef<R> c, CF<R> ub, CF<R> Dv, int hasD,
-                                               CF<double> src, int has_src, R tau, MF<R> Rout) {
-  int nj = g.nt + (D == 1), nk = D == 2 ? g.npf : g.np;
-  int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
-      i = blockIdx.z * blockDim.z + threadIdx.z;
-  bool inner = tile_inner(g) && !g.hasw;  // with wall data every tile takes the checked path
-  if (k >= nk || j >= nj || i >= g.nr + (D == 0)) return;
-  int t = (i * nj + j) * nk + k;
-  bool wall = D == 0 ? (i == 0 || i == g.nr) : D == 1 ? (j == 0 || j == g.nt) : (!g.per && (k == 0 || k == g.np));
-  if (wall) { Rout.f[1 + D][t] = R(0); return; }
-  if (inner) rhs_u_at<0, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
-  else rhs_u_at<W ? 2 : 1, D>(g, P, c, ub, Dv, hasD, src, has_src, tau, Rout, i, j, k, t);
-}
 
 // ------------------------------------------------------------ line solvers
 
