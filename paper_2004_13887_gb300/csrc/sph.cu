@@ -901,7 +901,7 @@ static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> 
   memset(&S, 0, sizeof S);
   S.g = b.g; S.P = c->P; S.c = b.c; S.ub = ub; S.d = d; S.h = (R)(0.5 * tau);
   S.rhs = rhs; S.x = x; S.update = update; S.base = base; S.uk = uk;
-  S.scr = b.scr; S.acc = c->acc; S.flag = c->flag;
+  S.scr = b.scr; S.acc = c->acc; S.norms = norms; S.flag = c->flag;
   line_layout(c->d64.g, d, S);
   if constexpr (sizeof(R) == sizeof(float)) {
     if (lines2_use(c, d)) {
@@ -915,6 +915,7 @@ static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> 
   }
   if (sizeof(R) == sizeof(float) && c->line_solver != SPH_LINES_THOMAS && lines_ok(c, d)) {
     SweepArgs<float>& Sf = *reinterpret_cast<SweepArgs<float>*>(&S);
+    lines2_rows(c, d, tau, &Sf);
     const Geo<double>& g = c->d64.g;
     int n = d == 0 ? g.nr : d == 1 ? g.nt : g.np;
     if (d == 0) return run_lines_d<0>(c, Sf, n);

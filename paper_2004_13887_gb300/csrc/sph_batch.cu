@@ -502,6 +502,8 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
           S.uk = mf5(c->U[1 - cur]);
           S.scr = B.scr; S.acc = c->acc; S.flag = c->flag;
           line_layout(g, d, S);
+          lines2_rows(c, d, dt, &S);
+          S.norms = 1;
           for (int k = 0; k < 3; k++) ng[k] = lines_groups(S, k, NW);
           T.ng1 = ng[1];
           ltab[li][p][it].push_back(T);

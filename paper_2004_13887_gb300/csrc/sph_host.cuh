@@ -135,6 +135,8 @@ void s32_rhs(sph_ctx* c, CF<float> ub, int hasD, double tau, CF<double> src, int
 size_t lines2_tab_floats(int nr, int nt);
 size_t lines2_scratch(const Geo<double>& g, int d);
 void lines2_tables(sph_ctx* c);
+// (the tables and constants of a direction's rows, for the partitioned solver too)
+void lines2_rows(const sph_ctx* c, int d, double tau, SweepArgs<float>* S);
 void lines2_fill(const sph_ctx* c, int d, double tau, CF<float> ub, CF<float> rhs, MF<float> x, lines2::Args* A, int* nblk,
                  int* nsca);
 void lines2_run(sph_ctx* c, int d, double tau, CF<float> ub, CF<float> rhs, MF<float> x, int update, int norms,

@@ -226,8 +226,13 @@ struct SweepArgs {
   int scr_off[3];         // offsets of the three kinds
   int nl[3];              // lines per kind
   int a0[3], nb[3], b0[3];
-  double* acc;            // 5 sums of squares (mode 1)
+  double* acc;            // 5 sums of squares (mode 1, when norms is set)
+  int norms;
   int* flag;
+  // FP32 lines: the tables of the direction's block and scalar lines
+  // (sph_lines2.cuh) and the constants their rows use
+  const float *tb, *ts[2];
+  float hgm, hgm1, hvp2, hmu2, gm1, iRg;
 };
 
 // Per-thread sums of squares of the increments, per field (the iteration
@@ -293,7 +298,7 @@ __device__ __forceinline__ void put(const SweepArgs<R>& A, int f, int idx, V v, 
     double nv = A.base.f[f][idx] + f2d(v);
     if (!isfinite(v)) *bad |= FLAG_NONFINITE;  // the state was finite; only a non-finite increment spoils it
     A.uk.f[f][idx] = nv;
-    ss.add(f, (R)v);
+    if (A.norms) ss.add(f, (R)v);
   }
 }
 // the update-mode store with the FP64 state value already loaded
@@ -301,7 +306,7 @@ template <typename R, typename V, typename Acc>
 __device__ __forceinline__ void put_upd(const SweepArgs<R>& A, int f, int idx, double base, V v, Acc& ss, int* bad) {
   if (!isfinite(v)) *bad |= FLAG_NONFINITE;
   A.uk.f[f][idx] = base + f2d(v);
-  ss.add(f, (R)v);
+  if (A.norms) ss.add(f, (R)v);
 }
 // wall face of field f: x = 0, or uk = base (mode 1)
 template <typename R>
@@ -713,7 +718,7 @@ __global__ void __launch_bounds__(128) k_sweep(SweepArgs<R> S) {
     else scalar_line<R, D, 2, TR>(S, line, a, b, ss, &bad);
   }
   if (bad) atomicOr(S.flag, bad);
-  if (S.update) {
+  if (S.update && S.norms) {
     for (int f = 0; f < 5; f++) {
       double v = ss.warp_total(f);
       if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(S.acc + f, v);

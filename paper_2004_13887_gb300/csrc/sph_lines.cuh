@@ -39,7 +39,17 @@
 // are read back within microseconds, so they are served by L2, and once the
 // back substitution is done the slot's cache lines are discarded from L2
 // (discard.global.L2) so that the dead factors are never written to DRAM.
+//
+// Bound by instruction issue and the elimination chain at 16 warps per SM (128
+// registers), with DRAM at a quarter of its rate.  So a block line's rows come
+// from lines2::form's tables (one record of 3 float4 a row, the parameters
+// already multiplied together) instead of products formed from the grid and
+// the parameters per cell, and the sums of squared increments are taken in a
+// step's last iteration alone, which is the one that is read: phi sweep of 128
+// x 256 x 256 528 -> 470 us, all three of 16 x 64 x 64 51 -> 43 us.
 #pragma once
+
+#include "sph_lines2.cuh"
 
 namespace lines {
 
@@ -181,8 +191,9 @@ __device__ __forceinline__ void normalise3(const float* A, const float* B, const
 // the rows of lanes l -+ s:
 //   B = I - A C_lo - C A_up,  A' = -A A_lo,  C' = -C C_up,
 //   r' = r - A r_lo - C r_up,
-// then renormalises; a missing neighbour (end of a non-cyclic line) is a zero
-// row.  After strides 1, 2, .., L/4 every row couples only to the row of lane
+// then renormalises.  Beyond the end of a non-cyclic line A (C) is zero in every
+// step -- the first lane's row has none, and A' = -A A_lo -- so the wrapped row
+// that the exchange brings there drops out.  After strides 1, 2, .., L/4 every row couples only to the row of lane
 // l ^ L/2 (both sides of a cyclic line meet there; on a non-cyclic line one of
 // A, C is zero):  x + M x_p = r,  x_p + M_p x = r_p  =>  (I - M M_p) x = r - M r_p.
 template <int L>
@@ -190,7 +201,7 @@ __device__ __forceinline__ void pcr3(float* X, int lane, int cyc, float* x, int*
 #pragma unroll 1
   for (int s = 1; s < L / 2; s <<= 1) {
     float o[NR3], A[9], B[9], C[9], r[3], t[9], u[3];
-    xget<NR3, L>(X, o, (lane - s) & (L - 1), !cyc && lane < s, xb);
+    xget<NR3, L>(X, o, (lane - s) & (L - 1), false, xb);
     mm3(X, o + 9, t);
 #pragma unroll
     for (int q = 0; q < 9; q++) B[q] = (q % 4 == 0 ? 1.f : 0.f) - t[q];
@@ -200,7 +211,7 @@ __device__ __forceinline__ void pcr3(float* X, int lane, int cyc, float* x, int*
     mv3(X, o + 18, u);
 #pragma unroll
     for (int q = 0; q < 3; q++) r[q] = X[18 + q] - u[q];
-    xget<NR3, L>(X, o, (lane + s) & (L - 1), !cyc && lane + s > L - 1, xb);
+    xget<NR3, L>(X, o, (lane + s) & (L - 1), false, xb);
     mm3(X + 9, o, t);
 #pragma unroll
     for (int q = 0; q < 9; q++) B[q] -= t[q];
@@ -235,8 +246,8 @@ __device__ __forceinline__ float pcr1(float a, float c, float r, int lane, int c
 #pragma unroll 1
   for (int s = 1; s < L / 2; s <<= 1) {
     float v[3] = {a, c, r}, lv[3], uv[3];
-    xget<3, L>(v, lv, (lane - s) & (L - 1), !cyc && lane < s, xb);
-    xget<3, L>(v, uv, (lane + s) & (L - 1), !cyc && lane + s > L - 1, xb);
+    xget<3, L>(v, lv, (lane - s) & (L - 1), false, xb);
+    xget<3, L>(v, uv, (lane + s) & (L - 1), false, xb);
     float la = lv[0], lc = lv[1], lr = lv[2], ua = uv[0], uc = uv[1], ur = uv[2];
     float b = 1.f - a * lc - c * ua;
     if (b == 0.f || !isfinite(b)) *bad |= FLAG_SINGULAR;
@@ -345,7 +356,7 @@ __device__ __forceinline__ Group group_of(const SweepArgs<float>& S, int kind, i
 template <typename Acc>
 __device__ __forceinline__ void flush_norms(const SweepArgs<float>& S, const Acc& ss, int bad) {
   if (bad) atomicOr(S.flag, bad);
-  if (S.update) {
+  if (S.update && S.norms) {
 #pragma unroll
     for (int f = 0; f < 5; f++) {
       double v = ss.warp_total(f);
@@ -354,7 +365,6 @@ __device__ __forceinline__ void flush_norms(const SweepArgs<float>& S, const Acc
   }
 }
 
-// ------------------------------------------------------------------ kernels
 // ------------------------------------------------------------------ kernels
 
 // Block lines (p, T, u_D) of direction D, n = L P cells per line, L lanes per
@@ -369,7 +379,6 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
   const int n = SH::n, cyc = (D == 2 && g.per);
   const int wid = threadIdx.x >> 5, wl = threadIdx.x & 31;  // warp, lane of the warp
   const int w = threadIdx.x / L, lane = threadIdx.x % L;    // block line, lane of the line
-  const float h = S.h;
   SqSum<float> ss;
   int bad = 0;
   float* slot = S.scr + ((size_t)grp * SH::NWW + wid) * (32 * slot_floats(P));
@@ -407,39 +416,50 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
         uf = S.ub.f[1 + D][face_idx(g, D, i, j, k)];
       }
     }
-    Thermo<float> th;
+    lines2::Th th;
     {
       int i, j, k, m0 = lane * P, s0 = sidx<P, L, CB>(w, m0);
       line_pos(D, a, b, m0, i, j, k);
-      th = thermo(g, S.P, i, sm[s0], sm[FS + s0]);
+      th = lines2::thermo(S, i, sm[s0], sm[FS + s0]);
     }
 #pragma unroll 1
     for (int t = 0; t < P; t++) {
       int m = lane * P + t;
       int si = sidx<P, L, CB>(w, m);
-      int i, j, k, fi, fj, fk;
+      int i, j, k;
       line_pos(D, a, b, m, i, j, k);
-      next_face(D, n, cyc, m, i, j, k, fi, fj, fk);
-      float ufn = sm[7 * FS + si];
-      CPt<float> cq;
-      cq.Pb = th.Pb; cq.Tb = th.Tb; cq.beta = th.beta;
-      cq.uc = 0.5f * (uf + ufn);
-      cq.grr = sm[2 * FS + si]; cq.gtt = sm[3 * FS + si]; cq.gpp = sm[4 * FS + si];
-      cq.s1 = D > 0 ? sm[5 * FS + si] : 0.f;
-      cq.s2 = D > 0 ? sm[6 * FS + si] : 0.f;
-      FPt<float> fq = {th.rho, 1.f, ufn};
-      if (m < n - 1 || cyc) {
+      const float4* tb = reinterpret_cast<const float4*>(S.tb + (size_t)lines2::NB * (D == 0 ? i : i * g.nt + j));
+      const float4 q0 = tb[0], q1 = tb[1], q2 = tb[2];
+      const float ufn = sm[7 * FS + si];
+      const lines2::Th t0 = th;
+      const bool face = m < n - 1 || cyc;
+      if (face) {
         // the next cell along the line: its thermodynamics serve this face row and the next step
         int mn = m + 1 == n ? 0 : m + 1, sn = sidx<P, L, CB>(w, mn);
         int in_, jn, kn;
         line_pos(D, a, b, mn, in_, jn, kn);
-        th = thermo(g, S.P, in_, sm[sn], sm[FS + sn]);
-        fq.rho1 = th.rho;
+        th = lines2::thermo(S, in_, sm[sn], sm[FS + sn]);
       }
-      uf = ufn;
       float rr[3] = {sm[8 * FS + si], sm[9 * FS + si], sm[10 * FS + si]};
       float A[9], B[9], C[9];
-      assemble_pts(g, S.P, cq, fq, D, n, cyc, m, i, j, fi, fj, h, A, B, C);
+      lines2::form<D>(S, q0, q1, q2, t0, th.rho, face, uf, ufn, sm[2 * FS + si], sm[3 * FS + si], sm[4 * FS + si],
+                      D > 0 ? sm[5 * FS + si] : 0.f, D > 1 ? sm[6 * FS + si] : 0.f, A, B, C);
+      A[3] = A[6] = A[7] = 0.f;
+      C[2] = C[3] = C[5] = C[7] = 0.f;
+      if (!cyc && (m == 0 || m == n - 1)) {   // zero-gradient ghosts of p and T
+        if (m == 0) {
+          B[0] += A[0]; B[1] += A[1]; B[4] += A[4];
+#pragma unroll
+          for (int q = 0; q < 9; q++) A[q] = 0.f;
+        }
+        if (m == n - 1) {
+          B[0] += C[0]; B[1] += C[1]; B[4] += C[4];
+#pragma unroll
+          for (int q = 0; q < 9; q++) C[q] = 0.f;
+          B[2] = B[5] = 0.f;
+        }
+      }
+      uf = ufn;
       if (t < P - 1) {
         float Sm[9], rv[3], Hs[9], Si[9];
         if (t == 0) {
@@ -678,13 +698,13 @@ __device__ __forceinline__ void lines_sca(const SweepArgs<float>& S, int grp) {
     for (int t = 0; t < P; t++) {
       int m = lane * P + t;
       int si = sidx<P, L, CB>(w, m);
-      SPt<float> q = {sm[si], sm[FS + si], 0.5f * (sm[2 * FS + si] + sm[3 * FS + si])};
       float r = sm[4 * FS + si];
       int i, j, k;
       line_pos(D, a, b, m, i, j, k);
-      float wt[3];
-      row_sw(g, S.P, q, cc, D, i, j, wt);
-      float am = h * wt[0], bm = 1.f + h * wt[1], cm = h * wt[2];
+      const float4 wt = reinterpret_cast<const float4*>(S.ts[KIND - 1])[D == 0 ? i : D == 2 && KIND == 2 ? i * (g.nt + 1) + j
+                                                                                                        : i * g.nt + j];
+      const float hv = __fdividef(h, sm[si] + sm[FS + si]), adv = h * (sm[2 * FS + si] + sm[3 * FS + si]) * wt.w;
+      float am = fmaf(hv, wt.x, -adv), bm = fmaf(hv, wt.y, 1.f), cm = fmaf(hv, wt.z, adv);
       if (!cyc) {
         if (m == 0) { bm -= am; am = 0.f; }
         if (m == n - 1) { bm -= cm; cm = 0.f; }

@@ -41,6 +41,15 @@ size_t lines2_scratch(const Geo<double>& g, int d) {
          ((cyc ? 21 : 12) * (size_t)nb[0] + (cyc ? 3 : 2) * (size_t)(nb[1] + nb[2]));
 }
 
+void lines2_rows(const sph_ctx* c, int d, double tau, SweepArgs<float>* S) {
+  const lines2::Tabs T = tabs(c);
+  const double h = 0.5 * tau, gm = c->P.gamma, mu = c->P.mu;
+  S->tb = T.b[d];
+  S->ts[0] = T.s[d][0]; S->ts[1] = T.s[d][1];
+  S->hgm = (float)(h * gm); S->hgm1 = (float)(h * (gm - 1.0)); S->hvp2 = (float)(h * 2.0 * mu * (gm - 1.0));
+  S->hmu2 = (float)(h * 2.0 * mu); S->gm1 = (float)(gm - 1.0); S->iRg = c->P.iRg_f;
+}
+
 void lines2_fill(const sph_ctx* c, int d, double tau, CF<float> ub, CF<float> rhs, MF<float> x, lines2::Args* A, int* nblk,
                  int* nsca) {
   int nb[3];

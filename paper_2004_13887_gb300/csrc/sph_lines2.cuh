@@ -89,7 +89,8 @@ template <int D> __device__ __forceinline__ int fx_of(const Geo<float>& g, int a
 }
 
 struct Th { float Pb, Tb, rho, be; };
-__device__ __forceinline__ Th thermo(const Args& A, int i, float pp, float Tp) {
+template <typename Consts>
+__device__ __forceinline__ Th thermo(const Consts& A, int i, float pp, float Tp) {
   Th t;
   t.Pb = A.g.pcen[i] + pp;
   t.Tb = A.g.Tcen[i] + Tp;
@@ -102,8 +103,8 @@ __device__ __forceinline__ Th thermo(const Args& A, int i, float pp, float Tp) {
 // its thermodynamics; rho1: the density beyond face m + 1, when it has that face
 // as an unknown (face); ulo, uhi: Ubar's u_D on its faces; the gradients; s1, s2:
 // the cross sums).
-template <int D>
-__device__ __forceinline__ void form(const Args& A, const float4& q0, const float4& q1, const float4& q2, const Th& th,
+template <int D, typename Consts>
+__device__ __forceinline__ void form(const Consts& A, const float4& q0, const float4& q1, const float4& q2, const Th& th,
                                      float rho1, bool face, float ulo, float uhi, float grr, float gtt, float gpp, float s1,
                                      float s2, float* Ab, float* Bb, float* Cb) {
   const float G0 = q0.x, G1 = q0.y, K0 = q0.z, K1 = q0.w, LIN = q1.x, COT2 = q1.y, MD = q1.z, HM = q1.w, WP = q2.x,
