@@ -34,11 +34,12 @@ struct Tile { int tk, tj, ti, gx, gy, n; };
 
 // Consecutive tiles of one problem a block of a stencil launch takes (one
 // descriptor load for all of them), and the blocks per SM the coefficient and
-// centre-row kernels are compiled for (48 and 64 registers a thread): the
+// right-hand-side kernels are compiled for (48 and 72 registers a thread): the
 // descriptor in shared memory costs registers that at the single-problem
-// kernels' 32 spill heavily.  Measured on the 64-instance ensemble (ms per
-// step): 1 tile at 32 registers 49.1, 4 tiles 49.4, 4 tiles at 48/64
-// registers 45.8, 8 tiles at 48/64 45.5.
+// kernels' 40 and 56 spill.  Measured, ms a step of the 64-instance ensemble: 1 tile
+// 49.1, 4 tiles 45.8, 8 tiles 45.5; right-hand side, ms a pass of 12 problems: 4
+// blocks 16.25, 5 16.00, 6 15.67, 7 15.62, 8 15.75, 9 16.20 (four launches' worth
+// of rows in one, a thread a row: 16.96).
 #ifndef FUSED_TILES
 #define FUSED_TILES 8
 #endif
@@ -47,17 +48,12 @@ constexpr int TILES = FUSED_TILES;
 #define FUSED_MINB_COEF 10
 #endif
 #ifndef FUSED_MINB_RHS
-#define FUSED_MINB_RHS 10
+#define FUSED_MINB_RHS 7
 #endif
 
-struct CoefTab {
+struct StenTab {   // a stencil stage of a problem
   s32::Args A;
   Tile t;
-};
-
-struct RhsTab {
-  s32::Args A;
-  Tile t[4];  // centres (p, T rows), then the faces of u_r, u_theta, u_phi
 };
 
 struct LineTab {
@@ -123,8 +119,8 @@ __global__ void __launch_bounds__(256) k_avg_f(const AvgArgs<float>* tab, const 
 }
 
 // the coefficient stage over the tiles of every problem
-__global__ void __launch_bounds__(128, FUSED_MINB_COEF) k_coef_f(const CoefTab* tab, const int2* map) {
-  __shared__ CoefTab S;
+__global__ void __launch_bounds__(128, FUSED_MINB_COEF) k_coef_f(const StenTab* tab, const int2* map) {
+  __shared__ StenTab S;
   const int2 m = map[blockIdx.x];
   load_args(S, tab[m.x]);
   const Geo<float>& g = S.A.g;
@@ -133,24 +129,22 @@ __global__ void __launch_bounds__(128, FUSED_MINB_COEF) k_coef_f(const CoefTab* 
     const Pt p = point_of(S.t, b);
     const bool inner = tile_inner_at(g, p.i0, p.j0, S.t.ti, S.t.tj);
     if (p.k >= g.np || p.j >= g.nt || p.i >= g.nr) continue;
-    const int t = IC(g, p.i, p.j, p.k);
-    if (inner) s32::coef<0>(S.A, p.i, p.j, p.k, t);
-    else s32::coef<1>(S.A, p.i, p.j, p.k, t);
+    const s32::Loc L = s32::loc_of(g, p.i, p.j, p.k);
+    if (inner) s32::coef<0>(S.A, L);
+    else s32::coef<1>(S.A, L);
   }
 }
 
-// the right-hand side over every problem: map = (problem, kind * 2^28 + first tile),
-// the tiles of a problem's four kinds one after another
-__global__ void __launch_bounds__(128, FUSED_MINB_RHS) k_rhs_f(const RhsTab* tab, const int2* map) {
-  __shared__ RhsTab S;
+// the right-hand side over the tiles of every problem
+__global__ void __launch_bounds__(128, FUSED_MINB_RHS) k_rhs_f(const StenTab* tab, const int2* map) {
+  __shared__ StenTab S;
+  __shared__ float own[s32::NO][128];
   const int2 m = map[blockIdx.x];
   load_args(S, tab[m.x]);
-  const int kind = m.y >> 28, b0 = m.y & 0xfffffff;
-  const Tile& tl = S.t[kind];
-  const int b1 = min(b0 + TILES, tl.n);
-  for (int b = b0; b < b1; b++) {
-    const Pt p = point_of(tl, b);
-    s32::rhs_point<false>(S.A, kind, p.i, p.j, p.k, tile_inner_at(S.A.g, p.i0, p.j0, tl.ti, tl.tj));
+  const int b1 = min(m.y + TILES, S.t.n);
+  for (int b = m.y; b < b1; b++) {
+    const Pt p = point_of(S.t, b);
+    s32::rhs_cell<false>(S.A, p.i, p.j, p.k, tile_inner_at(S.A.g, p.i0, p.j0, S.t.ti, S.t.tj), &own[0][threadIdx.x]);
   }
 }
 
@@ -381,9 +375,9 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
   std::vector<AvgArgs<float>> avg[2][2];
   std::vector<int4> mavg;
   // ---- stencil stages
-  std::vector<fused::CoefTab> coef(n);
-  std::vector<fused::RhsTab> rhs[2][2];
-  std::vector<int2> mcoef, mrhs;
+  std::vector<fused::StenTab> coef(n);
+  std::vector<fused::StenTab> rhs[2][2];
+  std::vector<int2> msten;
   std::vector<double*> accs(n);
   for (int p = 0; p < 2; p++)
     for (int it = 0; it < 2; it++) {
@@ -407,29 +401,21 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
           A.a[f] = un[f]; A.b[f] = uk[f]; A.o[f] = B.Ub[f]; A.lo[f] = B.UbLo[f]; A.d[f] = B.Db[f];
           A.n[f] = (long)c->nf[f];
         }
-        fused::RhsTab& R = rhs[p][it][q];
+        fused::StenTab& R = rhs[p][it][q];
         memset(&R, 0, sizeof R);
         s32_fill(c, cf5(B.Ub), dt, &R.A);
         R.A.hasD = it;
       }
-    int nb[5];
-    fused::Tile tc = tile_of(c, g.np, g.nt, g.nr, &nb[0]);
-    fused::Tile tu[3] = {tile_of(c, g.np, g.nt, g.nr + 1, &nb[1]), tile_of(c, g.np, g.nt + 1, g.nr, &nb[2]),
-                         tile_of(c, g.npf, g.nt, g.nr, &nb[3])};
-    fused::CoefTab& C = coef[q];
+    int nb;
+    fused::Tile tc = tile_of(c, g.np, g.nt, g.nr, &nb);
+    fused::StenTab& C = coef[q];
     memset(&C, 0, sizeof C);
     s32_fill(c, cf5(B.Ub), dt, &C.A);
     C.t = tc;
     for (int p = 0; p < 2; p++)
-      for (int it = 0; it < 2; it++) {
-        fused::RhsTab& R = rhs[p][it][q];
-        R.t[0] = tc;
-        for (int d = 0; d < 3; d++) R.t[1 + d] = tu[d];
-      }
+      for (int it = 0; it < 2; it++) rhs[p][it][q].t = tc;
     // a block per fused::TILES consecutive tiles of the problem
-    for (int k = 0; k < nb[0]; k += fused::TILES) mcoef.push_back(make_int2(q, k));
-    for (int d = 0; d < 4; d++)
-      for (int k = 0; k < nb[d]; k += fused::TILES) mrhs.push_back(make_int2(q, (d << 28) + k));
+    for (int k = 0; k < nb; k += fused::TILES) msten.push_back(make_int2(q, k));
     for (int f = 0; f < 5; f++) {
       const long pairs = (long)c->nf[f] >> 1;
       for (long s = 0; s < pairs || (s == 0 && pairs == 0); s += 1024)
@@ -520,8 +506,7 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
       oavg[p][it] = blob.put(avg[p][it]);
       orhs[p][it] = blob.put(rhs[p][it]);
     }
-  const size_t ocoef = blob.put(coef), omavg = blob.put(mavg), omcoef = blob.put(mcoef), oacc = blob.put(accs);
-  const size_t omrhs = blob.put(mrhs);
+  const size_t ocoef = blob.put(coef), omavg = blob.put(mavg), omsten = blob.put(msten), oacc = blob.put(accs);
   size_t ol2[2], ol2b[2], ol2s[2];
   for (int d = 0; d < 2; d++) { ol2[d] = blob.put(l2tab[d]); ol2b[d] = blob.put(l2b[d]); ol2s[d] = blob.put(l2s[d]); }
   for (size_t z = 0; z < lay.size(); z++) {
@@ -548,11 +533,11 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
       const int il = it > 0;
       fused::k_avg_f<<<(unsigned)mavg.size(), 256, 0, b->st>>>((const AvgArgs<float>*)(base + oavg[p][il]),
                                                                (const int4*)(base + omavg));
-      fused::k_coef_f<<<(unsigned)mcoef.size(), 128, 0, b->st>>>((const fused::CoefTab*)(base + ocoef),
-                                                                (const int2*)(base + omcoef));
+      fused::k_coef_f<<<(unsigned)msten.size(), 128, 0, b->st>>>((const fused::StenTab*)(base + ocoef),
+                                                                (const int2*)(base + omsten));
       nk += 2;
-      const fused::RhsTab* rt = (const fused::RhsTab*)(base + orhs[p][il]);
-      fused::k_rhs_f<<<(unsigned)mrhs.size(), 128, 0, b->st>>>(rt, (const int2*)(base + omrhs));
+      const fused::StenTab* rt = (const fused::StenTab*)(base + orhs[p][il]);
+      fused::k_rhs_f<<<(unsigned)msten.size(), 128, 0, b->st>>>(rt, (const int2*)(base + omsten));
       nk++;
       for (int d = 0; d < 3 && !err; d++) {
         if (d == 2 && it == n_iter - 1) {

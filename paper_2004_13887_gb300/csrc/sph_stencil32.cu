@@ -45,23 +45,24 @@ __global__ void k_pack(Geo<double> g, f64::Tabs S, Tabs T) {
 }
 
 template <bool W>
-__global__ void __launch_bounds__(128, 16) k_coef(const __grid_constant__ Args A) {
+__global__ void __launch_bounds__(128, 12) k_coef(const __grid_constant__ Args A) {
   const Geo<float>& g = A.g;
   const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y,
             i = blockIdx.z * blockDim.z + threadIdx.z;
   const bool inner = !W && tile_inner(g);   // with wall data every tile takes the checked path
   if (k >= g.np || j >= g.nt || i >= g.nr) return;
-  const int t = IC(g, i, j, k);
-  if (inner) coef<0>(A, i, j, k, t);
-  else coef<W ? 2 : 1>(A, i, j, k, t);
+  const Loc L = loc_of(g, i, j, k);
+  if (inner) coef<0>(A, L);
+  else coef<W ? 2 : 1>(A, L);
 }
 
-// the rows of one kind: 0 the centres, 1 + C the faces of component C
-template <bool W, int KIND>
-__global__ void __launch_bounds__(128, 16) k_rhs(const __grid_constant__ Args A) {
+template <bool W>
+__global__ void __launch_bounds__(128, 9) k_rhs(const __grid_constant__ Args A) {
+  __shared__ float own[NO][128];
   const int i0 = blockIdx.z * blockDim.z, j0 = blockIdx.y * blockDim.y;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x, j = j0 + threadIdx.y, i = i0 + threadIdx.z;
-  rhs_point<W>(A, KIND, i, j, k, !W && tile_inner_at(A.g, i0, j0, (int)blockDim.z, (int)blockDim.y));
+  float* sh = &own[0][(threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x];
+  rhs_cell<W>(A, i0 + threadIdx.z, j0 + threadIdx.y, blockIdx.x * blockDim.x + threadIdx.x,
+              !W && tile_inner_at(A.g, i0, j0, (int)blockDim.z, (int)blockDim.y), sh);
 }
 
 }  // namespace s32
@@ -92,21 +93,13 @@ void s32_coef(sph_ctx* c, CF<float> ub, int thermo) {
   else s32::k_coef<false><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
 }
 
-template <bool W>
-static void launch_rhs(sph_ctx* c, const s32::Args& A) {
-  const Geo<double>& g = c->d64.g;
-  s32::k_rhs<W, 0><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
-  s32::k_rhs<W, 1><<<tile_grid(g.np, g.nt, g.nr + 1), TILE_BLOCK, 0, c->aux[0]>>>(A);
-  s32::k_rhs<W, 2><<<tile_grid(g.np, g.nt + 1, g.nr), TILE_BLOCK, 0, c->aux[1]>>>(A);
-  s32::k_rhs<W, 3><<<tile_grid(g.npf, g.nt, g.nr), TILE_BLOCK, 0, c->aux[2]>>>(A);
-}
-
 void s32_rhs(sph_ctx* c, CF<float> ub, int hasD, double tau, CF<double> src, int has_src, MF<float> R) {
   s32::Args A;
   s32_fill(c, ub, tau, &A);
   A.hasD = hasD; A.src = src; A.has_src = has_src; A.R = R;
-  if (c->d32.g.hasw) launch_rhs<true>(c, A);
-  else launch_rhs<false>(c, A);
+  const Geo<double>& g = c->d64.g;
+  if (c->d32.g.hasw) s32::k_rhs<true><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
+  else s32::k_rhs<false><<<tile_grid(g.np, g.nt, g.nr), TILE_BLOCK, 0, c->st>>>(A);
 }
 
 #ifdef SPH_CHECKED
