@@ -292,6 +292,8 @@ class Solver:
                 keep.append(a)
                 ptrs[(c * 3 + d) * 2 + s] = ptr
             arrs.append((_DP * 18)(*ptrs))
+        if dev:
+            self._after_caller()
         _check(load().sph_set_bc(self._h, arrs[0], arrs[1], int(bool(dev))), "sph_set_bc")
 
     # The library works on the solver's stream.  Device arrays handed in were

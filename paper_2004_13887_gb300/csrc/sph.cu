@@ -510,27 +510,56 @@ extern "C" int sph_set_iterate(sph_ctx* c, const double* const* fields, int on_d
   return e;
 }
 
-extern "C" int sph_set_bc(sph_ctx* c, const double* const* wn, const double* const* wnp1, int on_device) {
-  if (!c) return SPH_ERR_ARG;
-  const Geo<double>& g = c->d64.g;
-  if (cudaStreamSynchronize(c->st) != cudaSuccess) return SPH_ERR_CUDA;  // steps in flight read the old data
-  int any = 0;
-  size_t tot = 0;
-  for (int q = 0; q < 18; q++) {
-    int cc = q / 6, d = (q / 2) % 3;
-    int given = (wn && wn[q]) || (wnp1 && wnp1[q]);
-    if (d == 2 && g.per) given = 0;  // no phi walls on a periodic line
-    c->wset[q] = given;
-    c->woff[q] = tot;
-    if (given) { tot += wall_count(g, cc, d); any = 1; }
+// The means of the t^n and t^{n+1} wall values and the latter, from the caller's
+// device arrays (NULL: zero): one launch for all 18 arrays in place of a copy of
+// each to the host, the sums there and three copies back (14 x 45 x 135 cells, moving
+// walls, FP64: 1791 -> 1262 us a step with its call).
+struct WallArgs {
+  const double *a[18], *b[18];
+  unsigned off[19];
+  double *mean, *next;
+  float* mean32;         // NULL in FP64 mode
+};
+static __global__ void k_walls(const __grid_constant__ WallArgs A) {
+  const int q = blockIdx.y;
+  const unsigned n = A.off[q + 1] - A.off[q];
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const double a = A.a[q] ? A.a[q][t] : 0.0, b = A.b[q] ? A.b[q][t] : 0.0;
+    const double m = 0.5 * a + 0.5 * b;
+    A.mean[A.off[q] + t] = m;
+    A.next[A.off[q] + t] = b;
+    if (A.mean32) A.mean32[A.off[q] + t] = (float)m;
   }
-  for (int q = 0; q < 18; q++) { c->d64.g.w[q] = c->wzero64; c->d32.g.w[q] = c->wzero32; }
-  c->d64.g.hasw = c->d32.g.hasw = 0;
-  c->hasbc = 0;
+}
+
+// whether a kernel on the context's device may read p (memory of another device,
+// or of the host, takes the way through the host)
+static bool readable_here(const sph_ctx* c, const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+  return a.type == cudaMemoryTypeDevice && a.device == c->dev;
+}
+
+// the wall buffers for tot values, kept from call to call while they are large enough
+static int wall_alloc(sph_ctx* c, size_t tot) {
+  if (c->wcap >= tot) return SPH_OK;
   cudaFree(c->wmean64); cudaFree(c->wmean32); cudaFree(c->wnext);
   c->wmean64 = NULL; c->wmean32 = NULL; c->wnext = NULL;
-  c->wtot = tot;
-  if (!any) return SPH_OK;
+  c->wcap = 0;
+  if (cudaMalloc((void**)&c->wmean64, tot * sizeof(double)) != cudaSuccess ||
+      cudaMalloc((void**)&c->wnext, tot * sizeof(double)) != cudaSuccess ||
+      (c->prec == SPH_PREC_MIXED && cudaMalloc((void**)&c->wmean32, tot * sizeof(float)) != cudaSuccess)) {
+    cudaGetLastError();
+    return SPH_ERR_NOMEM;
+  }
+  c->wcap = tot;
+  return SPH_OK;
+}
+
+// the way through the host: arrays in host memory, or not readable from a kernel
+static int walls_by_host(sph_ctx* c, const double* const* wn, const double* const* wnp1, int on_device) {
+  const Geo<double>& g = c->d64.g;
+  const size_t tot = c->wtot;
   double* hm = (double*)calloc(tot, sizeof(double));
   double* hn = (double*)calloc(tot, sizeof(double));
   float* hf = (float*)calloc(tot, sizeof(float));
@@ -553,15 +582,63 @@ extern "C" int sph_set_bc(sph_ctx* c, const double* const* wn, const double* con
     }
     for (size_t t = 0; t < n; t++) hf[o + t] = (float)hm[o + t];
   }
-  if (!e && (cudaMalloc((void**)&c->wmean64, tot * sizeof(double)) != cudaSuccess ||
-             cudaMalloc((void**)&c->wnext, tot * sizeof(double)) != cudaSuccess ||
-             (c->prec == SPH_PREC_MIXED && cudaMalloc((void**)&c->wmean32, tot * sizeof(float)) != cudaSuccess)))
-    e = SPH_ERR_NOMEM;
   if (!e && (cudaMemcpy(c->wmean64, hm, tot * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
              cudaMemcpy(c->wnext, hn, tot * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
              (c->wmean32 && cudaMemcpy(c->wmean32, hf, tot * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)))
     e = SPH_ERR_CUDA;
   free(hm); free(hn); free(hf); free(tmp);
+  return e;
+}
+
+// arrays of this device: read on the context's stream, after what the legacy
+// default stream holds (a copy to the host waited for that, too); done on return
+static int walls_by_kernel(sph_ctx* c, const double* const* wn, const double* const* wnp1) {
+  WallArgs A;
+  memset(&A, 0, sizeof A);
+  unsigned mx = 0;
+  for (int q = 0; q < 18; q++) {
+    if (c->wset[q]) { A.a[q] = wn ? wn[q] : NULL; A.b[q] = wnp1 ? wnp1[q] : NULL; }
+    A.off[q] = (unsigned)c->woff[q];
+    const unsigned end = (unsigned)(q < 17 ? c->woff[q + 1] : c->wtot);
+    if (end - A.off[q] > mx) mx = end - A.off[q];
+  }
+  A.off[18] = (unsigned)c->wtot;
+  A.mean = c->wmean64; A.next = c->wnext; A.mean32 = c->wmean32;
+  if (cudaEventRecord(c->efork, cudaStreamLegacy) != cudaSuccess || cudaStreamWaitEvent(c->st, c->efork, 0) != cudaSuccess)
+    return SPH_ERR_CUDA;
+  const unsigned nb = (mx + 255) / 256;
+  k_walls<<<dim3(nb < 1024 ? nb : 1024, 18), 256, 0, c->st>>>(A);
+  c->launches++;
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->st) != cudaSuccess) return SPH_ERR_CUDA;
+  return SPH_OK;
+}
+
+extern "C" int sph_set_bc(sph_ctx* c, const double* const* wn, const double* const* wnp1, int on_device) {
+  if (!c) return SPH_ERR_ARG;
+  const Geo<double>& g = c->d64.g;
+  if (cudaStreamSynchronize(c->st) != cudaSuccess) return SPH_ERR_CUDA;  // steps in flight read the old data
+  int any = 0;
+  bool here = on_device != 0;
+  size_t tot = 0;
+  for (int q = 0; q < 18; q++) {
+    int cc = q / 6, d = (q / 2) % 3;
+    int given = (wn && wn[q]) || (wnp1 && wnp1[q]);
+    if (d == 2 && g.per) given = 0;  // no phi walls on a periodic line
+    c->wset[q] = given;
+    c->woff[q] = tot;
+    if (!given) continue;
+    tot += wall_count(g, cc, d);
+    any = 1;
+    if (here && wn && wn[q]) here = readable_here(c, wn[q]);
+    if (here && wnp1 && wnp1[q]) here = readable_here(c, wnp1[q]);
+  }
+  for (int q = 0; q < 18; q++) { c->d64.g.w[q] = c->wzero64; c->d32.g.w[q] = c->wzero32; }
+  c->d64.g.hasw = c->d32.g.hasw = 0;
+  c->hasbc = 0;
+  c->wtot = tot;
+  if (!any) return SPH_OK;
+  int e = wall_alloc(c, tot);
+  if (!e) e = here && tot < 0xffffffffu ? walls_by_kernel(c, wn, wnp1) : walls_by_host(c, wn, wnp1, on_device);
   if (e) { cudaGetLastError(); return e; }
   for (int q = 0; q < 18; q++) {
     if (!c->wset[q]) continue;

@@ -80,6 +80,7 @@ struct sph_ctx {
   double* wmean64;
   float* wmean32;
   double* wnext;
+  size_t wcap;             // values the three buffers hold
   double* wzero64;        // zeros of the largest wall size: the arrays without data
   float* wzero32;
   // adjoint workspace (sph_step_adjoint), allocated on first use
