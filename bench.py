@@ -36,12 +36,12 @@ WORKLOAD = ("rising thermal bubble, regional sector r=[6371,6381] km x 20 km x 2
 METRIC = "grid-point updates/s"
 UNIT = "points/s"
 
-# FP64 operations (DADD + DMUL + 2 DFMA, counted from the kernels' SASS
-# instruction mix with ncu, profiles/fp64_counts_bubble_64cubed.md) per grid
-# point of one K = 2 step of the FP64 mode: 2 x (1000 right-hand side, which
-# also stores the line rows + 158 coefficients + 834 sweeps, which read them)
-# + 15 (the second iteration's average).
-FP64_FLOP_PER_POINT_STEP = 4000.0
+# FP64 operations (DADD + DMUL + 2 DFMA, from the instruction counters of ncu,
+# profiles/fp64_counts_bubble_64x128x128.md) per grid point of one K = 2 step of
+# the FP64 mode: 2 x (365 right-hand side, which also stores the line rows + 93
+# coefficients + 631 sweeps, which read them) + 15 (the second iteration's
+# average) + 11 (the last sweep's norms).
+FP64_FLOP_PER_POINT_STEP = 2203.0
 # FP64 FMA throughput of GB300 measured on this machine with independent FMA
 # chains (152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz); MEASURED_PEAKS.json has no
 # FP64 figure, so this is the library's own measurement.
@@ -336,7 +336,7 @@ def run_ours(args, rank, world, dist):
                              "peak": FP64_PEAK_TFLOPS, "frac": ach64 / FP64_PEAK_TFLOPS,
                              "peak_source": "FP64 FMA rate measured by this library on the pool's GB300 "
                                             "(MEASURED_PEAKS.json has no FP64 figure)",
-                             "hbm_note": "the FP64 step does ~4000 FP64 flop per point against ~2.5 KB of traffic: "
+                             "hbm_note": "the FP64 step does ~2200 FP64 flop per point against ~2.5 KB of traffic: "
                                          "bound by the FP64 pipe, not HBM"}}
 
     # dominant kernel of the mixed step and its HBM roofline
