@@ -457,9 +457,18 @@ __device__ __forceinline__ void scalar_lines(const Args& A, float (*ex)[32], flo
 // A phi line is contiguous, so the lanes of a warp (32 lines) read addresses np
 // apart: each lane takes its line in groups of 4 cells with 16-byte loads (VEC:
 // np a multiple of 4; single loads otherwise), the next group in flight while
-// the current one is eliminated.  The split lies at a multiple of 4 cells.
+// the current one is eliminated.  The split lies at a multiple of 4 cells, so that
+// each side's groups are whole -- but for lines of up to 4 cells (5 cyclic ones),
+// which it halves: either side holds a cell, the bottom one the last of the walled
+// line or of the ring's others, whose wall fold and coupling are made there.
 // Cyclic lines keep their last cell X out and carry three more columns H (x = y -
 // Z X), like the FP64 mode's (sph_fp64_lines.cuh).
+
+// the first cell of the bottom side, N >= 2 cells
+__device__ __forceinline__ int phi_split(int N) {
+  const int h = (N + 1) / 2, c = (h + 3) & ~3;
+  return c < N ? c : h;
+}
 
 template <bool VEC>
 __device__ __forceinline__ void load4(const float* f, int m0, int lim, float* o) {
@@ -618,7 +627,7 @@ __device__ __forceinline__ void block_lines_phi(const Args& A, float (*ex)[32], 
   const int nl = g.nr * g.nt, l0 = blk * 32 + lane;
   const bool valid = l0 < nl;
   const int line = valid ? l0 : nl - 1, i = line / g.nt, j = line - i * g.nt;
-  const int half = ((N + 1) / 2 + 3) & ~3, c = half < N ? half : N, lo = side ? c : 0, hi = side ? N : c;
+  const int c = phi_split(N), lo = side ? c : 0, hi = side ? N : c;
   constexpr int W = CYC ? 21 : 12;
   float* scr = A.scr + (size_t)blk * n * (W * 32) + lane;
   float E[9], gv[3], H[9];
@@ -743,10 +752,9 @@ __device__ __forceinline__ void block_lines_phi(const Args& A, float (*ex)[32], 
     float Ab[9], Bb[9], Cb[9], Bi[9], X[3], y[3] = {A.rhs.f[0][e], A.rhs.f[4][e], A.rhs.f[3][fc]};
     form<2>(A, tb[0], tb[1], tb[2], th, t0.rho, true, A.ub.f[3][fc + n - 1], A.ub.f[3][fc], A.c.grr[e], A.c.gtt[e],
             A.c.gpp[e], A.c.srp[e], A.c.stp[e], Ab, Bb, Cb);
-    const int hs = c < N ? 1 : 0;      // the side that holds the last cell of the others
 #pragma unroll
-    for (int w = 0; w < 2; w++) {
-      const float* o = &ex[(w ? hs : 0) * W][lane];
+    for (int w = 0; w < 2; w++) {      // cell 0 lies with the top side, cell N - 1 with the bottom
+      const float* o = &ex[w * W][lane];
       float Zw[9], yw[3];
 #pragma unroll
       for (int q = 0; q < 9; q++) Zw[q] = o[q * 32];
@@ -802,7 +810,7 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
   const int nj = CC == 1 ? g.nt - 1 : g.nt, nl = (CC == 0 ? g.nr - 1 : g.nr) * nj, l0 = blk * 32 + lane;
   const bool valid = l0 < nl;
   const int line = valid ? l0 : nl - 1, i = line / nj + (CC == 0), j = line % nj + (CC == 1);
-  const int half = ((N + 1) / 2 + 3) & ~3, c = half < N ? half : N, lo = side ? c : 0, hi = side ? N : c;
+  const int c = phi_split(N), lo = side ? c : 0, hi = side ? N : c;
   float* scr = A.scr + (size_t)A.nb0 * n * ((CYC ? 21 : 12) * 32) + (size_t)slot * n * (W * 32) + lane;
   const int p0 = CC == 0 ? IC(g, i - 1, j, 0) : IC(g, i, j - 1, 0), p1 = IC(g, i, j, 0);
   const int fx = CC == 0 ? IRf(g, i, j, 0) : ITf(g, i, j, 0);
@@ -929,12 +937,12 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
     ex[side * 3][lane] = Z;
     ex[side * 3 + 1][lane] = x;
     __syncthreads();
-    const int hs = c < N ? 3 : 0, m = n - 1;
+    const int m = n - 1;
     const float hv = __fdividef(A.h, A.c.rho[p0 + m] + A.c.rho[p1 + m]), adv = A.h * (A.c.uc2[p0 + m] + A.c.uc2[p1 + m]) * w.w;
     const float am = fmaf(hv, w.x, -adv), cm = fmaf(hv, w.z, adv);
-    const float den = fmaf(-cm, ex[0][lane], fmaf(-am, ex[hs][lane], fmaf(hv, w.y, 1.f)));
+    const float den = fmaf(-cm, ex[0][lane], fmaf(-am, ex[3][lane], fmaf(hv, w.y, 1.f)));
     if (den == 0.f || !isfinite(den)) sing |= FLAG_SINGULAR;
-    const float X = __fdividef(fmaf(-cm, ex[1][lane], fmaf(-am, ex[hs + 1][lane], A.rhs.f[1 + CC][fx + m])), den);
+    const float X = __fdividef(fmaf(-cm, ex[1][lane], fmaf(-am, ex[4][lane], A.rhs.f[1 + CC][fx + m])), den);
     for (int m0 = lo; m0 < hi; m0 = (m0 & ~3) + 4) {
       const int m1 = (m0 & ~3) + 4 < hi ? (m0 & ~3) + 4 : hi;
       float out[4];
