@@ -979,12 +979,15 @@ static int lines2_use(const sph_ctx* c, int d) {
 }
 
 // The FP64 sweep along d on the rows the right-hand side (or f64_rows) stored;
-// transposed: the adjoint's.  norms: accumulate the squares of the increments.
+// transposed: the adjoint's, which is no stage of a step and is not timed.  norms:
+// accumulate the squares of the increments.
 static int run_lines64(sph_ctx* c, int d, double tau, CF<double> rhs, MF<double> x, int update, CF<double> base,
                        MF<double> uk, bool transposed, bool norms) {
   if (!transposed) k_begin(c, SPH_K_SWEEP_R + d);
   f64_lines(c, d, tau, rhs, x, update, base, uk, transposed, norms);
-  return launch_ok(c);
+  if (!transposed) return launch_ok(c);
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_ERR_CUDA;
 }
 
 template <typename R>
