@@ -236,39 +236,43 @@ static int bufs_alloc(Bufs<R>& b, size_t nmet, int nr, const size_t* nf, long N,
   return SPH_OK;
 }
 
+// The tables of one bulk type, on the context's stream: rounded into tm (nmet
+// values, then as many for the pairs) and td, which have to live until the stream
+// has been waited for.
 template <typename R>
-static int upload_tables(sph_ctx* c, Bufs<R>& b, const double* hmet, const double* hder, int nr) {
+static int upload_tables(sph_ctx* c, Bufs<R>& b, const double* hmet, const double* hder, int nr, R* tm, R* td) {
   size_t nd = 7 * (size_t)nr + 1;
-  R* tm = (R*)malloc(c->nmet * sizeof(R));
-  R* td = (R*)malloc(nd * sizeof(R));
-  if (!tm || !td) { free(tm); free(td); return SPH_ERR_NOMEM; }
   for (size_t q = 0; q < c->nmet; q++) tm[q] = (R)hmet[q];
   for (size_t q = 0; q < nd; q++) td[q] = (R)hder[q];
-  int e = SPH_OK;
-  if (!cuda_ok(cudaMemcpy(b.metric, tm, c->nmet * sizeof(R), cudaMemcpyHostToDevice)) ||
-      !cuda_ok(cudaMemcpy(b.bgder, td, nd * sizeof(R), cudaMemcpyHostToDevice)))
-    e = SPH_ERR_CUDA;
-  // rf^2 and sin(theta_f) as hi + lo pairs (tm has room: nmet > 2 (nr+1) + 2 (nt+1))
+  if (!cuda_ok(cudaMemcpyAsync(b.metric, tm, c->nmet * sizeof(R), cudaMemcpyHostToDevice, c->st)) ||
+      !cuda_ok(cudaMemcpyAsync(b.bgder, td, nd * sizeof(R), cudaMemcpyHostToDevice, c->st)))
+    return SPH_ERR_CUDA;
+  // rf^2 and sin(theta_f) as hi + lo pairs (nmet > 2 (nr+1) + 2 (nt+1))
   int nt = c->d64.g.nt;
   const double* rf = hmet + (nr + 1);
   const double* sf = hmet + 4 * (nr + 1) + (nt + 1);
+  tm += c->nmet;
   R* rh = tm; R* rl = tm + (nr + 1); R* sh = tm + 2 * (nr + 1); R* sl = sh + (nt + 1);
   for (int i = 0; i <= nr; i++) { double v = rf[i] * rf[i]; rh[i] = (R)v; rl[i] = (R)(v - (double)rh[i]); }
   for (int j = 0; j <= nt; j++) { double v = sf[j]; sh[j] = (R)v; sl[j] = (R)(v - (double)sh[j]); }
   size_t nm = 2 * (size_t)(nr + 1) + 2 * (size_t)(nt + 1);
-  if (e == SPH_OK && !cuda_ok(cudaMemcpy(b.mdf, tm, nm * sizeof(R), cudaMemcpyHostToDevice))) e = SPH_ERR_CUDA;
-  free(tm); free(td);
-  return e;
+  return cuda_ok(cudaMemcpyAsync(b.mdf, tm, nm * sizeof(R), cudaMemcpyHostToDevice, c->st)) ? SPH_OK : SPH_ERR_CUDA;
 }
 
-// Background-derived tables (FP64 on the host, then in each bulk type).
+// Background-derived tables (FP64 on the host, then in each bulk type) and the
+// kernels' tables made from them.  Copies and kernels run in order on the
+// context's stream and are done on return: other streams (a batch's) read the
+// tables without waiting for the context's.
 static int upload_background(sph_ctx* c, const double* pref, const double* Tref) {
   const Geo<double>& g = c->d64.g;
   int nr = g.nr;
   const double* rc = c->hmet;
   const double* rf = rc + (nr + 1);
-  double* der = (double*)calloc(7 * (size_t)nr + 1, sizeof(double));
-  if (!der) return SPH_ERR_NOMEM;
+  const size_t nd = 7 * (size_t)nr + 1, nt2 = 2 * c->nmet + nd;
+  double* der = (double*)calloc(nd, sizeof(double));
+  double* t64 = (double*)malloc(nt2 * sizeof(double));
+  float* t32 = (float*)malloc(nt2 * sizeof(float));
+  if (!der || !t64 || !t32) { free(der); free(t64); free(t32); return SPH_ERR_NOMEM; }
   double* dbgp = der; double* dbgT = der + nr; double* lapT = der + 2 * nr; double* rhoref = der + 3 * nr;
   double* ehyd = der + 4 * nr;
   double* pcen = der + 5 * nr + 1; double* Tcen = der + 6 * nr + 1;
@@ -287,14 +291,15 @@ static int upload_background(sph_ctx* c, const double* pref, const double* Tref)
     double rf_ = 0.5 * (rhoref[i - 1] + rhoref[i]);
     ehyd[i] = rf_ != 0.0 ? (pref[i + 1] - pref[i]) / (g.dr * rf_) + c->P.g : c->P.g;
   }
-  int e = upload_tables(c, c->d64, c->hmet, der, nr);
-  if (e == SPH_OK && c->prec == SPH_PREC_MIXED) e = upload_tables(c, c->d32, c->hmet, der, nr);
+  int e = upload_tables(c, c->d64, c->hmet, der, nr, t64, t64 + 2 * c->nmet);
+  if (e == SPH_OK && c->prec == SPH_PREC_MIXED) e = upload_tables(c, c->d32, c->hmet, der, nr, t32, t32 + 2 * c->nmet);
   if (e == SPH_OK && c->tab64) {
     f64_tables(c);
     if (c->tab32s) s32_tables(c);
     if (cudaGetLastError() != cudaSuccess) e = SPH_ERR_CUDA;
   }
-  free(der);
+  if (cudaStreamSynchronize(c->st) != cudaSuccess) e = SPH_ERR_CUDA;   // (the host buffers' copies, too)
+  free(der); free(t64); free(t32);
   return e;
 }
 
@@ -411,11 +416,13 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
       c->tabs = f64::tabs_of(c->tab64, nr, nt);
   }
   if (err != SPH_OK) { cudaGetLastError(); free_all(c); free(c); return err; }
-  if (!cuda_ok(cudaMemset(c->bg, 0, 2 * (size_t)(nr + 2) * sizeof(double))) || !cuda_ok(cudaMemset(c->flag, 0, sizeof(int))))
+  // (on the context's stream, which upload_background waits for below)
+  if (!cuda_ok(cudaMemsetAsync(c->bg, 0, 2 * (size_t)(nr + 2) * sizeof(double), c->st)) ||
+      !cuda_ok(cudaMemsetAsync(c->flag, 0, sizeof(int), c->st)))
     err = SPH_ERR_CUDA;
   for (int f = 0; f < 5 && err == SPH_OK; f++)
-    if (!cuda_ok(cudaMemset(c->U[0][f], 0, c->nf[f] * sizeof(double))) ||
-        !cuda_ok(cudaMemset(c->U[1][f], 0, c->nf[f] * sizeof(double))))
+    if (!cuda_ok(cudaMemsetAsync(c->U[0][f], 0, c->nf[f] * sizeof(double), c->st)) ||
+        !cuda_ok(cudaMemsetAsync(c->U[1][f], 0, c->nf[f] * sizeof(double), c->st)))
       err = SPH_ERR_CUDA;
   if (err != SPH_OK) { free_all(c); free(c); return err; }
   set_geo_ptrs(c->d64, g, c->bg, nr, nt);
@@ -431,8 +438,8 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
     if (cudaMalloc((void**)&c->wzero64, wmax * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void**)&c->wzero32, wmax * sizeof(float)) != cudaSuccess)
       err = SPH_ERR_NOMEM;
-    else if (cudaMemset(c->wzero64, 0, wmax * sizeof(double)) != cudaSuccess ||
-             cudaMemset(c->wzero32, 0, wmax * sizeof(float)) != cudaSuccess)
+    else if (cudaMemsetAsync(c->wzero64, 0, wmax * sizeof(double), c->st) != cudaSuccess ||
+             cudaMemsetAsync(c->wzero32, 0, wmax * sizeof(float), c->st) != cudaSuccess)
       err = SPH_ERR_CUDA;
     for (int q = 0; q < 18; q++) { c->d64.g.w[q] = c->wzero64; c->d32.g.w[q] = c->wzero32; }
     if (err) { cudaGetLastError(); free_all(c); free(c); return err; }
@@ -444,9 +451,11 @@ extern "C" int sph_create(const sph_grid* gr, const sph_params* pa, void* stream
   free(zb); free(tb);
   if (err != SPH_OK) { free_all(c); free(c); return err; }
   if (mixed && (err = lines_prepare(c)) != SPH_OK) { free_all(c); free(c); return err; }
-  if (mixed) {
+  if (mixed) {   // (from the grid alone)
     lines2_tables(c);
-    if (cudaGetLastError() != cudaSuccess) { free_all(c); free(c); return SPH_ERR_CUDA; }
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c->st) != cudaSuccess) {
+      free_all(c); free(c); return SPH_ERR_CUDA;
+    }
   }
   if (cudaEventCreateWithFlags(&c->efork, cudaEventDisableTiming) != cudaSuccess) err = SPH_ERR_CUDA;
   for (int q = 0; q < 3 && !err; q++)
@@ -468,11 +477,11 @@ extern "C" int sph_set_background(sph_ctx* c, const double* p_ref, const double*
   if (p_ref) memcpy(hp_, p_ref, n * sizeof(double));
   if (T_ref) memcpy(hT, T_ref, n * sizeof(double));
   int e = SPH_OK;
-  if (cudaStreamSynchronize(c->st) != cudaSuccess ||
-      cudaMemcpy(c->bg, hp_, n * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(c->bg + n, hT, n * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (cudaMemcpyAsync(c->bg, hp_, n * sizeof(double), cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
+      cudaMemcpyAsync(c->bg + n, hT, n * sizeof(double), cudaMemcpyHostToDevice, c->st) != cudaSuccess)
     e = SPH_ERR_CUDA;
   if (e == SPH_OK) e = upload_background(c, hp_, hT);
+  else cudaStreamSynchronize(c->st);   // (a copy may still read the host buffers)
   free(hp_); free(hT);
   return e;
 }

@@ -26,7 +26,7 @@ static f64::Args args64(sph_ctx* c, CF<double> ub) {
   return A;
 }
 
-// on the context's stream, after the (synchronous) uploads of the tables it reads
+// on the context's stream, in order after the uploads of the tables it reads
 void f64_tables(sph_ctx* c) {
   const Geo<double>& g = c->d64.g;
   f64::k_tab<<<((g.nr + 1) * (g.nt + 1) + 127) / 128, 128, 0, c->st>>>(g, c->P, c->tabs);
