@@ -137,11 +137,12 @@ __device__ __forceinline__ void form(const Consts& A, const float4& q0, const fl
   }
 }
 
-__device__ __forceinline__ void inverse_or_nan(const float* S, float* I, int* bad) {
+template <typename R>
+__device__ __forceinline__ void inverse_or_nan(const R* S, R* I, int* bad) {
   if (!inv3(S, I)) {
     *bad |= FLAG_SINGULAR;
 #pragma unroll
-    for (int q = 0; q < 9; q++) I[q] = NAN;
+    for (int q = 0; q < 9; q++) I[q] = R(NAN);
   }
 }
 
@@ -462,7 +463,9 @@ __device__ __forceinline__ void scalar_lines(const Args& A, float (*ex)[32], flo
 // which it halves: either side holds a cell, the bottom one the last of the walled
 // line or of the ring's others, whose wall fold and coupling are made there.
 // Cyclic lines keep their last cell X out and carry three more columns H (x = y -
-// Z X), like the FP64 mode's (sph_fp64_lines.cuh).
+// Z X), like the FP64 mode's (sph_fp64_lines.cuh).  X's own system and every x = y -
+// Z X are FP64, as in the one-thread-per-line solver: y and Z X cancel where the
+// ring is stiff, and the increment reaches the FP64 state unrounded.
 
 // the first cell of the bottom side, N >= 2 cells
 __device__ __forceinline__ int phi_split(int N) {
@@ -562,19 +565,23 @@ __device__ __forceinline__ void eliminate_phi(const Args& A, int i, int j, int N
   }
 }
 
+// an integer test for FP64 values, whose compares take the FP64 pipe
+__device__ __forceinline__ bool finite_(float v) { return isfinite(v); }
+__device__ __forceinline__ bool finite_(double v) { return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u; }
+
 // cells [m0, m1) of one group of a line's field: x (update = 0) or uk = base + x;
-// v[q] belongs to index m0 - m0 % 4 + q
-template <bool VEC>
-__device__ __forceinline__ void emit4(const Args& A, int f, int at, int m0, int m1, const float* v, SqSum<float>& ss,
-                                      int* bad) {
+// v[q] belongs to index m0 - m0 % 4 + q.  V: float, or double on cyclic lines,
+// whose increment reaches the state unrounded.
+template <bool VEC, typename V>
+__device__ __forceinline__ void emit4(const Args& A, int f, int at, int m0, int m1, const V* v, SqSum<float>& ss, int* bad) {
   const int g0 = m0 & ~3;
   if (!A.update) {
     float* x = A.x.f[f] + at;
     if (VEC && m1 - m0 == 4) {
-      *reinterpret_cast<float4*>(x + g0) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<float4*>(x + g0) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
     } else {
 #pragma unroll
-      for (int q = 0; q < 4; q++) if (g0 + q >= m0 && g0 + q < m1) x[g0 + q] = v[q];
+      for (int q = 0; q < 4; q++) if (g0 + q >= m0 && g0 + q < m1) x[g0 + q] = (float)v[q];
     }
     return;
   }
@@ -583,8 +590,8 @@ __device__ __forceinline__ void emit4(const Args& A, int f, int at, int m0, int 
 #pragma unroll
   for (int q = 0; q < 4; q++)
     if (g0 + q >= m0 && g0 + q < m1) {
-      if (!isfinite(v[q])) *bad |= FLAG_NONFINITE;
-      if (A.norms) ss.add(f, v[q]);
+      if (!finite_(v[q])) *bad |= FLAG_NONFINITE;
+      if (A.norms) ss.add(f, (float)v[q]);
     }
   if (VEC && m1 - m0 == 4) {
     const double2 b0 = reinterpret_cast<const double2*>(b)[0], b1 = reinterpret_cast<const double2*>(b)[1];
@@ -603,9 +610,9 @@ __device__ __forceinline__ void emit_wall(const Args& A, int f, int idx) {
   else A.x.f[f][idx] = 0.f;
 }
 // cells [m0, m1) of one group of a block line: p, T, and u on their faces m + 1
-template <bool CYC, bool VEC>
-__device__ __forceinline__ void emit_cells(const Args& A, int i, int j, int m0, int m1, const float (*v)[4],
-                                           SqSum<float>& ss, int* bad) {
+template <bool CYC, bool VEC, typename V>
+__device__ __forceinline__ void emit_cells(const Args& A, int i, int j, int m0, int m1, const V (*v)[4], SqSum<float>& ss,
+                                           int* bad) {
   const Geo<float>& g = A.g;
   const int n = g.np, ic = IC(g, i, j, 0), fc = IPf(g, i, j, 0);
   emit4<VEC>(A, 0, ic, m0, m1, v[0], ss, bad);
@@ -749,35 +756,38 @@ __device__ __forceinline__ void block_lines_phi(const Args& A, float (*ex)[32], 
     const int ic = IC(g, i, j, 0), fc = IPf(g, i, j, 0), e = ic + n - 1;
     const float4* tb = reinterpret_cast<const float4*>(A.T.b[2] + (size_t)NB * (i * g.nt + j));
     const Th th = thermo(A, i, A.ub.f[0][e], A.ub.f[4][e]), t0 = thermo(A, i, A.ub.f[0][ic], A.ub.f[4][ic]);
-    float Ab[9], Bb[9], Cb[9], Bi[9], X[3], y[3] = {A.rhs.f[0][e], A.rhs.f[4][e], A.rhs.f[3][fc]};
+    float Ab[9], Bb[9], Cb[9];
     form<2>(A, tb[0], tb[1], tb[2], th, t0.rho, true, A.ub.f[3][fc + n - 1], A.ub.f[3][fc], A.c.grr[e], A.c.gtt[e],
             A.c.gpp[e], A.c.srp[e], A.c.stp[e], Ab, Bb, Cb);
+    double L[9], B[9], Bi[9], X[3], y[3] = {A.rhs.f[0][e], A.rhs.f[4][e], A.rhs.f[3][fc]};
+#pragma unroll
+    for (int q = 0; q < 9; q++) B[q] = Bb[q];
 #pragma unroll
     for (int w = 0; w < 2; w++) {      // cell 0 lies with the top side, cell N - 1 with the bottom
       const float* o = &ex[w * W][lane];
-      float Zw[9], yw[3];
+      double Zw[9], yw[3];
 #pragma unroll
-      for (int q = 0; q < 9; q++) Zw[q] = o[q * 32];
+      for (int q = 0; q < 9; q++) { Zw[q] = o[q * 32]; L[q] = (w ? M_A : M_C) >> q & 1 ? (w ? Ab : Cb)[q] : 0.f; }
 #pragma unroll
       for (int q = 0; q < 3; q++) yw[q] = o[(9 + q) * 32];
-      if (w) { sub_mul<M_A, 3>(Ab, Zw, Bb); sub_mul<M_A, 1>(Ab, yw, y); }
-      else { sub_mul<M_C, 3>(Cb, Zw, Bb); sub_mul<M_C, 1>(Cb, yw, y); }
+      if (w) { sub_mul<M_A, 3>(L, Zw, B); sub_mul<M_A, 1>(L, yw, y); }
+      else { sub_mul<M_C, 3>(L, Zw, B); sub_mul<M_C, 1>(L, yw, y); }
     }
-    inverse_or_nan(Bb, Bi, &sing);
+    inverse_or_nan(B, Bi, &sing);
     mv(Bi, y, X);
     for (int m0 = lo; m0 < hi; m0 = (m0 & ~3) + 4) {
       const int m1 = (m0 & ~3) + 4 < hi ? (m0 & ~3) + 4 : hi;
-      float out[3][4];
+      double out[3][4];
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int m = (m0 & ~3) + q;
         if (m < m0 || m >= m1) continue;
         const float* sp = scr + (size_t)m * (W * 32);
-        float Zm[9], v[3];
+        double Zm[9], v[3];
 #pragma unroll
-        for (int k = 0; k < 9; k++) Zm[k] = sp[k * 32];
+        for (int k = 0; k < 9; k++) Zm[k] = f2d(sp[k * 32]);
 #pragma unroll
-        for (int k = 0; k < 3; k++) v[k] = sp[(9 + k) * 32];
+        for (int k = 0; k < 3; k++) v[k] = f2d(sp[(9 + k) * 32]);
         sub_mul<M_ALL, 1>(Zm, X, v);
 #pragma unroll
         for (int k = 0; k < 3; k++) out[k][q] = v[k];
@@ -788,7 +798,7 @@ __device__ __forceinline__ void block_lines_phi(const Args& A, float (*ex)[32], 
         asm volatile("discard.global.L2 [%0], 128;" ::"l"(scr - lane + ((size_t)m0 * W + k) * 32) : "memory");
     }
     if (side == 0 && valid) {
-      float out[3][4];
+      double out[3][4];
 #pragma unroll
       for (int q = 0; q < 4; q++)
 #pragma unroll
@@ -939,19 +949,19 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
     __syncthreads();
     const int m = n - 1;
     const float hv = __fdividef(A.h, A.c.rho[p0 + m] + A.c.rho[p1 + m]), adv = A.h * (A.c.uc2[p0 + m] + A.c.uc2[p1 + m]) * w.w;
-    const float am = fmaf(hv, w.x, -adv), cm = fmaf(hv, w.z, adv);
-    const float den = fmaf(-cm, ex[0][lane], fmaf(-am, ex[3][lane], fmaf(hv, w.y, 1.f)));
-    if (den == 0.f || !isfinite(den)) sing |= FLAG_SINGULAR;
-    const float X = __fdividef(fmaf(-cm, ex[1][lane], fmaf(-am, ex[4][lane], A.rhs.f[1 + CC][fx + m])), den);
+    const double am = fmaf(hv, w.x, -adv), cm = fmaf(hv, w.z, adv);
+    const double den = fma(-cm, (double)ex[0][lane], fma(-am, (double)ex[3][lane], (double)fmaf(hv, w.y, 1.f)));
+    if (den == 0.0 || !finite_(den)) sing |= FLAG_SINGULAR;
+    const double X = fma(-cm, (double)ex[1][lane], fma(-am, (double)ex[4][lane], (double)A.rhs.f[1 + CC][fx + m])) / den;
     for (int m0 = lo; m0 < hi; m0 = (m0 & ~3) + 4) {
       const int m1 = (m0 & ~3) + 4 < hi ? (m0 & ~3) + 4 : hi;
-      float out[4];
+      double out[4];
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int k = (m0 & ~3) + q;
         if (k < m0 || k >= m1) continue;
         const float* sp = scr + (size_t)k * (W * 32);
-        out[q] = fmaf(-sp[0], X, sp[32]);
+        out[q] = fma(-f2d(sp[0]), X, f2d(sp[32]));
       }
       if (valid) {
         emit4<VEC>(A, 1 + CC, fx, m0, m1, out, ss, bad);
@@ -959,7 +969,7 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
       }
     }
     if (side == 0 && valid) {
-      const float out[4] = {X, X, X, X};
+      const double out[4] = {X, X, X, X};
       emit4<VEC>(A, 1 + CC, fx, n - 1, n, out, ss, bad);
       if (wl || wh) wall(n - 1, n, wl, wh);
     }
