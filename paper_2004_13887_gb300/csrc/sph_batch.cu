@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(CB / P, 65536 * P / (CB * 48)) k_lines_sca_f(c
 template <int D>
 __global__ void __launch_bounds__(64, LINES2_MINB) k_l2_blk_f(const lines2::Args* tab, const int2* map) {
   __shared__ lines2::Args S;
-  __shared__ float ex[24][32];
+  __shared__ float ex[lines2::NEX][32];
   __shared__ float rings[2 * lines2::RING][32];
   const int2 m = map[blockIdx.x];
   load_args(S, tab[m.x]);

@@ -443,7 +443,7 @@ __device__ __forceinline__ void lines_blk(const SweepArgs<float>& S, int grp) {
       float rr[3] = {sm[8 * FS + si], sm[9 * FS + si], sm[10 * FS + si]};
       float A[9], B[9], C[9];
       lines2::form<D>(S, q0, q1, q2, t0, th.rho, face, uf, ufn, sm[2 * FS + si], sm[3 * FS + si], sm[4 * FS + si],
-                      D > 0 ? sm[5 * FS + si] : 0.f, D > 1 ? sm[6 * FS + si] : 0.f, A, B, C);
+                      D > 0 ? sm[5 * FS + si] : 0.f, D > 1 ? sm[6 * FS + si] : 0.f, A, B, C, rr);
       A[3] = A[6] = A[7] = 0.f;
       C[2] = C[3] = C[5] = C[7] = 0.f;
       if (!cyc && (m == 0 || m == n - 1)) {   // zero-gradient ghosts of p and T

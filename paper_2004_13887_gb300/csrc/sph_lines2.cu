@@ -1,5 +1,5 @@
-// sph_lines2.cu -- launches of the r- and theta-sweeps of the mixed mode over many
-// lines (sph_lines2.cuh; Section 2.2, eqs. spl1, spl2).
+// sph_lines2.cu -- launches of the sweeps of the mixed mode over many lines
+// (sph_lines2.cuh; Section 2.2, eqs. spl1-spl3).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>

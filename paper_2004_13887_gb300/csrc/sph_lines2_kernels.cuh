@@ -45,7 +45,7 @@ __global__ void k_tab(Geo<double> g, Par P, Tabs T) {
         w[2] = 2.0 * mu * m2 * (q * (c0 + c1) + f1 * (ic1 + ic0) / 3.0);
         w[3] = -2.0 * mu * m2 * (q * c1 + fp * ic1 / 3.0);
       }
-      b[B_WP] = (float)w[0]; b[B_F0] = (float)w[1]; b[B_F1] = (float)w[2]; b[B_F2] = (float)w[3];
+      b[B_WP] = (float)w[0]; b[B_F0] = (float)w[1]; b[B_FS] = (float)(w[1] + w[2] + w[3]); b[B_F2] = (float)w[3];
       float* s = T.s[0][0] + (size_t)NS * i;
       s[S_W0] = (float)(-2.0 * mu * l00); s[S_W1] = (float)(2.0 * mu * (l00 + l01)); s[S_W2] = (float)(-2.0 * mu * l01);
       s[S_Q] = (float)(0.25 * g.idr);
@@ -64,7 +64,7 @@ __global__ void k_tab(Geo<double> g, Par P, Tabs T) {
       w[2] = 2.0 * mu * m2 * (isf * (c0 + c1) + g.sf[j + 1] * (ic1 + ic0) / 3.0);
       w[3] = -2.0 * mu * m2 * (isf * c1 + g.sf[j + 2] * ic1 / 3.0);
     }
-    b[B_WP] = (float)w[0]; b[B_F0] = (float)w[1]; b[B_F1] = (float)w[2]; b[B_F2] = (float)w[3];
+    b[B_WP] = (float)w[0]; b[B_F0] = (float)w[1]; b[B_FS] = (float)(w[1] + w[2] + w[3]); b[B_F2] = (float)w[3];
     const double mp = ir * is * g.idph;
     float* f = T.b[2] + (size_t)NB * (i * g.nt + j);
     f[B_G0] = f[B_G1] = (float)mp;
@@ -72,7 +72,7 @@ __global__ void k_tab(Geo<double> g, Par P, Tabs T) {
     f[B_LIN] = (float)(0.25 * ir); f[B_COT2] = (float)g.cotc[j];
     f[B_M] = (float)mp; f[B_HM] = (float)(0.5 * mp);
     f[B_WP] = (float)(2.0 * mp);
-    f[B_F0] = f[B_F2] = (float)(-8.0 / 3.0 * mu * mp * mp); f[B_F1] = (float)(16.0 / 3.0 * mu * mp * mp);
+    f[B_F0] = f[B_F2] = (float)(-8.0 / 3.0 * mu * mp * mp); f[B_FS] = 0.f;
     float* s = T.s[1][1] + (size_t)NS * (i * g.nt + j);
     s[S_W0] = (float)(-2.0 * mu * l10); s[S_W1] = (float)(2.0 * mu * (l10 + l11)); s[S_W2] = (float)(-2.0 * mu * l11);
     s[S_Q] = (float)(0.25 * mt);
@@ -87,7 +87,7 @@ __global__ void k_tab(Geo<double> g, Par P, Tabs T) {
 
 template <int D>
 __global__ void __launch_bounds__(64, LINES2_MINB) k_blk(const __grid_constant__ Args A) {
-  __shared__ float ex[24][32];
+  __shared__ float ex[NEX][32];
   __shared__ float rings[2 * RING][32];
   int bad = 0;
   block_lines<D>(A, ex, rings, blockIdx.x, &bad);
@@ -115,7 +115,7 @@ __device__ __forceinline__ void finish(const Args& A, const SqSum<float>& ss, in
 }
 template <bool CYC, bool VEC>
 __global__ void __launch_bounds__(64) k_blk_phi(const __grid_constant__ Args A) {
-  __shared__ float ex[CYC ? 42 : 24][32];
+  __shared__ float ex[CYC ? 42 : NEX][32];
   int bad = 0;
   SqSum<float> ss;
   block_lines_phi<CYC, VEC>(A, ex, blockIdx.x, ss, &bad);
