@@ -553,7 +553,8 @@ __device__ __forceinline__ void scalar_line(const LineArgs& S, double (*ex)[32],
   double x, z = 0.0;
   {
     const double* o = &ex[(1 - side) * NEX][lane];
-    const double id = 1.0 / fma(-e, o[0], 1.0);
+    const double den = fma(-e, o[0], 1.0), id = 1.0 / den;
+    if (bad_pivot(den)) *bad |= FLAG_SINGULAR;
     x = fma(-e, o[32], gy) * id;
     if (CYC) z = fma(-e, o[64], hz) * id;
   }

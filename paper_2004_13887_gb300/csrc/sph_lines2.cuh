@@ -528,8 +528,9 @@ __device__ __forceinline__ void scalar_lines(const Args& A, float (*ex)[32], flo
   for (int t = 0; t < SBACK; t++) back(t);
   float x;
   {
-    const float ep = ex[(1 - side) * 2][lane], gp = ex[(1 - side) * 2 + 1][lane];
-    x = __fdividef(fmaf(-e, gp, gy), fmaf(-e, ep, 1.f));
+    const float ep = ex[(1 - side) * 2][lane], gp = ex[(1 - side) * 2 + 1][lane], den = fmaf(-e, ep, 1.f);
+    if (den == 0.f || !isfinite(den)) sing |= FLAG_SINGULAR;
+    x = __fdividef(fmaf(-e, gp, gy), den);
   }
   for (int s = cnt - 1; s >= 0; s--) {
     const int m = cell(s);
@@ -1070,8 +1071,9 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
   __syncthreads();
   float x, Z = 0.f;
   {
-    const float ep = ex[(1 - side) * 3][lane], gp = ex[(1 - side) * 3 + 1][lane];
-    const float id = __fdividef(1.f, fmaf(-e, ep, 1.f));
+    const float ep = ex[(1 - side) * 3][lane], gp = ex[(1 - side) * 3 + 1][lane], den = fmaf(-e, ep, 1.f);
+    if (den == 0.f || !isfinite(den)) sing |= FLAG_SINGULAR;
+    const float id = __fdividef(1.f, den);
     x = fmaf(-e, gp, gy) * id;
     if (CYC) Z = fmaf(-e, ex[(1 - side) * 3 + 2][lane], hz) * id;
   }
