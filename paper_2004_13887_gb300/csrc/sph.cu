@@ -1222,23 +1222,31 @@ extern "C" int sph_step(sph_ctx* c, double dt, int n_iter, const double* const* 
 // ------------------------------------------------------------ adjoint
 
 static int adj_alloc(sph_ctx* c, int K) {
-  if (c->adjS && c->adjK >= K) return SPH_OK;
-  cudaFree(c->adjS);
-  c->adjS = NULL;
-  c->adjK = 0;
   // every field of a set starts on a 256-byte boundary: the averaging kernel
   // reads the state in 16-byte pairs, and aligned rows keep the loads whole
   size_t fs = 0;
   for (int f = 0; f < 5; f++) { c->foff[f] = fs; fs += (c->nf[f] + 31) / 32 * 32; }
   c->fset = fs;
-  if (cudaMalloc((void**)&c->adjS, (size_t)K * fs * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return SPH_ERR_NOMEM; }
-  c->adjK = K;
-  if (c->adjW) return SPH_OK;
-  if (cudaMalloc((void**)&c->adjW, 10 * fs * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&c->adjC, (size_t)f64::ADJ_PLANES * c->N * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(c->adjW);
+  if (!c->adjS || c->adjK < K) {
+    cudaFree(c->adjS);
+    c->adjS = NULL;
+    c->adjK = 0;
+    if (cudaMalloc((void**)&c->adjS, (size_t)K * fs * sizeof(double)) != cudaSuccess) {
+      c->adjS = NULL;
+      cudaGetLastError();
+      return SPH_ERR_NOMEM;
+    }
+    c->adjK = K;
+  }
+  // (each on its own: a call after a failed one asks for what is missing)
+  if (!c->adjW && cudaMalloc((void**)&c->adjW, 10 * fs * sizeof(double)) != cudaSuccess) {
     c->adjW = NULL;
+    cudaGetLastError();
+    return SPH_ERR_NOMEM;
+  }
+  if (!c->adjC && cudaMalloc((void**)&c->adjC, (size_t)f64::ADJ_PLANES * c->N * sizeof(double)) != cudaSuccess) {
+    c->adjC = NULL;
+    cudaGetLastError();
     return SPH_ERR_NOMEM;
   }
   return SPH_OK;
