@@ -987,6 +987,11 @@ static int lines2_use(const sph_ctx* c, int d) {
   return d < 2 && lines >= LINES2_MIN;
 }
 
+// Whether the FP64 sweeps take the one-thread-per-line solver: by choice, or for a
+// step so short that the others, whose rows are divided by h, would overflow in a
+// block's determinant (1/h^3 times the pivots' other factors).
+static bool thomas64(const sph_ctx* c, double tau) { return c->line_solver == SPH_LINES_THOMAS || tau < 1e-60; }
+
 // The FP64 sweep along d on the rows the right-hand side (or f64_rows) stored;
 // transposed: the adjoint's, which is no stage of a step and is not timed.  norms:
 // accumulate the squares of the increments.
@@ -1003,7 +1008,7 @@ template <typename R>
 static int run_sweep(sph_ctx* c, Bufs<R>& b, int d, double tau, CF<R> ub, CF<R> rhs, MF<R> x, int update,
                      CF<double> base, MF<double> uk, int norms = 0) {
   if constexpr (sizeof(R) == sizeof(double))
-    if (c->line_solver != SPH_LINES_THOMAS) return run_lines64(c, d, tau, rhs, x, update, base, uk, false, norms);
+    if (!thomas64(c, tau)) return run_lines64(c, d, tau, rhs, x, update, base, uk, false, norms);
   SweepArgs<R> S;
   memset(&S, 0, sizeof S);
   S.g = b.g; S.P = c->P; S.c = b.c; S.ub = ub; S.d = d; S.h = (R)(0.5 * tau);
@@ -1109,7 +1114,7 @@ static int sweep_impl(sph_ctx* c, Bufs<R>& b, int dir, double dt, const double* 
   CF<double> base = cf_of(c->U[c->cur]);
   MF<double> ukm = mf_of(c->U[1 - c->cur]);
   if constexpr (sizeof(R) == sizeof(double)) {
-    if (c->line_solver != SPH_LINES_THOMAS) {
+    if (!thomas64(c, dt)) {
       f64_rows(c, ub, dir);
       c->launches++;
     }
@@ -1267,7 +1272,7 @@ static int adj_axpy(sph_ctx* c, double s, double* x, double* y) {
 // the transposed sweep along d: x = P A_d^{-T} P rhs (P: zero on the wall faces)
 static int run_sweep_T(sph_ctx* c, int d, double tau, CF<double> ub, CF<double> rhs, MF<double> x) {
   Bufs<double>& b = c->d64;
-  if (c->line_solver != SPH_LINES_THOMAS) return run_lines64(c, d, tau, rhs, x, 0, rhs, x, true, false);
+  if (!thomas64(c, tau)) return run_lines64(c, d, tau, rhs, x, 0, rhs, x, true, false);
   SweepArgs<double> S;
   memset(&S, 0, sizeof S);
   S.g = b.g; S.P = c->P; S.c = b.c; S.ub = ub; S.d = d; S.h = 0.5 * tau;
