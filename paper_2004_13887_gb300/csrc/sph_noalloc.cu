@@ -147,8 +147,10 @@ __global__ void __launch_bounds__(32) k_block_thomas_split(int nlines, int n, co
     if (hi >= 0x7ff00000u || (hi | (unsigned)__double2loint(det)) == 0u) bad = true;   // zero or non-finite pivot
     const double u0 = q < 3 ? c0 : 0.0, u1 = q < 3 ? c1 : 0.0, u2 = q < 3 ? c2 : 0.0;
     const double y0 = at(t, 0, 3), y1 = at(t, 1, 3), y2 = at(t, 2, 3);
-    const double w = fma(at(adj, r, 2), q < 3 ? u2 : y2, fma(at(adj, r, 1), q < 3 ? u1 : y1, at(adj, r, 0) * (q < 3 ? u0 : y0)));
-    v = w * (1.0 / det);
+    // (the inverse before it meets the right-hand side, as one thread per line does: adj(S)
+    // alone has the square of S's scale, and its product may leave FP64's range)
+    const double inv = adj * (1.0 / det);
+    v = fma(at(inv, r, 2), q < 3 ? u2 : y2, fma(at(inv, r, 1), q < 3 ? u1 : y1, at(inv, r, 0) * (q < 3 ? u0 : y0)));
     if (m < n - 1 && valid && e < 12) scr[(l * n + m) * 12 + e] = v;
   }
   __syncwarp();
