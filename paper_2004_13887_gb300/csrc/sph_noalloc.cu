@@ -18,13 +18,13 @@
 #include "../../include/sph.h"
 
 #define NOALLOC_MAX_DEVICES 64
-#define SPLIT_LINES 8192
 
 static __device__ __align__(256) double g_noalloc_scratch[(size_t)SPH_NOALLOC_MAX_BLOCKS * 12];
 
 // Device address of the array on each device, looked up once per device: in
 // host code the symbol's name is only a host-side stand-in, not an address.
 static double* s_scratch[NOALLOC_MAX_DEVICES];
+static int s_nsm[NOALLOC_MAX_DEVICES];   // and its SMs
 
 static __device__ __forceinline__ bool inv3_na(const double* S, double* I) {
   double c00 = S[4] * S[8] - S[5] * S[7];
@@ -107,7 +107,7 @@ __global__ void k_block_thomas_noalloc(int nlines, int n, const double* __restri
 // warps.  Here lane 4 r + q holds element (r, q) of [C'_m | d'_m] (3 x 4; lanes 12-15
 // repeat row 2) and every product of the same elimination, in the same order,
 // is one element per lane, its operands exchanged by shuffles: 17 FP64
-// instructions a block.  1024 lines of 128 blocks: 685 -> 154 us.
+// instructions a block.  1024 lines of 128 blocks: 661 -> 146 us.
 __device__ __forceinline__ double from(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
 __global__ void __launch_bounds__(32) k_block_thomas_split(int nlines, int n, const double* __restrict__ A,
@@ -176,11 +176,12 @@ __global__ void __launch_bounds__(32) k_block_thomas_split(int nlines, int n, co
   }
 }
 
-// Per-device set-up, with that device current: the device address of the array.
+// Per-device set-up, with that device current: its SMs, the device address of the array.
 static int noalloc_setup(int dev) {
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return SPH_ERR_ARG;
   if (s_scratch[dev]) return SPH_OK;
   void* p = NULL;
+  if (cudaDeviceGetAttribute(&s_nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SPH_ERR_CUDA;
   if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return SPH_ERR_CUDA;
   s_scratch[dev] = (double*)p;
   return SPH_OK;
@@ -195,11 +196,12 @@ extern "C" int sph_block_thomas_noalloc(int nlines, int n, const double* A, cons
   int e = noalloc_setup(dev);
   if (e != SPH_OK) return e;
   cudaStream_t st = (cudaStream_t)stream;
-  // the lane-split form needs 17 FP64 instructions a block on nlines / 2 warps,
-  // one thread per line about 120 on nlines / 32, over the 608 SM quarters: the
-  // split's time grows with the lines once they fill the quarters (1216 lines)
-  // and reaches the other's at about 8192
-  if (nlines <= SPLIT_LINES) {
+  // the lane-split form needs 17 FP64 instructions a block on nlines / 2 warps, one
+  // thread per line about 120 on nlines / 32: the split's time grows with the lines
+  // once they fill the SM quarters (8 lines an SM) and reaches the other's near 47 an
+  // SM (us, 16 blocks a line, 152 SMs: 6144 lines 74 against 82, 7168 80 against 82, 8192
+  // 92 against 83)
+  if (nlines <= 47 * s_nsm[dev]) {
     k_block_thomas_split<<<(nlines + 1) / 2, 32, 0, st>>>(nlines, n, A, B, C, d, x, s_scratch[dev]);
   } else {
     int threads = 32;

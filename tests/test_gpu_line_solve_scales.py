@@ -10,7 +10,7 @@ import paper_2004_13887_gb300 as sph
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nl", [5, 20001])   # 16 lanes a line, one thread a line
+@pytest.mark.parametrize("nl", [5, 7144, 7145, 20001])   # 16 lanes a line, one thread a line (from 7145 on 152 SMs)
 @pytest.mark.parametrize("blocks,sol", [(330, 100), (-330, -100), (330, -300), (-330, 300), (0, 600), (0, -600)])
 def test_power_of_two_scales(nl, blocks, sol):
     import torch
