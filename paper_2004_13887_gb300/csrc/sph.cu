@@ -969,22 +969,23 @@ template <typename R>
 static constexpr int sweep_block() { return sizeof(R) == sizeof(double) ? 32 : 128; }
 
 // Whether the many-lines solver (sph_lines2.cuh) takes the sweep along d of the
-// mixed mode (with the default line solver).  Lengths the partitioned solver
-// takes: r and theta with enough lines to fill the SMs (measured at 5 to 50 us
-// a sweep's launch, many-lines against partitioned: r, 4096 lines of 16 cells 14.3
-// vs 13.8 us, 8192 of 32 22 vs 26, 16384 of 64 49 vs 63; theta, 8192 lines of 128
-// 74 vs 70, 9216 of 192 114 vs 109, 16384 of 192 144 vs 181; 32768 of 256 376 vs
-// 496; phi 740 + 220 vs 345 + 195: not taken).  Other lengths, where the
-// alternative is one thread a line: any direction from 1024 lines (30 x 60 x 60:
-// 20 vs 43, 31 vs 87, 48 vs 176 us; 100 x 200 x 200: 165 vs 247, 188 vs 437, 350 vs
-// 1268); fewer lines gain little and keep the one-sided elimination, the more
-// accurate one on long stiff lines (512 cells: 6.6e-6 vs 1.1e-5).
+// mixed mode (with the default line solver).  Lengths the partitioned solver takes:
+// r and theta with enough lines to fill the SMs.  Measured, us a sweep, many-lines
+// against partitioned: r, 10240 lines of 16, 32, 64, 128, 192, 256 cells 15 vs 22, 23 vs
+// 31, 43 vs 44, 83 vs 93, 123 vs 113, 164 vs 176; theta 15 vs 21, 22 vs 31, 41 vs 44, 80
+// vs 91, 122 vs 115, 163 vs 170; 12288 lines of 192 cells 132 vs 133 and 128 vs 135; 8192
+// lines of 64 cells and more 3 to 30 % behind.  (Phi 740 + 220 vs 345 + 195 at 128 x
+// 256 x 256: not taken.)  Other lengths, where the alternative is one thread a line:
+// any direction from 1024 lines of 4 cells (1155 lines of 4, 20, 100 cells: r 9.5 vs
+// 10.4, 15 vs 33, 46 vs 146; walled phi 12 vs 16, 22 vs 60, 76 vs 312; cyclic phi 20 vs
+// 26, 40 vs 108, 188 vs 555; 10201 lines of 3 cells 10.1 vs 10.1, 16 vs 15, 25 vs 24).
 static int lines2_use(const sph_ctx* c, int d) {
   if (c->line_solver != SPH_LINES_PARTITIONED) return 0;
   const Geo<double>& g = c->d64.g;
   const long lines = d == 2 ? (long)g.nr * g.nt : (long)(d == 0 ? g.nt : g.nr) * g.np;
-  if (!lines_ok(c, d)) return lines >= LINES2_MIN_OTHER;
-  return d < 2 && lines >= LINES2_MIN;
+  const int n = d == 0 ? g.nr : d == 1 ? g.nt : g.np;
+  if (!lines_ok(c, d)) return n >= LINES2_MIN_CELLS && lines >= LINES2_MIN_OTHER;
+  return d < 2 && lines >= (n == 192 ? LINES2_MIN_192 : LINES2_MIN);
 }
 
 // Whether the FP64 sweeps take the one-thread-per-line solver: by choice, or for a

@@ -20,17 +20,20 @@
 // the one-sided solver's error in u on long stiff lines: from below, a cell's
 // pressure is then eliminated before the face that its flux leaves by.  Against FP64,
 // lines of 512 and 200 stiff cells along r, smooth right-hand side: 1.7e-3 and 1.6e-4
-// then, 2.9e-4 and 6.3e-5 now, 3.9e-4 and 7.8e-5 one-sided.)  Any length n >= 2.  (E, g)
+// then, 2.9e-4 and 6.3e-5 now, 3.9e-4 and 7.8e-5 one-sided.)  Any length n >= 4.  (E, g)
 // of a side's cells go to a scratch region of the block (12 floats a cell,
 // lane-interleaved: 128-byte rows), read back in reverse and then discarded from L2.
 #pragma once
 
 #include "sph_blk3.cuh"
 
-// Lines from which these kernels are the faster ones along r and theta (below, the
-// partitioned solver has more lanes a line), where that solver takes the length.
+// Lines from which these kernels are the faster ones along r and theta, where the
+// partitioned solver takes the length (lines of 192 cells: from more), and lines and
+// cells from which they are where it does not (the measurements: lines2_use).
 #define LINES2_MIN 10240
+#define LINES2_MIN_192 12288
 #define LINES2_MIN_OTHER 1024
+#define LINES2_MIN_CELLS 4
 #ifndef LINES2_MINB
 #define LINES2_MINB 8
 #endif
@@ -347,7 +350,6 @@ __device__ __forceinline__ void eliminate(const Args& A, int a, int b, int n, in
     const float* w = ring + (cnt % FWD) * (NV * 32);      // (arrived with cell cnt - 1)
     form_cell<D>(A, row(cnt)[0], row(cnt)[1], th, uf, w[V_U * 32], w[V_GRR * 32], w[V_GTT * 32], w[V_GPP * 32],
                  D == 1 ? w[V_S1 * 32] : 0.f, 0.f, mid->a, mid->b, mid->c);
-    if (cnt == n - 1) { mid->b[0] += mid->c[0]; mid->b[1] += mid->c[1]; mid->b[4] += mid->c[4]; }   // two cells: a wall above
     mid->y[0] = w[V_R0 * 32];
     mid->y[1] = w[V_R4 * 32];
   }
@@ -373,9 +375,6 @@ __device__ __forceinline__ void block_lines(const Args& A, float (*ex)[32], floa
   if (side == 0) {
     eliminate<D, 0>(A, a, b, n, cnt, ring, scr, E, gv, &mid, &sing);
   } else {
-#pragma unroll
-    for (int k = 0; k < 9; k++) E[k] = 0.f;               // (no cell above the middle one of two)
-    gv[0] = gv[1] = gv[2] = 0.f;
     eliminate<D, 1>(A, a, b, n, cnt, ring, scr, E, gv, nullptr, &sing);
 #pragma unroll
     for (int k = 0; k < 9; k++) ex[k][lane] = E[k];
@@ -571,12 +570,11 @@ __device__ __forceinline__ void scalar_lines(const Args& A, float (*ex)[32], flo
 // Z X are FP64, as in the one-thread-per-line solver: y and Z X cancel where the
 // ring is stiff, and the increment reaches the FP64 state unrounded.
 
-// the first cell of the bottom side of N >= 2 cells (its walled line's middle cell is
-// the one before; past the last cell of a line of two)
-template <bool CYC>
+// the first cell of the bottom side of N cells (3 and more); a walled line's middle cell
+// is the one before
 __device__ __forceinline__ int phi_split(int N) {
-  const int h = (N + 1) / 2, c = (h + 3) & ~3;
-  return c < N ? c : CYC ? h : N / 2 + 1;
+  const int c = ((N + 1) / 2 + 3) & ~3;
+  return c < N ? c : N / 2 + 1;
 }
 
 template <bool VEC>
@@ -667,7 +665,6 @@ __device__ __forceinline__ void eliminate_phi(const Args& A, int i, int j, int N
         th = t1;
       }
       if (!CYC && !SIDE && m == hi - 1) {                 // the middle cell
-        if (m == n - 1) { Bb[0] += Cb[0]; Bb[1] += Cb[1]; Bb[4] += Cb[4]; }   // two cells: a wall above
 #pragma unroll
         for (int k = 0; k < 6; k++) { mid->a[k] = Ab[k]; mid->b[k] = Bb[k]; mid->c[k] = Cb[k]; }
         mid->y[0] = y[0];
@@ -759,7 +756,7 @@ __device__ __forceinline__ void block_lines_phi_walled(const Args& A, float (*ex
   const bool valid = l0 < nl;
   const int line = valid ? l0 : nl - 1, i = line / g.nt, j = line - i * g.nt;
   // the sides' cells, the middle one the top side's last
-  const int c = phi_split<false>(n), lo = side ? c : 0, hi = side ? n : c;
+  const int c = phi_split(n), lo = side ? c : 0, hi = side ? n : c;
   const int ic = IC(g, i, j, 0), fc = IPf(g, i, j, 0);
   float* scr = A.scr + (size_t)blk * n * (12 * 32) + lane;
   float E[9], gv[3], x[3];
@@ -768,10 +765,7 @@ __device__ __forceinline__ void block_lines_phi_walled(const Args& A, float (*ex
   if (side == 0) {
     eliminate_phi<0, false, VEC>(A, i, j, n, lo, hi, scr, E, gv, nullptr, &mid, &sing);
   } else {
-#pragma unroll
-    for (int k = 0; k < 9; k++) E[k] = 0.f;               // (no cell above the middle one of two)
-    gv[0] = gv[1] = gv[2] = 0.f;
-    if (lo < hi) eliminate_phi<1, false, VEC>(A, i, j, n, lo, hi, scr, E, gv, nullptr, nullptr, &sing);
+    eliminate_phi<1, false, VEC>(A, i, j, n, lo, hi, scr, E, gv, nullptr, nullptr, &sing);
 #pragma unroll
     for (int k = 0; k < 9; k++) ex[k][lane] = E[k];
 #pragma unroll
@@ -796,7 +790,7 @@ __device__ __forceinline__ void block_lines_phi_walled(const Args& A, float (*ex
   if (side) { x[0] = ex[12][lane]; x[1] = ex[13][lane]; x[2] = ex[14][lane]; }
   // substitution outwards, group by group
   const int dir = side ? 1 : -1, m_in = side ? lo : hi - 2;   // the first cell with factors
-  if (lo < hi) {
+  {
     float En[9], gn[3], out[3][4];
     auto fetch = [&](int m) {
       const float* sp = scr + (size_t)m * (12 * 32);
@@ -859,7 +853,7 @@ __device__ __forceinline__ void block_lines_phi_ring(const Args& A, float (*ex)[
   const int nl = g.nr * g.nt, l0 = blk * 32 + lane;
   const bool valid = l0 < nl;
   const int line = valid ? l0 : nl - 1, i = line / g.nt, j = line - i * g.nt;
-  const int c = phi_split<true>(N), lo = side ? c : 0, hi = side ? N : c;
+  const int c = phi_split(N), lo = side ? c : 0, hi = side ? N : c;
   constexpr int W = 21;
   float* scr = A.scr + (size_t)blk * n * (W * 32) + lane;
   float E[9], gv[3], H[9];
@@ -1008,7 +1002,7 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
   const int nj = CC == 1 ? g.nt - 1 : g.nt, nl = (CC == 0 ? g.nr - 1 : g.nr) * nj, l0 = blk * 32 + lane;
   const bool valid = l0 < nl;
   const int line = valid ? l0 : nl - 1, i = line / nj + (CC == 0), j = line % nj + (CC == 1);
-  const int c = phi_split<true>(N), lo = side ? c : 0, hi = side ? N : c;
+  const int c = phi_split(N), lo = side ? c : 0, hi = side ? N : c;
   float* scr = A.scr + (size_t)A.nb0 * n * ((CYC ? 21 : 12) * 32) + (size_t)slot * n * (W * 32) + lane;
   const int p0 = CC == 0 ? IC(g, i - 1, j, 0) : IC(g, i, j - 1, 0), p1 = IC(g, i, j, 0);
   const int fx = CC == 0 ? IRf(g, i, j, 0) : ITf(g, i, j, 0);
@@ -1043,7 +1037,7 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
       if (CYC) sp[64] = hz;
     }
   };
-  if (lo < hi) {
+  {
     G5 cg, nx;
     int gr = side ? (hi - 1) / 4 : 0;
     const int ge = side ? lo / 4 : (hi - 1) / 4;
@@ -1086,7 +1080,7 @@ __device__ __forceinline__ void scalar_lines_phi(const Args& A, float (*ex)[32],
   };
   const bool wl = CC == 0 ? i == 1 : j == 1, wh = CC == 0 ? i == g.nr - 1 : j == g.nt - 1;
   const int ms = side ? lo : hi - 1, dir = side ? 1 : -1;
-  if (lo < hi) {
+  {
     float en = 0.f, gn = 0.f, hn = 0.f, out[4];
     auto fetch = [&](int m) {
       const float* sp = scr + (size_t)m * (W * 32);
