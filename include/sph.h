@@ -175,10 +175,13 @@ int sph_batch_create(sph_ctx* const* ctxs, int n, void* stream, sph_batch** out)
 int sph_batch_capture(sph_batch* batch, double dt, int n_iter, int steps);
 /* sph_batch_capture_fused: the same graph of `steps` steps built from batched
  * launches instead of per-context ones -- each stage of an iteration (Ubar,
- * coefficients, the four right-hand-side kernels, and per sweep one block-line
- * and one scalar-line launch for each line layout present) is ONE kernel over
+ * coefficients, right-hand side, and per sweep one block-line and one
+ * scalar-line launch for each line layout present) is ONE kernel over
  * every context, reading a per-context descriptor table and a per-block map
- * (context, tile or line group) from device memory the batch allocates.  The
+ * (context, tile or line group) from device memory the batch allocates.  From
+ * 10240 r lines (theta lines) in all contexts together, the r (theta) sweep takes
+ * the many-lines kernels for every context, and a context's sph_set_line_solver
+ * counts for its other sweeps only.  The
  * results are those of per-context steps to FP32 rounding (the same device
  * code, compiled into other kernels).  Every context must be
  * in SPH_PREC_MIXED mode with a partitioned line solver that takes all three

@@ -176,9 +176,9 @@ __global__ void __launch_bounds__(CB / P, 65536 * P / (CB * 48)) k_lines_sca_f(c
   else lines::lines_sca<D, P, L, CB, 2>(S, m.y - ng1);
 }
 
-// The r- (D = 0) and theta-lines (1) of every problem, of any length, 32 lines a
-// block (sph_lines2.cuh): one launch for the block lines and one for the scalar
-// lines over all problems; map = (problem, block of its launch).
+// The r- (D = 0) and theta-lines (1) of every problem, 32 lines a block
+// (sph_lines2.cuh): one launch for the block lines and one for the scalar lines over
+// all problems; map = (problem, block of its launch).
 template <int D>
 __global__ void __launch_bounds__(64, LINES2_MINB) k_l2_blk_f(const lines2::Args* tab, const int2* map) {
   __shared__ lines2::Args S;
@@ -426,8 +426,12 @@ extern "C" int sph_batch_capture_fused(sph_batch* b, double dt, int n_iter, int 
   std::vector<Layout> lay;
   std::vector<fused::LineTab> ltab[64][2][2];   // per layout (at most 3 x 15 exist)
   std::vector<int2> lmb[64], lms[64];
-  // r and theta: lines of any length in one pair of launches where the batch has
-  // enough of them to fill the SMs, as for a single problem (lines2_use)
+  // r and theta: the lines of all problems, whatever their lengths, in one pair of
+  // launches where the batch has enough of them to fill the SMs.  A problem's own
+  // choice among the partitioned layouts then counts for its phi lines alone: a pair of
+  // launches for every layout chosen costs what the layouts gain (the ensemble of 64, 4
+  // of 45 grids with the one-warp layout: 33.33 ms a step with their own launches, 33.28
+  // without; 12 instances 7.16 against 7.05).
   bool two[3] = {false, false, false};
   std::vector<lines2::Args> l2tab[2];
   std::vector<int2> l2b[2], l2s[2];
