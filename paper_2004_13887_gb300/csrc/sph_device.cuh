@@ -6,11 +6,13 @@
 //
 // Rows of the split operators, with coefficients frozen at Ubar (eq.
 // chapter3mainsd) and moved to staggered points by arithmetic means:
-//   row_c : p-row (A1^d, A2^d, A3^d) or T-row (C2^d, C3^d) at a cell centre;
-//   row_f : normal-velocity row (B1^d, B2^{d,d}) on a d-face;
-//   row_s : transverse row B2^{d,c} of velocity component c along d;
-//   D_M   : cross derivatives, curvature, Coriolis, the off-line parts of
-//           grad(div v)/3 and of the vector Laplacian (explicit, in k_rhs).
+//   row_cw : p-row (A1^d, A2^d, A3^d) or T-row (C2^d, C3^d) at a cell centre;
+//   row_fw : normal-velocity row (B1^d, B2^{d,d}) on a d-face;
+//   row_sw : transverse row B2^{d,c} of velocity component c along d;
+//   D_M    : cross derivatives, curvature, Coriolis, the off-line parts of
+//            grad(div v)/3 and of the vector Laplacian (explicit, in the right-hand side).
+// (for the one-thread-per-line solver; the other kernels form the same rows from
+// tables: sph_fp64.cuh, sph_stencil32.cuh, sph_lines2.cuh)
 // The viscous-heating linearisation follows A2/C2 of Appendix B except that the
 // G_phiphi*cot(theta) term printed in A2^phi / C2^phi is dropped: it does not
 // follow from grad(u):sigma(v) (only A2^theta has it).
@@ -127,10 +129,6 @@ __device__ __forceinline__ void d2ff(double d, float& hi, float& lo) {
 }
 // the nearest float of a double
 __device__ __forceinline__ float d2f(double d) { float h, l; d2ff(d, h, l); return h; }
-// a double in the bulk type R (exact for R = double)
-template <typename R> __device__ __forceinline__ R to_bulk(double d) { return (R)d; }
-template <> __device__ __forceinline__ float to_bulk<float>(double d) { return d2f(d); }
-
 // s + e = a + b exactly (Knuth)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;
@@ -219,67 +217,58 @@ template <typename G> __device__ __forceinline__ int wrapk(const G& g, int k) { 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 // ---------------------------------------------------------------- accessors
-// CIJ = 0 skips the checks on i and j: for points whose +-2 neighbourhood in
-// r and theta is inside the grid (the kernels decide this per block, so warps
-// do not diverge); k (phi) is always checked.
-//
 // Centre perturbation with zero Neumann ghosts (the background has its own).
 template <typename P> using ValOf = typename std::decay<decltype(std::declval<P>()[0])>::type;
 
 template <int CIJ = 2, typename G, typename P>
 __device__ __forceinline__ ValOf<P> cpert(const G& g, const P& f, int i, int j, int k) {
-  int ii = CIJ ? clampi(i, 0, g.nr - 1) : i, jj = CIJ ? clampi(j, 0, g.nt - 1) : j;
   int kk = g.per ? wrapk(g, k) : clampi(k, 0, g.np - 1);
-  return f[IC(g, ii, jj, kk)];
+  return f[IC(g, clampi(i, 0, g.nr - 1), clampi(j, 0, g.nt - 1), kk)];
 }
 // Velocities with Dirichlet ghosts on tangential walls: ghost = 2 w - interior
-// (w = 0, no-slip, unless wall data were set).  CIJ = 0: interior points, no
-// checks on i and j and the homogeneous rule for the phi walls; 1: checked,
-// homogeneous walls; 2: checked, wall data read (the kernels send every tile
-// to 2 when wall data are set and are instantiated without it otherwise, so
-// the other paths carry no wall code).
+// (w = 0, no-slip, unless wall data were set).  CIJ = 1: homogeneous walls; 2: wall
+// data read (the mixed mode's kernels send every tile to 2 when wall data are set and
+// are instantiated without it otherwise, so that the other paths carry no wall code).
 template <int CIJ = 2, typename G, typename P>
 __device__ __forceinline__ ValOf<P> vr(const G& g, const P& u, int i, int j, int k) {
-  if (CIJ && j < 0) return WALL2(0, 1, 0, i * g.np + k) - u[IRf(g, i, 0, k)];
-  if (CIJ && j >= g.nt) return WALL2(0, 1, 1, i * g.np + k) - u[IRf(g, i, g.nt - 1, k)];
+  if (j < 0) return WALL2(0, 1, 0, i * g.np + k) - u[IRf(g, i, 0, k)];
+  if (j >= g.nt) return WALL2(0, 1, 1, i * g.np + k) - u[IRf(g, i, g.nt - 1, k)];
   if (k < 0 || k >= g.np) {
     if (g.per) k = wrapk(g, k);
-    else if constexpr (CIJ != 0) return WALL2(0, 2, k >= g.np, i * g.nt + j) - u[IRf(g, i, j, k < 0 ? 0 : g.np - 1)];
-    else return -u[IRf(g, i, j, k < 0 ? 0 : g.np - 1)];
+    else return WALL2(0, 2, k >= g.np, i * g.nt + j) - u[IRf(g, i, j, k < 0 ? 0 : g.np - 1)];
   }
   return u[IRf(g, i, j, k)];
 }
 template <int CIJ = 2, typename G, typename P>
 __device__ __forceinline__ ValOf<P> vt(const G& g, const P& u, int i, int j, int k) {
-  if (CIJ && i < 0) return WALL2(1, 0, 0, j * g.np + k) - u[ITf(g, 0, j, k)];
-  if (CIJ && i >= g.nr) return WALL2(1, 0, 1, j * g.np + k) - u[ITf(g, g.nr - 1, j, k)];
+  if (i < 0) return WALL2(1, 0, 0, j * g.np + k) - u[ITf(g, 0, j, k)];
+  if (i >= g.nr) return WALL2(1, 0, 1, j * g.np + k) - u[ITf(g, g.nr - 1, j, k)];
   if (k < 0 || k >= g.np) {
     if (g.per) k = wrapk(g, k);
-    else if constexpr (CIJ != 0) return WALL2(1, 2, k >= g.np, i * (g.nt + 1) + j) - u[ITf(g, i, j, k < 0 ? 0 : g.np - 1)];
-    else return -u[ITf(g, i, j, k < 0 ? 0 : g.np - 1)];
+    else return WALL2(1, 2, k >= g.np, i * (g.nt + 1) + j) - u[ITf(g, i, j, k < 0 ? 0 : g.np - 1)];
   }
   return u[ITf(g, i, j, k)];
 }
 template <int CIJ = 2, typename G, typename P>
 __device__ __forceinline__ ValOf<P> vp(const G& g, const P& u, int i, int j, int k) {
   if (g.per) k = wrapk(g, k);
-  if (CIJ && i < 0) return WALL2(2, 0, 0, j * g.npf + k) - u[IPf(g, 0, j, k)];
-  if (CIJ && i >= g.nr) return WALL2(2, 0, 1, j * g.npf + k) - u[IPf(g, g.nr - 1, j, k)];
-  if (CIJ && j < 0) return WALL2(2, 1, 0, i * g.npf + k) - u[IPf(g, i, 0, k)];
-  if (CIJ && j >= g.nt) return WALL2(2, 1, 1, i * g.npf + k) - u[IPf(g, i, g.nt - 1, k)];
+  if (i < 0) return WALL2(2, 0, 0, j * g.npf + k) - u[IPf(g, 0, j, k)];
+  if (i >= g.nr) return WALL2(2, 0, 1, j * g.npf + k) - u[IPf(g, g.nr - 1, j, k)];
+  if (j < 0) return WALL2(2, 1, 0, i * g.npf + k) - u[IPf(g, i, 0, k)];
+  if (j >= g.nt) return WALL2(2, 1, 1, i * g.npf + k) - u[IPf(g, i, g.nt - 1, k)];
   return u[IPf(g, i, j, k)];
 }
-template <int CIJ = 2, typename G, typename P>
+template <typename G, typename P>
 __device__ __forceinline__ ValOf<P> hr(const G& g, const P& u, int i, int j, int k) {
-  return ValOf<P>(0.5) * (vr<CIJ>(g, u, i, j, k) + vr<CIJ>(g, u, i + 1, j, k));
+  return ValOf<P>(0.5) * (vr(g, u, i, j, k) + vr(g, u, i + 1, j, k));
 }
-template <int CIJ = 2, typename G, typename P>
+template <typename G, typename P>
 __device__ __forceinline__ ValOf<P> ht(const G& g, const P& u, int i, int j, int k) {
-  return ValOf<P>(0.5) * (vt<CIJ>(g, u, i, j, k) + vt<CIJ>(g, u, i, j + 1, k));
+  return ValOf<P>(0.5) * (vt(g, u, i, j, k) + vt(g, u, i, j + 1, k));
 }
-template <int CIJ = 2, typename G, typename P>
+template <typename G, typename P>
 __device__ __forceinline__ ValOf<P> hp(const G& g, const P& u, int i, int j, int k) {
-  return ValOf<P>(0.5) * (vp<CIJ>(g, u, i, j, k) + vp<CIJ>(g, u, i, j, k + 1));
+  return ValOf<P>(0.5) * (vp(g, u, i, j, k) + vp(g, u, i, j, k + 1));
 }
 template <typename R>
 __device__ __forceinline__ R rho_at(const Geo<R>& g, const Coef<R>& c, int i, int j, int k) {
@@ -287,59 +276,10 @@ __device__ __forceinline__ R rho_at(const Geo<R>& g, const Coef<R>& c, int i, in
   return c.rho[IC(g, i, j, k)];
 }
 
-// A velocity component averaged to centre (i, j, k): in interior blocks
-// (CIJ = 0) read from the coefficient plane k_coef wrote (uc0/uc1/uc2, the
-// same FP32 operations, so the same value), with the no-slip ghost -- minus the
-// mirrored centre -- beyond a phi wall (interior blocks run only without wall
-// data) and the periodic wrap (only used for the components tangential to phi);
-// elsewhere the face average with all checks.
-template <int CC, typename R>
-__device__ __forceinline__ R ucen(const Geo<R>& g, const R* plane, int i, int j, int k) {
-  if (k < 0 || k >= g.np) {
-    if (g.per) k = wrapk(g, k);
-    else return -plane[IC(g, i, j, k < 0 ? 0 : g.np - 1)];
-  }
-  return plane[IC(g, i, j, k)];
-}
-template <int CIJ, typename R, typename P>
-__device__ __forceinline__ R hrc(const Geo<R>& g, const Coef<R>& c, const P& u, int i, int j, int k) {
-  if constexpr (CIJ != 0) return hr<CIJ>(g, u, i, j, k);
-  else return ucen<0>(g, c.uc0, i, j, k);
-}
-template <int CIJ, typename R, typename P>
-__device__ __forceinline__ R htc(const Geo<R>& g, const Coef<R>& c, const P& u, int i, int j, int k) {
-  if constexpr (CIJ != 0) return ht<CIJ>(g, u, i, j, k);
-  else return ucen<1>(g, c.uc1, i, j, k);
-}
-template <int CIJ, typename R, typename P>
-__device__ __forceinline__ R hpc(const Geo<R>& g, const Coef<R>& c, const P& u, int i, int j, int k) {
-  if constexpr (CIJ != 0) return hp<CIJ>(g, u, i, j, k);
-  else return ucen<2>(g, c.uc2, i, j, k);
-}
-
 // whether the +-2 neighbourhood of (i, j) in r and theta is inside the grid
 template <typename G>
 __device__ __forceinline__ bool inner_ij(const G& g, int i, int j) {
   return i >= 2 && i <= g.nr - 3 && j >= 2 && j <= g.nt - 3;
-}
-
-// --------------------------------------------------------- thermodynamics
-// Coefficients of a centre from the midpoint perturbations p', T' and the
-// background at radius index i; k_coef and the line kernels both call this, so
-// their values are the same.
-template <typename R>
-struct Thermo { R Pb, Tb, rho, beta; };
-template <typename R>
-__device__ __forceinline__ Thermo<R> thermo(const Geo<R>& g, const Par& P, int i, R pp, R Tp) {
-  R pref = g.pcen[i], Tref = g.Tcen[i];
-  Thermo<R> t;
-  t.Pb = pref + pp;
-  t.Tb = Tref + Tp;
-  R iRg = pick<R>(1.0 / P.Rg, P.iRg_f);
-  R itb = sdiv(R(1), t.Tb);
-  t.rho = t.Pb * itb * iRg;
-  t.beta = sdiv((pick<R>(P.gamma, P.gamma_f) - R(1)) * t.Tb, t.Pb);
-  return t;
 }
 
 // ------------------------------------------------------------------- rows
@@ -438,12 +378,6 @@ __device__ __forceinline__ void row_cw(const Geo<R>& g, const Par& P, const CPt<
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void row_c(const Geo<R>& g, const Par& P, const Coef<R>& c, int d, int isT, int i, int j,
-                                      int k, RowC<R>& w) {
-  row_cw(g, P, load_c(c, d, IC(g, i, j, k)), d, isT, i, j, w);
-}
-
 // Normal-velocity row of D_d on the d-face (i,j,k): p at centres m-1, m and
 // u_d on faces m-1, m, m+1.  It reads rho at the two centres and Ubar's u_d on
 // the face.
@@ -500,30 +434,24 @@ __device__ __forceinline__ void row_fw(const Geo<R>& g, const Par& P, const FPt<
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void row_f(const Geo<R>& g, const Par& P, const Coef<R>& c, const R* ubd, int d, int i,
-                                      int j, int k, R wp[2], R wu[3]) {
-  row_fw(g, P, load_f(g, c, ubd, d, i, j, k), d, i, j, wp, wu);
-}
-
 // Transverse row of D_d for velocity component cc at its location (i,j,k): it
 // reads rho at the two centres beside the face and the advecting Ubar component.
 template <typename R>
 struct SPt { R rho0, rho1, ua; };
 
-template <int CIJ = 2, typename R>
+template <typename R>
 __device__ __forceinline__ SPt<R> load_s(const Geo<R>& g, const Coef<R>& c, const CF<R>& ub, int cc, int d, int i,
                                          int j, int k) {
   SPt<R> q;
   if (cc == 0) { q.rho0 = rho_at(g, c, i - 1, j, k); q.rho1 = rho_at(g, c, i, j, k); }
   else if (cc == 1) { q.rho0 = rho_at(g, c, i, j - 1, k); q.rho1 = rho_at(g, c, i, j, k); }
   else { q.rho0 = rho_at(g, c, i, j, k - 1); q.rho1 = rho_at(g, c, i, j, k); }
-  if (cc == 0) q.ua = d == 1 ? R(0.5) * (htc<CIJ>(g, c, ub.f[2], i - 1, j, k) + htc<CIJ>(g, c, ub.f[2], i, j, k))
-                             : R(0.5) * (hpc<CIJ>(g, c, ub.f[3], i - 1, j, k) + hpc<CIJ>(g, c, ub.f[3], i, j, k));
-  else if (cc == 1) q.ua = d == 0 ? R(0.5) * (hrc<CIJ>(g, c, ub.f[1], i, j - 1, k) + hrc<CIJ>(g, c, ub.f[1], i, j, k))
-                                  : R(0.5) * (hpc<CIJ>(g, c, ub.f[3], i, j - 1, k) + hpc<CIJ>(g, c, ub.f[3], i, j, k));
-  else q.ua = d == 0 ? R(0.5) * (hrc<CIJ>(g, c, ub.f[1], i, j, k - 1) + hrc<CIJ>(g, c, ub.f[1], i, j, k))
-                     : R(0.5) * (htc<CIJ>(g, c, ub.f[2], i, j, k - 1) + htc<CIJ>(g, c, ub.f[2], i, j, k));
+  if (cc == 0) q.ua = d == 1 ? R(0.5) * (ht(g, ub.f[2], i - 1, j, k) + ht(g, ub.f[2], i, j, k))
+                             : R(0.5) * (hp(g, ub.f[3], i - 1, j, k) + hp(g, ub.f[3], i, j, k));
+  else if (cc == 1) q.ua = d == 0 ? R(0.5) * (hr(g, ub.f[1], i, j - 1, k) + hr(g, ub.f[1], i, j, k))
+                                  : R(0.5) * (hp(g, ub.f[3], i, j - 1, k) + hp(g, ub.f[3], i, j, k));
+  else q.ua = d == 0 ? R(0.5) * (hr(g, ub.f[1], i, j, k - 1) + hr(g, ub.f[1], i, j, k))
+                     : R(0.5) * (ht(g, ub.f[2], i, j, k - 1) + ht(g, ub.f[2], i, j, k));
   return q;
 }
 
@@ -549,10 +477,10 @@ __device__ __forceinline__ void row_sw(const Geo<R>& g, const Par& P, const SPt<
   }
 }
 
-template <int CIJ = 2, typename R>
+template <typename R>
 __device__ __forceinline__ void row_s(const Geo<R>& g, const Par& P, const Coef<R>& c, const CF<R>& ub, int cc, int d,
                                       int i, int j, int k, R w[3]) {
-  row_sw(g, P, load_s<CIJ>(g, c, ub, cc, d, i, j, k), cc, d, i, j, w);
+  row_sw(g, P, load_s(g, c, ub, cc, d, i, j, k), cc, d, i, j, w);
 }
 
 }  // namespace sph

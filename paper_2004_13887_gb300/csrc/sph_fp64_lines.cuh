@@ -239,7 +239,7 @@ __device__ __forceinline__ void eliminate(const LineArgs& S, const Cells<D, CYC>
     Z.load(m, rb);
     Z.load_rhs(m, r);
   };
-  if (cnt > 0) fetch(SIDE ? N - 1 : 0);
+  fetch(SIDE ? N - 1 : 0);
   for (int s = 0; s < cnt; s++) {
     const int m = SIDE ? N - 1 - s : s;
     double A[9], B[9], C[9], y[3];
@@ -310,13 +310,9 @@ __device__ __forceinline__ void block_line(const LineArgs& S, double (*ex)[32], 
   constexpr int W = CYC ? 21 : 12;
   double* scr = S.scr + S.scr_off[0];
   double E[9], g[3], H[9];
-#pragma unroll
-  for (int q = 0; q < 9; q++) { E[q] = 0.0; H[q] = 0.0; }
-  g[0] = g[1] = g[2] = 0.0;
   if (side == 0) eliminate<D, CYC, TR, 0>(S, Z, N, cnt, line, valid, E, g, H, bad);
   else eliminate<D, CYC, TR, 1>(S, Z, N, cnt, line, valid, E, g, H, bad);
-  // the meeting cells (the empty bottom side of a one-cell line has zero
-  // factors, which leave x = g - H X on the top side)
+  // the meeting cells (N >= 2: a cell on either side)
   {
     double* mine = &ex[side * NEX][lane];
 #pragma unroll
@@ -436,13 +432,11 @@ __device__ __forceinline__ void block_line(const LineArgs& S, double (*ex)[32], 
     }
 #pragma unroll
     for (int q = 0; q < 3; q++) v[q] = r[q] * S.ih;
-    // y and Z of the line's first cell (the top side's) and its last (the
-    // bottom side's, or the top's when it holds the only cell)
-    const int lo = 0, hi = N - h > 0 ? 1 : 0;
+    // y and Z of the line's first cell (the top side's) and its last (the bottom's)
     double Y[9], yv[3];
 #pragma unroll
     for (int e = 0; e < 2; e++) {
-      const double* src = &ex[(e ? hi : lo) * NEX][lane];
+      const double* src = &ex[e * NEX][lane];
 #pragma unroll
       for (int q = 0; q < 9; q++) Y[q] = src[q * 32];
 #pragma unroll
@@ -524,7 +518,7 @@ __device__ __forceinline__ void scalar_line(const LineArgs& S, double (*ex)[32],
     rn = rhs[Z.idx(m)];
   };
   double e = 0.0, gy = 0.0, hz = 0.0;
-  if (cnt > 0) fetch(cell(0));
+  fetch(cell(0));
   for (int s = 0; s < cnt; s++) {
     const int m = cell(s);
     double am = wn[0], bm = wn[1] + S.ih, cm = wn[2], r = rn * S.ih;
@@ -584,9 +578,8 @@ __device__ __forceinline__ void scalar_line(const LineArgs& S, double (*ex)[32],
     double* mine = &ex[side * NEX][lane];
     mine[0] = z; mine[32] = x;
     __syncthreads();
-    const int hi = N - h > 0 ? 1 : 0;
     const double* o0 = &ex[0][lane];
-    const double* o1 = &ex[hi * NEX][lane];
+    const double* o1 = &ex[NEX][lane];
     const double am = TR ? Z.w(n - 2, 2) : Z.w(n - 1, 0), cm = TR ? Z.w(0, 0) : Z.w(n - 1, 2);
     const double den = fma(-cm, o0[0], fma(-am, o1[0], Z.w(n - 1, 1) + S.ih));
     if (bad_pivot(den)) *bad |= FLAG_SINGULAR;
@@ -680,10 +673,10 @@ __device__ __forceinline__ void block_line_split(const LineArgs& S, int line, bo
   // both sides run the same instructions for the same count (the longer, top
   // side's); a side that has finished repeats its last cell without a store
   // and keeps its factors
-  if (cnt > 0) fetch(cell(0));
+  fetch(cell(0));
   for (int s = 0; s < h; s++) {
     const bool live = s < cnt;
-    const int m = live ? cell(s) : cell(cnt > 0 ? cnt - 1 : 0);
+    const int m = cell(live ? s : cnt - 1);
     double A[9], B[9], C[9], t[3], u[3];
     Z.form(ra, A);
     Z.form(rc, C);

@@ -1,8 +1,7 @@
-// sph_kernels.cuh -- the device code of the scheme's stages (Section 2.2,
-// eqs. chapter3mainsd, splitting2, spl1-spl3; operators of Appendix B): the
-// averaging, coefficient and right-hand-side kernels and the one-thread-per-
-// line block and scalar line solvers, shared by the single-problem library
-// (sph.cu) and the batched launches over many problems (sph_batch.cu).
+// sph_kernels.cuh -- device code of the scheme's stages (Section 2.2, eqs.
+// chapter3mainsd, splitting2, spl1-spl3) that every part of the library shares: the
+// averaging kernel, the one-thread-per-line block and scalar line solvers, and what
+// the other line solvers take from them.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -616,7 +615,7 @@ __device__ void scalar_line(const SweepArgs<R>& S, int line, int a, int b, SqSum
   auto fetch = [&](int m) {
     int i, j, k;
     line_pos(d, a, b, m, i, j, k);
-    qn = load_s<2>(g, S.c, S.ub, cc, d, i, j, k);
+    qn = load_s(g, S.c, S.ub, cc, d, i, j, k);
     rn = rhs[face_idx(g, cc, i, j, k)];
   };
   if constexpr (!TR) fetch(0);
