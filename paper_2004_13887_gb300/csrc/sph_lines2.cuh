@@ -577,8 +577,16 @@ __device__ __forceinline__ int phi_split(int N) {
   return c < N ? c : N / 2 + 1;
 }
 
+// (the rows are addressed from their first element: the bounds-checked build looks at
+// the range [m0, m1) of a row of lim values that an access takes)
+__device__ __forceinline__ void row_checked(int f, int m0, int m1, int lim) {
+#ifdef SPH_CHECKED
+  if (m1 > m0) { checked(f, 0, 0, m0, 1, 1, lim, 0); checked(f, 0, 0, m1 - 1, 1, 1, lim, 0); }
+#endif
+}
 template <bool VEC>
 __device__ __forceinline__ void load4(const float* f, int m0, int lim, float* o) {
+  row_checked(0, m0, VEC ? m0 + 4 : m0 + 1, lim);
   if (VEC) {
     const float4 v = *reinterpret_cast<const float4*>(f + m0);
     o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
@@ -700,6 +708,7 @@ __device__ __forceinline__ bool finite_(double v) { return ((unsigned)__double2h
 template <bool VEC, typename V>
 __device__ __forceinline__ void emit4(const Args& A, int f, int at, int m0, int m1, const V* v, SqSum<float>& ss, int* bad) {
   const int g0 = m0 & ~3;
+  row_checked(f & 3, at + m0, at + m1, A.g.nt * (f == 3 ? A.g.nr * A.g.npf : (A.g.nr + (f == 1)) * A.g.np) + (f == 2 ? A.g.nr * A.g.np : 0));
   if (!A.update) {
     float* x = A.x.f[f] + at;
     if (VEC && m1 - m0 == 4) {
@@ -930,11 +939,11 @@ __device__ __forceinline__ void block_lines_phi_ring(const Args& A, float (*ex)[
 #pragma unroll
   for (int q = 0; q < 3; q++) mine[(9 + q) * 32] = x[q];
   __syncthreads();
-  const int ic = IC(g, i, j, 0), fc = IPf(g, i, j, 0), e = ic + n - 1;
+  const int ic = IC(g, i, j, 0), fc = IPf(g, i, j, 0), e = IC(g, i, j, n - 1);
   const float4* tb = reinterpret_cast<const float4*>(A.T.b[2] + (size_t)NB * (i * g.nt + j));
   const Th th = thermo(A, i, A.ub.f[0][e], A.ub.f[4][e]), t0 = thermo(A, i, A.ub.f[0][ic], A.ub.f[4][ic]);
   float Ab[9], Bb[9], Cb[9], r[3] = {A.rhs.f[0][e], A.rhs.f[4][e], A.rhs.f[3][fc]};
-  form<2>(A, tb[0], tb[1], tb[2], th, t0.rho, true, A.ub.f[3][fc + n - 1], A.ub.f[3][fc], A.c.grr[e], A.c.gtt[e],
+  form<2>(A, tb[0], tb[1], tb[2], th, t0.rho, true, A.ub.f[3][IPf(g, i, j, n - 1)], A.ub.f[3][fc], A.c.grr[e], A.c.gtt[e],
           A.c.gpp[e], A.c.srp[e], A.c.stp[e], Ab, Bb, Cb, r);
   double L[9], B[9], Bi[9], X[3], y[3] = {r[0], r[1], r[2]};
 #pragma unroll
