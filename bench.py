@@ -595,7 +595,6 @@ def run_adjoint(args, rank, world, dist):
             fd = (float(J_of(th0 + eps * v)) - float(J_of(th0 - eps * v))) / (2 * eps)
             ad = float(torch.sum(grad * v))
             checks.append(abs(fd - ad) / max(abs(fd), 1e-300))
-    longest, cap = s.tape_use()
     s.close()
     # forward 20 steps + backward (20 recomputed steps + 20 adjoint steps)
     N = g.npoints
@@ -608,7 +607,7 @@ def run_adjoint(args, rank, world, dist):
                                    "potential-temperature perturbation, bubble 96x192x192 + 1e-3 white noise, K=2, "
                                    "dt=1 s, checkpoints every 5 steps", "grid": [g.nr, g.nt, g.np]},
             "forward_s": t1 - t0, "backward_s": t2 - t1, "kinetic_energy": float(J),
-            "fd_check_rel_diff": checks, "tape_longest": longest, "tape_capacity": cap,
+            "fd_check_rel_diff": checks,
             "gpu_launches": launches, "clocks": clocks}
     return line
 
@@ -679,7 +678,7 @@ def main():
         try:
             a = run_adjoint(args, rank, world, dist)
             line["adjoint"] = {k: a[k] for k in ("metric", "value", "unit", "ms_per_step", "forward_s", "backward_s",
-                                                 "fd_check_rel_diff", "tape_longest", "gpu_launches", "clocks")}
+                                                 "fd_check_rel_diff", "gpu_launches", "clocks")}
             line["adjoint"]["workload"] = a["config"]["workload"]
         except Exception as ex:
             line["adjoint"] = {"error": str(ex)}

@@ -214,21 +214,26 @@ int sph_sweep(sph_ctx* ctx, int dir, double dt, const double* const* rhs, double
  * each lane back-substitutes; lines of up to 128 cells take 16 lanes (two
  * lines per warp, chunks of 1 to 8 cells), lines of 192 and 256 take 32
  * (chunks of 6 and 8), phi lines of 512 and 1024 take 64 and 128 lanes (2 and
- * 4 warps, chunks of 8); other lines use the block Thomas path.
+ * 4 warps, chunks of 8).  From 10240 lines along r or theta (12288 of 192 cells),
+ * and from 1024 lines of at least 4 cells of any other length, a lane takes a line
+ * from each of its ends (phi lines in groups of 4 cells; a ring's closing cell and
+ * its increments in FP64); shorter and fewer other lines use the block Thomas path.
  * SPH_LINES_PARTITIONED_WARP: the same with 32 lanes (one line per warp) for
  * the lines of 64 and 128 cells.  SPH_LINES_PARTITIONED_NARROW: fewer lanes and
  * longer chunks for the short lines -- 4 lanes with chunks of 4 for lines of
  * 16 cells, 8 lanes with chunks of 4, 6 and 8 for lines of 32, 48 and 64 --
- * so that less of the work is in the reduction; other lengths as
- * SPH_LINES_PARTITIONED.  SPH_LINES_THOMAS: block (and scalar) Thomas, one thread per
+ * so that less of the work is in the reduction.  Both take the partitioned layout
+ * for any number of lines and block Thomas for the other lengths (batched launches:
+ * sph_batch_capture_fused).  SPH_LINES_THOMAS: block (and scalar) Thomas, one thread per
  * line, with the Woodbury / Sherman-Morrison correction on cyclic lines.  All
  * give the exact solution up to rounding (no pivoting between blocks in any).
- * The FP64 mode always uses block Thomas: with SPH_LINES_THOMAS one thread per
- * line; with any other value (the default) two threads per walled line, one
- * eliminating from each end, the two meeting at the middle cells (a 3x3 solve
- * there), which halves the dependent chain for the same arithmetic; cyclic
- * lines keep one thread and the Woodbury correction.  Returns SPH_ERR_ARG for
- * other values. */
+ * The FP64 mode always uses block Thomas: with SPH_LINES_THOMAS (and for steps
+ * below 1e-60) one thread per line; with any other value (the default) from both
+ * ends of a line, the two sides meeting at the middle cells (a 3x3 solve there),
+ * which halves the dependent chain for the same arithmetic: a lane per line and
+ * side, or with few lines a lane per column of the 3x3 blocks; cyclic lines the
+ * same way around one cell that closes the ring.  Returns SPH_ERR_ARG for other
+ * values. */
 #define SPH_LINES_THOMAS 0
 #define SPH_LINES_PARTITIONED 1
 #define SPH_LINES_PARTITIONED_WARP 2
@@ -237,8 +242,9 @@ int sph_set_line_solver(sph_ctx* ctx, int which);
 
 /* Tile shape of the stencil kernels (coefficients, right-hand side): blocks of
  * 128 threads over 128/(tj*ti) phi points x tj theta rows x ti r rows; tj, ti
- * powers of two with tj*ti <= 8 (SPH_ERR_ARG otherwise).  Default 1 x 1 (one
- * row of 128 phi points).  The results do not depend on it. */
+ * powers of two with tj*ti <= 8 (SPH_ERR_ARG otherwise).  Default: ti = 1 and tj =
+ * 1, 2 or 4, the widest tile with the fewest idle threads at the end of a phi row.
+ * The results do not depend on it. */
 int sph_set_tile(sph_ctx* ctx, int tj, int ti);
 
 /* Number of this library's kernel launches since creation (for accounting). */
@@ -254,8 +260,8 @@ long long sph_launch_count(const sph_ctx* ctx);
 int sph_bounds_report(int* first);
 
 /* Per-kernel timing.  sph_profile(ctx, 1) clears the record and starts timing
- * every kernel stage (one launch, the four of the right-hand side, or the
- * two of a partitioned sweep) with a pair of CUDA events on the context's
+ * every kernel stage (one launch, the four of the FP64 right-hand side, or the two
+ * of a mixed-mode sweep; not the adjoint's transposed sweeps) with a pair of CUDA events on the context's
  * stream, around the side streams' work; 0
  * stops.  sph_profile_read synchronises the stream and writes, for each kernel
  * kind SPH_K_* (SPH_NKERNELS entries), the summed duration in ms and the stage

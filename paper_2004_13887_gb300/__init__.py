@@ -403,7 +403,7 @@ class Solver:
         return lam_in
 
     def tape_use(self):
-        """(longest per-thread tape used by the adjoint so far, capacity)"""
+        """(0, 512): the adjoint records no tape any more (sph_adjoint_tape_use)"""
         a, b = C.c_int(0), C.c_int(0)
         _check(load().sph_adjoint_tape_use(self._h, C.byref(a), C.byref(b)), "sph_adjoint_tape_use")
         return a.value, b.value
@@ -434,9 +434,10 @@ class Solver:
     def set_line_solver(self, which: int):
         """SPH_LINES_PARTITIONED (default), SPH_LINES_PARTITIONED_WARP (one warp per line),
         SPH_LINES_PARTITIONED_NARROW (4 or 8 lanes for lines of 16 to 64 cells) or
-        SPH_LINES_THOMAS for the mixed-precision sweeps.  In the FP64 mode
-        SPH_LINES_THOMAS takes one thread per line and every other value two
-        threads per walled line (elimination from both ends)."""
+        SPH_LINES_THOMAS for the mixed-precision sweeps; the default also takes a
+        lane per line and end where there are many lines (sph_set_line_solver).  In the
+        FP64 mode SPH_LINES_THOMAS takes one thread per line and every other value
+        eliminates every line from both ends."""
         _check(load().sph_set_line_solver(self._h, int(which)), "sph_set_line_solver")
 
     def set_tile(self, tj: int, ti: int):

@@ -11,17 +11,23 @@
 //           of div Ubar)
 //   rhs   : R = -(U^k - U^n) - tau [N(Ubar) + G - S]  (the right-hand side of
 //           eq. spl1 after the linearity of D(Ubar) is used: the D(U^k - U^n),
-//           D U^n and D_M terms collapse to the full operator at Ubar); four
-//           launches: centre rows (p, T) and the three momentum rows
+//           D U^n and D_M terms collapse to the full operator at Ubar).  Mixed
+//           mode: one launch, a thread per cell with its lower faces; FP64 mode:
+//           four, centre rows (p, T) and the three momentum rows, which also
+//           store the line rows the sweeps read
 //   sweep : r, theta, phi line solves (I + tau/2 D_d) x = rhs (eqs. spl1-spl3):
 //           3x3-block systems for (p, T, u_d), scalar ones for the two
-//           transverse velocities, cyclic along a periodic phi.  FP64 mode: one
-//           thread per line (block Thomas, Woodbury / Sherman-Morrison on cyclic
-//           lines).  Mixed mode: the partitioned solver of sph_lines.cuh (lanes
-//           of a warp per line, chunk elimination + parallel cyclic reduction),
-//           one launch for the block lines and one for both transverse kinds.
+//           transverse velocities, cyclic along a periodic phi.  FP64 mode: block
+//           Thomas from both ends, a lane per line and side or a column of it
+//           (sph_fp64_lines.cuh).  Mixed mode, one launch for the block lines and
+//           one for both transverse kinds: the partitioned solver of sph_lines.cuh
+//           (lanes of a warp per line, chunk elimination + parallel cyclic
+//           reduction) for its lengths; a lane per line and side
+//           (sph_lines2.cuh) for many r or theta lines, and for other lengths
+//           from 1024 lines; else, and in either mode by choice, one thread per
+//           line with Woodbury / Sherman-Morrison on cyclic lines.
 //           The phi sweep also applies U^{k+1} = U^k + x and accumulates the
-//           increment norm.
+//           increment norm (a step's last iteration).
 //
 // Precision: everything is templated on the bulk type R.  R = double is the
 // plain FP64 scheme.  R = float ("mixed") keeps U^n, U^{n+1,k} and their update
@@ -29,7 +35,8 @@
 // FP64 state as hi + lo pairs on the FP32 pipe, div(Ubar) -- which multiplies
 // gamma (p + pi_inf) and nearly cancels at low Mach number -- is carried as a
 // pair, the hydrostatic part of the r-momentum row goes through density
-// perturbations, and the cyclic corrections of the Thomas path combine in FP64.
+// perturbations, and the cyclic corrections of the Thomas and many-lines paths
+// combine in FP64.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

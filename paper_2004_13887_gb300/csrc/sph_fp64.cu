@@ -60,10 +60,10 @@ void f64_rows(sph_ctx* c, CF<double> ub, int dir) {
 // Block lines below which the FP64 sweeps split a line's 3x3 arithmetic over
 // lanes: a warp then holds 4 lines (2 cyclic ones) instead of 16, and its
 // serial chain is about 0.4 times as long, at 1.6 times the FP64 instructions in
-// all.  The split pays while the unsplit launch leaves SM quarters idle (4 per
-// SM): nl / 16 warps on 4 nsm quarters.  (4096 lines of 128 cells along theta,
+// all.  The split pays while the unsplit launch, nl / 16 warps on 4 nsm SM quarters,
+// leaves half of them idle: 32 lines an SM.  (4096 lines of 128 cells along theta,
 // 8192 along r of 32 cells, unsplit: 413 and 262 us; 4096 cyclic ones split 1102.)
-static int lines64_split(const sph_ctx* c, int nl) { return nl <= 16 * 4 * c->nsm / 2; }
+static int lines64_split(const sph_ctx* c, int nl) { return nl <= 32 * c->nsm; }
 
 template <int D, bool CYC, bool TR>
 static void launch_lines64(sph_ctx* c, const f64::LineArgs& S) {

@@ -206,11 +206,11 @@ static int lines_groups(const SweepArgs<float>& S, int kind, int NW) {
 }
 
 // whether the partitioned solver takes the lines along d: lines of 16, 32, 48,
-// 64, 128, 192 and 256 cells, and phi lines of 512 and 1024 (one thread per
-// line would read those uncoalesced).  Along r and theta, lines of 512 cells run faster on the
-// block Thomas path, whose threads read adjacent lines together (measured:
-// theta 4.3 vs 5.0 ms per step on 64 x 512 x 1024), and more accurately where
-// I + tau/2 D_r is stiff.
+// 64, 128, 192 and 256 cells, and phi lines of 512 and 1024 (a lane per
+// line would read those uncoalesced).  Along r and theta, lines of 512 cells run faster
+// with a lane a line, whose loads of adjacent lines go together (measured: theta 4.3 vs
+// 5.0 ms per step on 64 x 512 x 1024 with one thread a line, and again less with the
+// many-lines kernels), and more accurately where I + tau/2 D_r is stiff.
 static int lines_ok(const sph_ctx* c, int d) {
   const Geo<double>& g = c->d64.g;
   int n = d == 0 ? g.nr : d == 1 ? g.nt : g.np;

@@ -101,8 +101,8 @@ __global__ void k_cvt_in(long n, const double* __restrict__ a, R* __restrict__ o
 // The stencil kernels run on tiles of TK x TJ x TI points (phi fastest; 128
 // threads; the shape is set per context, sph_set_tile).  A block takes the
 // fast path when its whole tile has its +-2 neighbourhood in r and theta
-// inside the grid (a uniform choice).  The default is one phi row; the
-// ensemble's autotuner picks the shape per grid.
+// inside the grid (a uniform choice).  The default is one r row of 1, 2 or 4 theta
+// rows by the length of a phi row; the ensemble's autotuner picks the shape per grid.
 template <typename G>
 __device__ __forceinline__ bool tile_inner_at(const G& g, int i0, int j0, int ti, int tj) {
   return inner_ij(g, i0, j0) && inner_ij(g, i0 + ti - 1, j0 + tj - 1);
