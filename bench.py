@@ -67,9 +67,9 @@ HBM_PEAK_GBS, HBM_PEAK_SOURCE = hbm_peak()
 #   sweep_r/theta : rhs in (5 x 4 B) + Ubar in (5 x 4) + increment out (5 x 4)        =  60
 #   sweep_phi     : rhs in (5 x 4) + Ubar in (5 x 4) + U^k in and out (2 x 5 x 8)     = 120
 #   rhs           : U^n and U^k in (2 x 5 x 8) + R out (5 x 4)                         = 100
-#   coef          : Ubar in (5 x 4) + 17 coefficient planes out (17 x 4)               =  88
+#   coef          : Ubar in (5 x 4) + 14 coefficient planes out (14 x 4)               =  76
 #   avg           : U^n and U^k in (2 x 5 x 8) + Ubar out (5 x 4)                      = 100
-MIXED_BYTES_PER_POINT = {"sweep_r": 60, "sweep_theta": 60, "sweep_phi": 120, "rhs": 100, "coef": 88, "avg": 100}
+MIXED_BYTES_PER_POINT = {"sweep_r": 60, "sweep_theta": 60, "sweep_phi": 120, "rhs": 100, "coef": 76, "avg": 100}
 
 # DRAM traffic of each mixed stage measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum over the stage's launches, per grid point, the mean of
@@ -82,9 +82,9 @@ MIXED_BYTES_PER_POINT = {"sweep_r": 60, "sweep_theta": 60, "sweep_phi": 120, "rh
 # count; the sweeps only where their line layouts are the same (theta and phi
 # lines of 256 cells; the window's r lines are 64 cells, the workload's 128).
 TRAFFIC_GRID = (64, 256, 256)
-MEASURED_TRAFFIC = {"avg": 92.6, "coef": 75.4, "rhs": 199.0, "sweep_theta": 68.6, "sweep_phi": 130.6}
+MEASURED_TRAFFIC = {"avg": 92.4, "coef": 65.6, "rhs": 116.0, "sweep_theta": 139.2, "sweep_phi": 131.0}
 PER_POINT_STAGES = ("avg", "coef", "rhs", "sweep_theta", "sweep_phi")
-TRAFFIC_SOURCE_HASH = "8343889b4a6ba17a"
+TRAFFIC_SOURCE_HASH = "7aa3b5a7ded9b052"
 
 
 def kernel_source_hash():

@@ -5,7 +5,7 @@
 // Along r and theta the lanes of a warp hold 32 lines adjacent in phi (the last of a
 // phi row and the first of the next side by side), so every load and store of the
 // chain is coalesced as it stands: no lane exchanges and no reduction across lanes --
-// 363 instructions a cell along r against 845 in the partitioned solver's phi lines
+// 340 instructions a cell along r against 850 in the partitioned solver's phi lines
 // (sph_lines.cuh), which is the better one only where there are too few lines to
 // fill the SMs (it has 4 to 128 lanes a line).  Two warps of a block take the two
 // sides of the same lines; q = n/2 is the middle cell of a walled line:
